@@ -201,9 +201,7 @@ pin_status pin_sync(pin_plan_t p, int64_t timeout_ns);
 pin_status pin_get_stats(pin_plan_t p, pin_stats* out);
 
 /* Number of kernels one pin_collapse_times call launches (for accounting):
- * per radius the x, y and z passes, the root pass unless the z pass of this
- * grid size computes the collapse times itself (N = 384 and 768, the sizes
- * with three-level line transforms), and the FP64 redo. */
+ * per radius the x, y and z passes and the FP64 redo. */
 int pin_kernels_per_call(pin_plan_t p);
 
 /* Measurement hooks.  pin_profile(p, 1) makes later pin_collapse_times calls
@@ -211,10 +209,8 @@ int pin_kernels_per_call(pin_plan_t p);
  * inside its graph); pin_pass_times() then waits for the plan's work and
  * returns, for the last completed call, the device time in milliseconds summed
  * over radii of: ms4[0] the x pass (filter + transform), ms4[1] the y pass,
- * ms4[2] the z pass (c2r + eigenvalues; at N = 384 and 768 also the collapse
- * time and running max), ms4[3] the root pass (collapse time + running max, where it
- * is a kernel of its own) with the FP64 redo of the queued ill-conditioned
- * particles.  Each is measured on the stream its pass runs on; under an
+ * ms4[2] the z pass (c2r, eigenvalues, collapse time and running max), ms4[3]
+ * the FP64 redo of the queued ill-conditioned particles.  Each is measured on the stream its pass runs on; under an
  * overlapped schedule (pin_set_schedule) the passes overlap, so the four sums
  * exceed the call's time. */
 pin_status pin_profile(pin_plan_t p, int enable);
@@ -282,8 +278,8 @@ pin_status pin_set_radii(pin_plan_t p, int nscales, const double* radii);
  * with velocities: pin_footprint_bytes does not count them), and the y pass of
  * s + 2 waits for the z pass of s.  Results are bit-identical in every
  * schedule; only the time changes (the z pass is bound by instruction issue,
- * the x/y passes by memory).  Needs a grid whose z pass computes the collapse
- * times itself (nz = 384 or 768), else PIN_EINVAL.  Waits for the plan's
+ * the x/y passes by memory).  Needs a grid with three-level z lines (nz = 384
+ * or 768), else PIN_EINVAL.  Waits for the plan's
  * stream; the next call re-captures its graph.  PIN_ENOMEM (plan unchanged)
  * when the second set of spectra does not fit. */
 pin_status pin_set_schedule(pin_plan_t p, int schedule);

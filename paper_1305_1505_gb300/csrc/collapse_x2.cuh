@@ -37,27 +37,71 @@ __device__ __forceinline__ float2 abs(float2 a) { return make_float2(fabsf(a.x),
 
 }  // namespace x2
 
+// Determinant of the deviator and squared norm (6 p^2) of two symmetric
+// matrices with diagonals b0, b1, b2 (trace removed), as the ratio
+// r = det / (2 p^3) needs them.  Two roundings of the same formulas are kept,
+// so that results do not move in the last bits: FUSED false, products and
+// differences rounded separately (the three-level line sizes); FUSED true, each
+// difference of products contracted into one fma, as the scalar eig3<float>
+// compiles (the two-level sizes).  The contracted form works with the negated
+// determinant, because the packed fma has no operand negation.
+template <bool FUSED>
+__device__ __forceinline__ void deviator_x2(const float2 h[6], float2 q, float2& p2, float2& p, float2& ratio,
+                                            bool& iso0, bool& iso1) {
+  using namespace x2;
+  const float2 b0 = sub(h[0], q), b1 = sub(h[1], q), b2 = sub(h[2], q);
+  float2 num, two;
+  if constexpr (FUSED) {
+    const float2 nb1 = sub(q, h[1]), nh3 = mul(h[3], splat(-1.0f)), h55 = mul(h[5], h[5]);
+    const float2 off = add(fma(h[3], h[3], mul(h[4], h[4])), h55);
+    p2 = fma(splat(2.0f), off, fma(b2, b2, fma(b0, b0, mul(b1, b1))));
+    const float2 nt1 = fma(nb1, b2, h55);
+    const float2 nt2 = fma(nh3, b2, mul(h[5], h[4]));
+    const float2 nt3 = fma(nh3, h[5], mul(b1, h[4]));
+    num = fma(h[4], nt3, fma(b0, nt1, mul(nh3, nt2)));  // -det
+    two = splat(-2.0f);
+  } else {
+    const float2 off = fma(h[5], h[5], fma(h[4], h[4], mul(h[3], h[3])));
+    p2 = fma(splat(2.0f), off, fma(b2, b2, fma(b1, b1, mul(b0, b0))));
+    const float2 t1 = sub(mul(b1, b2), mul(h[5], h[5]));
+    const float2 t2 = sub(mul(h[3], b2), mul(h[5], h[4]));
+    const float2 t3 = sub(mul(h[3], h[5]), mul(b1, h[4]));
+    num = sub(fma(h[4], t3, mul(b0, t1)), mul(h[3], t2));
+    two = splat(2.0f);
+  }
+  iso0 = !(p2.x > 0.0f);
+  iso1 = !(p2.y > 0.0f);
+  const float2 p6 = mul(p2, splat(1.0f / 6.0f));
+  p = make_float2(M<float>::sqrt_(iso0 ? 0.0f : p6.x), M<float>::sqrt_(iso1 ? 0.0f : p6.y));
+  ratio = div(num, mul(mul(two, p), mul(p, p)));
+}
+
+// Clamp to [-1, 1] that keeps a NaN.
+__device__ __forceinline__ float clamp1_nan(float x) {
+  float r;
+  asm("max.NaN.f32 %0, %1, 0fBF800000;" : "=f"(r) : "f"(x));
+  asm("min.NaN.f32 %0, %1, 0f3F800000;" : "=f"(r) : "f"(r));
+  return r;
+}
+
 // eig3<float> of two symmetric matrices h[c] = (particle 0, particle 1),
 // c = xx, yy, zz, xy, xz, yz; lam sorted per lane, largest first.  Returns the
-// per-lane |r| (near 1: a near-degenerate pair, see eig3).
+// per-lane |r| (near 1: a near-degenerate pair, see eig3).  FUSED: see
+// deviator_x2; that form also hands a NaN ratio on, as the scalar one does.
+template <bool FUSED = false>
 __device__ __forceinline__ float2 eig3_x2(const float2 h[6], float2 lam[3]) {
   using namespace x2;
   const float2 q = mul(add(add(h[0], h[1]), h[2]), splat(1.0f / 3.0f));
-  const float2 b0 = sub(h[0], q), b1 = sub(h[1], q), b2 = sub(h[2], q);
-  const float2 off = fma(h[5], h[5], fma(h[4], h[4], mul(h[3], h[3])));
-  const float2 p2 = fma(splat(2.0f), off, fma(b2, b2, fma(b1, b1, mul(b0, b0))));
-  const bool iso0 = !(p2.x > 0.0f), iso1 = !(p2.y > 0.0f);
-  const float2 p6 = mul(p2, splat(1.0f / 6.0f));
-  const float2 p = make_float2(M<float>::sqrt_(iso0 ? 0.0f : p6.x), M<float>::sqrt_(iso1 ? 0.0f : p6.y));
-  // det(A - qI)
-  const float2 t1 = sub(mul(b1, b2), mul(h[5], h[5]));
-  const float2 t2 = sub(mul(h[3], b2), mul(h[5], h[4]));
-  const float2 t3 = sub(mul(h[3], h[5]), mul(b1, h[4]));
-  const float2 det = sub(fma(h[4], t3, mul(b0, t1)), mul(h[3], t2));
-  const float2 den = mul(mul(splat(2.0f), p), mul(p, p));
-  float2 r = div(det, den);
-  r.x = iso0 ? 1.0f : fminf(fmaxf(r.x, -1.0f), 1.0f);
-  r.y = iso1 ? 1.0f : fminf(fmaxf(r.y, -1.0f), 1.0f);
+  float2 p2, p, r;
+  bool iso0, iso1;
+  deviator_x2<FUSED>(h, q, p2, p, r, iso0, iso1);
+  if constexpr (FUSED) {
+    r.x = iso0 ? 1.0f : clamp1_nan(r.x);
+    r.y = iso1 ? 1.0f : clamp1_nan(r.y);
+  } else {
+    r.x = iso0 ? 1.0f : fminf(fmaxf(r.x, -1.0f), 1.0f);
+    r.y = iso1 ? 1.0f : fminf(fmaxf(r.y, -1.0f), 1.0f);
+  }
   // acos (Abramowitz & Stegun 4.4.46, as M<float>::acos_), lanes in parallel
   const float2 ax = abs(r);
   float2 poly = splat(-0.0012624911f);
@@ -78,10 +122,17 @@ __device__ __forceinline__ float2 eig3_x2(const float2 h[6], float2 lam[3]) {
   M<float>::sincos_(phi.y, &sn.y, &cs.y);
   // cos(phi + 2 pi/3) = -cos(phi)/2 - (sqrt(3)/2) sin(phi)
   const float2 l0 = fma(mul(splat(2.0f), p), cs, q);
-  const float2 l2 = sub(q, mul(p, fma(splat(1.7320508075688772935f), sn, cs)));
+  const float2 w = fma(splat(1.7320508075688772935f), sn, cs);
   lam[0] = l0;
-  lam[2] = l2;
-  lam[1] = sub(sub(mul(splat(3.0f), q), l0), l2);
+  if constexpr (FUSED) {
+    const float2 l2 = fma(mul(p, splat(-1.0f)), w, q);
+    lam[2] = l2;
+    lam[1] = mul(add(fma(splat(-3.0f), q, l0), l2), splat(-1.0f));
+  } else {
+    const float2 l2 = sub(q, mul(p, w));
+    lam[2] = l2;
+    lam[1] = sub(sub(mul(splat(3.0f), q), l0), l2);
+  }
   return abs(r);
 }
 

@@ -32,25 +32,27 @@ template <int N> __host__ __device__ constexpr int field_stride() {
   return Shape<N>::P2 > 1 ? N + 2 : N + (Shape<N>::P >= 2 ? Shape<N>::P / 2 : 1);
 }
 
-// Compaction of the root solve in the fused z pass (1: queue the particles
-// that cannot be skipped and solve them after the main loop).
-#ifndef PIN_Z_COMPACT
-#define PIN_Z_COMPACT 1
-#endif
-
 // ---------------------------------------------------------------- z pass --
 // Lines along z: line index l = x*N + y, the half line src[f][l*nhp + kz],
 // kz in [0, N/2], is contiguous.  Fields are paired (A + iB) into one complex
 // length-N transform whose real and imaginary parts are the two real lines.
 // NP pairs per line: 3 (the six Hessian components) or 5 (plus the three
 // smoothed displacement components, kept for the velocity at R_max).
-// FUSE: the collapse time and the running maximum of every particle follow
-// its eigenvalues in this kernel (no eigenvalue round trip through memory);
-// otherwise the eigenvalues go to lam_out for k_roots.  SRC: instead, the
-// second-order LPT source S = sum_{i<j} (phi_ii phi_jj - phi_ij^2) of every
-// particle goes to out[0] (a real field).
-template <int N, int LINES, bool DUMP, int NP, bool FUSE, bool SRC = false>
-__global__ void __launch_bounds__(NP * LINES * Shape<N>::P, NP == 5 ? MinBlocks<N>::zv : MinBlocks<N>::z)
+// MODE: the collapse time and the running maximum of every particle follow
+// its eigenvalues in this kernel (kZCollapse); or the real fields go to out[]
+// (kZDump); or the second-order LPT source S = sum_{i<j} (phi_ii phi_jj -
+// phi_ij^2) of every particle goes to out[0], a real field (kZSource).
+// The eigenvalues never go through memory: writing them for a root kernel of
+// their own took 17.1 ps per particle and radius at 256^3 and 16.4 at 128^3
+// (z and roots together), this kernel 12.0 and 11.3; it is bound by
+// instruction issue.  The two-level sizes use the fma-contracted eigenvalue
+// form, which keeps their results to the last bit.
+enum ZMode { kZCollapse, kZDump, kZSource };
+
+template <int N, int LINES, int NP, ZMode MODE>
+__global__ void __launch_bounds__(NP * LINES * Shape<N>::P, MODE != kZCollapse ? MinBlocks<N>::zt
+                                                            : NP == 5          ? MinBlocks<N>::zv
+                                                                               : MinBlocks<N>::z)
     k_pass_z(ArgsZ a) {
   constexpr int E = Shape<N>::E, P = Shape<N>::P;
   constexpr int NC = NP * LINES;  // pair-columns of the block
@@ -128,7 +130,7 @@ __global__ void __launch_bounds__(NP * LINES * Shape<N>::P, NP == 5 ? MinBlocks<
     fft_line<N, L, 32 % Shape<N>::P == 0>(v, p, c, s_x, s_tw);
   }
 
-  if constexpr (DUMP) {
+  if constexpr (MODE == kZDump) {
     if (active) {
       float* oa = a.out[fa] + (size_t)line * N;
       float* ob = hasb ? a.out[fb] + (size_t)line * N : nullptr;
@@ -154,7 +156,7 @@ __global__ void __launch_bounds__(NP * LINES * Shape<N>::P, NP == 5 ? MinBlocks<
     }
     __syncthreads();
     const size_t total = (size_t)nlines * N;
-    if constexpr (SRC) {
+    if constexpr (MODE == kZSource) {
       for (int pt = tid; pt < kPts; pt += nthreads) {
         const int l = pt / N, z = pt % N;
         const int gl = blockIdx.x * LINES + l;
@@ -165,17 +167,13 @@ __global__ void __launch_bounds__(NP * LINES * Shape<N>::P, NP == 5 ? MinBlocks<
         a.out[0][(size_t)gl * N + z] =
             h[0] * h[1] + h[0] * h[2] + h[1] * h[2] - h[3] * h[3] - h[4] * h[4] - h[5] * h[5];
       }
-    } else if constexpr (FUSE && PIN_Z_ILP % 2 == 0) {
-      // eigenvalues, collapse time and running maximum of PIN_Z_ILP particles
-      // per thread and iteration, held two by two in the lanes of packed
-      // pairs (NPR independent pairs, so that their dependency chains
-      // interleave)
-      constexpr int NPR = PIN_Z_ILP / 2;
+    } else {
+      // eigenvalues, collapse time and running maximum of two particles per
+      // thread and iteration, held in the lanes of packed pairs
       const CollapseConsts<float> ccf{a.dcorr_f, a.correction};
       // Compaction: particles that cannot be skipped are queued and solved
       // after the main loop, two per thread, so that a warp's root solve runs
       // on full lanes
-      constexpr bool kCompact = PIN_Z_COMPACT != 0;
       unsigned short* s_q = reinterpret_cast<unsigned short*>(s_f + LINES * NF * kFS);
       // The end of a pair's computation: the rare minor-axis solve, the FP64
       // redo of an ill-conditioned root, and the running maximum.
@@ -217,264 +215,117 @@ __global__ void __launch_bounds__(NP * LINES * Shape<N>::P, NP == 5 ? MinBlocks<
           }
         }
       };
-      for (int pt0 = tid; pt0 < kPts; pt0 += 2 * NPR * nthreads) {
-        int q[NPR][2], lz[NPR][2];
-        bool valid[NPR][2];
-        float fm[NPR][2];
-        float2 lam[NPR][3];
+      for (int pt0 = tid; pt0 < kPts; pt0 += 2 * nthreads) {
+        int q[2], lz[2];
+        bool valid[2];
+        float fm[2];
+        float2 h[6], lam[3];
 #pragma unroll
-        for (int r = 0; r < NPR; ++r) {
-          float2 h[6];
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const int pt = pt0 + (2 * r + u) * nthreads;
-            const int l = pt / N, z = pt % N;
-            const int gl = blockIdx.x * LINES + l;
-            valid[r][u] = pt < kPts && gl < nlines;
-            q[r][u] = gl * N + z;  // < 2^31: checked at plan creation
-            lz[r][u] = (l * NF) * kFS + z;
-#pragma unroll
-            for (int f = 0; f < 6; ++f) {
-              const float v = valid[r][u] ? s_f[lz[r][u] + f * kFS] : 0.f;
-              if (u) h[f].y = v;
-              else h[f].x = v;
-            }
-          }
-          const float2 rabs = eig3_x2(h, lam[r]);
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            fm[r][u] = valid[r][u] ? a.fmax[q[r][u]] : 0.f;
-            if (valid[r][u] && (u ? rabs.y : rabs.x) > 1.f - a.tau_eig) {
-              // a near-degenerate pair: the FP32 eigenvalues are not trusted,
-              // but the invariant bound (no eigenvalues) may already show that
-              // the particle cannot beat F_max, by more than the FP32 error of
-              // the bound; then neither the redo nor anything else is needed
-              float hl[6];
-#pragma unroll
-              for (int f = 0; f < 6; ++f) hl[f] = u ? h[f].y : h[f].x;
-              if (fm[r][u] * (1.f - 1e-5f) > collapse_bound<float>(hl, ccf) * (1.f + 1e-5f)) {
-                valid[r][u] = false;
-                continue;
-              }
-              atomicAdd(a.counters + 0, 1ull);
-              const unsigned slot = atomicAdd(a.redo_count, 1u);
-              if (slot < a.redo_cap) {
-                RedoEntry e;
-                e.q = q[r][u];
-#pragma unroll
-                for (int f = 0; f < 6; ++f) e.h[f] = u ? h[f].y : h[f].x;
-                e.kind = 0;
-                a.redo_list[slot] = e;
-                if constexpr (NP == 5) {
-#pragma unroll
-                  for (int cpt = 0; cpt < 3; ++cpt)
-                    a.psi_out[cpt * total + q[r][u]] = s_f[lz[r][u] + (6 + cpt) * kFS];
-                }
-                valid[r][u] = false;  // the redo kernel updates this particle
-#pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                  if (u) lam[r][k].y = 0.f;
-                  else lam[r][k].x = 0.f;
-                }
-              } else {
-                atomicAdd(a.counters + 2, 1ull);  // queue full: keep the FP32 eigenvalues
-              }
-            }
-          }
-        }
-        // lanes that cannot beat their running maximum (the radii run
-        // smallest first, so most particles reach F_max early) or that the
-        // FP64 redo finishes skip the root solve
-        CollapseStateX2 csx[NPR];
-        unsigned done[NPR];
-#pragma unroll
-        for (int r = 0; r < NPR; ++r) {
-          float2 c0[3];
-          collapse_prep_x2(lam[r], ccf, csx[r], c0);
-          done[r] = cannot_beat_x2(c0, csx[r], make_float2(fm[r][0], fm[r][1])) | (valid[r][0] ? 0u : 1u) |
-                    (valid[r][1] ? 0u : 2u);
-          if constexpr (kCompact) {
-            // the rest wait in a queue: eigenvalues and F_max in the
-            // particle's own (already read) field slots 0-3
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-              if ((done[r] >> u) & 1u) continue;
-#pragma unroll
-              for (int k = 0; k < 3; ++k) s_f[lz[r][u] + k * kFS] = u ? lam[r][k].y : lam[r][k].x;
-              s_f[lz[r][u] + 3 * kFS] = fm[r][u];
-              s_q[atomicAdd(&s_nq, 1)] = (unsigned short)(pt0 + (2 * r + u) * nthreads);
-            }
-          } else {
-            // a pair solves if one of its lanes needs it
-            if (done[r] != 3u) collapse_root_x2(c0, csx[r]);
-          }
-        }
-        if constexpr (!kCompact) {
-#pragma unroll
-          for (int r = 0; r < NPR; ++r) finish(csx[r], done[r], lam[r], q[r], lz[r], fm[r]);
-        }
-      }
-      if constexpr (kCompact) {
-        // the queued particles, two per thread: the lanes of a warp all need
-        // the root (in the main loop a warp solved whenever one of its 64
-        // particles did: about 40 % of warps for 7 % of pairs at 768^3; z
-        // pass 5.52 -> 5.21 ms per radius)
-        __syncthreads();
-        const int nq = s_nq;
-        for (int k0 = 2 * tid; k0 < nq; k0 += 2 * nthreads) {
-          int q2[2], lz2[2];
-          float fm2[2];
-          float2 lam2[3];
-          unsigned dn = 0;
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const bool ok = k0 + u < nq;
-            const int pt = s_q[ok ? k0 + u : k0];
-            const int l = pt / N, z = pt % N;
-            q2[u] = (blockIdx.x * LINES + l) * N + z;
-            lz2[u] = (l * NF) * kFS + z;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-              const float x = s_f[lz2[u] + k * kFS];
-              if (u) lam2[k].y = x;
-              else lam2[k].x = x;
-            }
-            fm2[u] = s_f[lz2[u] + 3 * kFS];
-            dn |= ok ? 0u : (1u << u);
-          }
-          CollapseStateX2 cs2;
-          float2 c0[3];
-          collapse_prep_x2(lam2, ccf, cs2, c0);
-          collapse_root_x2(c0, cs2);
-          finish(cs2, dn, lam2, q2, lz2, fm2);
-        }
-      }
-    } else if constexpr (FUSE) {
-      // eigenvalues, collapse time and running maximum, PIN_Z_ILP particles
-      // per thread and iteration
-      constexpr int U = PIN_Z_ILP;
-      const CollapseConsts<float> ccf{a.dcorr_f, a.correction};
-      for (int pt0 = tid; pt0 < kPts; pt0 += U * nthreads) {
-        float lam[U][3], fm[U];
-        bool valid[U];
-        int q[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
+        for (int u = 0; u < 2; ++u) {
           const int pt = pt0 + u * nthreads;
           const int l = pt / N, z = pt % N;
           const int gl = blockIdx.x * LINES + l;
           valid[u] = pt < kPts && gl < nlines;
           q[u] = gl * N + z;  // < 2^31: checked at plan creation
-          fm[u] = 0.f;
-          lam[u][0] = lam[u][1] = lam[u][2] = 0.f;
-          if (valid[u]) {
-            float h[6];
+          lz[u] = (l * NF) * kFS + z;
 #pragma unroll
-            for (int f = 0; f < 6; ++f) h[f] = s_f[(l * NF + f) * kFS + z];
-            const float rabs = eig3<float>(h, lam[u]);
-            fm[u] = a.fmax[q[u]];
-            if (rabs > 1.f - a.tau_eig) {
-              atomicAdd(a.counters + 0, 1ull);
-              const unsigned slot = atomicAdd(a.redo_count, 1u);
-              if (slot < a.redo_cap) {
-                RedoEntry e;
-                e.q = q[u];
-#pragma unroll
-                for (int f = 0; f < 6; ++f) e.h[f] = h[f];
-                e.kind = 0;
-                a.redo_list[slot] = e;
-                if constexpr (NP == 5) {
-#pragma unroll
-                  for (int cpt = 0; cpt < 3; ++cpt)
-                    a.psi_out[cpt * total + q[u]] = s_f[(l * NF + 6 + cpt) * kFS + z];
-                }
-                valid[u] = false;  // the redo kernel updates this particle
-                lam[u][0] = lam[u][1] = lam[u][2] = 0.f;
-              } else {
-                atomicAdd(a.counters + 2, 1ull);  // queue full: keep the FP32 eigenvalues
-              }
-            }
+          for (int f = 0; f < 6; ++f) {
+            const float v = valid[u] ? s_f[lz[u] + f * kFS] : 0.f;
+            if (u) h[f].y = v;
+            else h[f].x = v;
           }
         }
-        CollapseState<float> cs[U];
+        const float2 rabs = eig3_x2<(Shape<N>::P2 == 1)>(h, lam);
 #pragma unroll
-        for (int u = 0; u < U; ++u) collapse_main<float>(lam[u], ccf, cs[u]);
+        for (int u = 0; u < 2; ++u) {
+          fm[u] = valid[u] ? a.fmax[q[u]] : 0.f;
+          if (valid[u] && (u ? rabs.y : rabs.x) > 1.f - a.tau_eig) {
+            // a near-degenerate pair: the FP32 eigenvalues are not trusted,
+            // but the invariant bound (no eigenvalues) may already show that
+            // the particle cannot beat F_max, by more than the FP32 error of
+            // the bound; then neither the redo nor anything else is needed
+            float hl[6];
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-          if (cs[u].need[0] || cs[u].need[1]) collapse_rare<float>(cs[u]);
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          if (!valid[u]) continue;
-          const int pt = pt0 + u * nthreads;
-          const int l = pt / N, z = pt % N;
-          const float F = cs[u].best + cs[u].corr;
-          if (cs[u].kappa < a.tau_root) {
-            atomicAdd(a.counters + 1, 1ull);
+            for (int f = 0; f < 6; ++f) hl[f] = u ? h[f].y : h[f].x;
+            if (fm[u] * (1.f - 1e-5f) > collapse_bound<float>(hl, ccf) * (1.f + 1e-5f)) {
+              valid[u] = false;
+              continue;
+            }
+            atomicAdd(a.counters + 0, 1ull);
             const unsigned slot = atomicAdd(a.redo_count, 1u);
             if (slot < a.redo_cap) {
               RedoEntry e;
               e.q = q[u];
-              e.h[0] = lam[u][0];
-              e.h[1] = lam[u][1];
-              e.h[2] = lam[u][2];
-              e.h[3] = e.h[4] = e.h[5] = 0.f;
-              e.kind = 1;
+#pragma unroll
+              for (int f = 0; f < 6; ++f) e.h[f] = u ? h[f].y : h[f].x;
+              e.kind = 0;
               a.redo_list[slot] = e;
               if constexpr (NP == 5) {
 #pragma unroll
-                for (int cpt = 0; cpt < 3; ++cpt)
-                  a.psi_out[cpt * total + q[u]] = s_f[(l * NF + 6 + cpt) * kFS + z];
+                for (int cpt = 0; cpt < 3; ++cpt) a.psi_out[cpt * total + q[u]] = s_f[lz[u] + (6 + cpt) * kFS];
               }
-              continue;
-            }
-            atomicAdd(a.counters + 2, 1ull);  // queue full: keep the FP32 value
-          }
-          if (F > fm[u] || (F == fm[u] && F > 0.f && a.scale < a.idx[q[u]])) {
-            a.fmax[q[u]] = F;
-            a.idx[q[u]] = a.scale;
-            if constexpr (NP == 5) {
+              valid[u] = false;  // the redo kernel updates this particle
 #pragma unroll
-              for (int cpt = 0; cpt < 3; ++cpt) a.vstate[cpt * total + q[u]] = s_f[(l * NF + 6 + cpt) * kFS + z];
+              for (int k = 0; k < 3; ++k) {
+                if (u) lam[k].y = 0.f;
+                else lam[k].x = 0.f;
+              }
+            } else {
+              atomicAdd(a.counters + 2, 1ull);  // queue full: keep the FP32 eigenvalues
             }
           }
+        }
+        // lanes that cannot beat their running maximum (the radii run
+        // smallest first, so most particles reach F_max early) or that the
+        // FP64 redo finishes skip the root solve; the rest wait in a queue:
+        // eigenvalues and F_max in the particle's own (already read) field
+        // slots 0-3
+        CollapseStateX2 csx;
+        float2 c0[3];
+        collapse_prep_x2(lam, ccf, csx, c0);
+        const unsigned done =
+            cannot_beat_x2(c0, csx, make_float2(fm[0], fm[1])) | (valid[0] ? 0u : 1u) | (valid[1] ? 0u : 2u);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          if ((done >> u) & 1u) continue;
+#pragma unroll
+          for (int k = 0; k < 3; ++k) s_f[lz[u] + k * kFS] = u ? lam[k].y : lam[k].x;
+          s_f[lz[u] + 3 * kFS] = fm[u];
+          s_q[atomicAdd(&s_nq, 1)] = (unsigned short)(pt0 + u * nthreads);
         }
       }
-    } else {
-      // eigenvalues of every particle of the block's lines; the collapse time
-      // and the running maximum follow in k_roots
-      for (int pt = tid; pt < kPts; pt += nthreads) {
-        const int l = pt / N, z = pt % N;
-        const int gl = blockIdx.x * LINES + l;
-        if (gl >= nlines) continue;
-        float h[6], lam[3];
+      // the queued particles, two per thread: the lanes of a warp all need
+      // the root (in the main loop a warp would solve whenever one of its 64
+      // particles did: about 40 % of warps for 7 % of pairs at 768^3; z pass
+      // 5.52 -> 5.21 ms per radius)
+      __syncthreads();
+      const int nq = s_nq;
+      for (int k0 = 2 * tid; k0 < nq; k0 += 2 * nthreads) {
+        int q2[2], lz2[2];
+        float fm2[2];
+        float2 lam2[3];
+        unsigned dn = 0;
 #pragma unroll
-        for (int f = 0; f < 6; ++f) h[f] = s_f[(l * NF + f) * kFS + z];
-        const float rabs = eig3<float>(h, lam);
-        const int q = gl * N + z;  // < 2^31: checked at plan creation
-        if (rabs > 1.f - a.tau_eig) {
-          atomicAdd(a.counters + 0, 1ull);
-          const unsigned slot = atomicAdd(a.redo_count, 1u);
-          if (slot < a.redo_cap) {
-            RedoEntry e;
-            e.q = q;
+        for (int u = 0; u < 2; ++u) {
+          const bool ok = k0 + u < nq;
+          const int pt = s_q[ok ? k0 + u : k0];
+          const int l = pt / N, z = pt % N;
+          q2[u] = (blockIdx.x * LINES + l) * N + z;
+          lz2[u] = (l * NF) * kFS + z;
 #pragma unroll
-            for (int f = 0; f < 6; ++f) e.h[f] = h[f];
-            e.kind = 0;
-            a.redo_list[slot] = e;
-            lam[0] = lam[1] = lam[2] = __int_as_float(0x7fc00000);  // NaN: skipped by k_roots
-          } else {
-            atomicAdd(a.counters + 2, 1ull);  // queue full: keep the FP32 eigenvalues
+          for (int k = 0; k < 3; ++k) {
+            const float x = s_f[lz2[u] + k * kFS];
+            if (u) lam2[k].y = x;
+            else lam2[k].x = x;
           }
+          fm2[u] = s_f[lz2[u] + 3 * kFS];
+          dn |= ok ? 0u : (1u << u);
         }
-        a.lam_out[q] = lam[0];
-        a.lam_out[total + q] = lam[1];
-        a.lam_out[2 * total + q] = lam[2];
-        if constexpr (NP == 5) {
-          // smoothed displacement of this radius, copied to the state by k_roots
-          // when F_max moves here
-#pragma unroll
-          for (int cpt = 0; cpt < 3; ++cpt) a.psi_out[cpt * total + q] = s_f[(l * NF + 6 + cpt) * kFS + z];
-        }
+        CollapseStateX2 cs2;
+        float2 c0[3];
+        collapse_prep_x2(lam2, ccf, cs2, c0);
+        collapse_root_x2(c0, cs2);
+        finish(cs2, dn, lam2, q2, lz2, fm2);
       }
     }
   }
@@ -558,146 +409,6 @@ __global__ void k_phi2(const float2* __restrict__ T, float2* out, int nx, int ny
   }
 }
 
-// ------------------------------------------------------------- root pass --
-// Per particle: the collapse time F from its eigenvalues (collapse.cuh), and
-// the running maximum F_max with its radius index, updated in place.  Few
-// registers, so many warps hide the latency of the dependent root iteration;
-// PIN_Z_ILP particles per thread and iteration.
-template <bool VEL>
-__global__ void __launch_bounds__(256) k_roots(ArgsZ a) {
-  constexpr int U = PIN_Z_ILP;
-  const int total = a.npart;
-  const float* L0 = a.lam_out;
-  const float* L1 = a.lam_out + total;
-  const float* L2 = a.lam_out + 2 * (size_t)total;
-  CollapseConsts<float> ccf{a.dcorr_f, a.correction};
-  const int stride = gridDim.x * blockDim.x;
-  if constexpr (U == 2) {
-    // two particles per thread in the lanes of packed pairs
-    for (int q0 = blockIdx.x * blockDim.x + threadIdx.x; q0 < total; q0 += 2 * stride) {
-      float2 lam[3];
-      float fm[2];
-      bool valid[2];
-      int q[2];
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        q[u] = q0 + u * stride;
-        const bool in = q[u] < total;
-        float l0 = in ? __ldg(L0 + q[u]) : 0.f, l1 = in ? __ldg(L1 + q[u]) : 0.f, l2 = in ? __ldg(L2 + q[u]) : 0.f;
-        fm[u] = in ? a.fmax[q[u]] : 0.f;
-        valid[u] = in && !isnan(l0);  // NaN: queued by the z pass
-        if (!valid[u]) l0 = l1 = l2 = 0.f;
-        if (u) {
-          lam[0].y = l0; lam[1].y = l1; lam[2].y = l2;
-        } else {
-          lam[0].x = l0; lam[1].x = l1; lam[2].x = l2;
-        }
-      }
-      CollapseStateX2 csx;
-      float2 c0[3];
-      collapse_prep_x2(lam, ccf, csx, c0);
-      const unsigned done = cannot_beat_x2(c0, csx, make_float2(fm[0], fm[1])) | (valid[0] ? 0u : 1u) |
-                            (valid[1] ? 0u : 2u);
-      if (done != 3u) collapse_root_x2(c0, csx);
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        if ((done >> u) & 1u) continue;
-        CollapseState<float> cs = lane_state(csx, u);
-        if (cs.need[0] || cs.need[1]) collapse_rare<float>(cs);
-        const float F = cs.best + cs.corr;
-        if (cs.kappa < a.tau_root) {
-          atomicAdd(a.counters + 1, 1ull);
-          const unsigned slot = atomicAdd(a.redo_count, 1u);
-          if (slot < a.redo_cap) {
-            RedoEntry e;
-            e.q = q[u];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) e.h[k] = u ? lam[k].y : lam[k].x;
-            e.h[3] = e.h[4] = e.h[5] = 0.f;
-            e.kind = 1;
-            a.redo_list[slot] = e;
-            continue;  // the redo kernel updates this particle
-          }
-          atomicAdd(a.counters + 2, 1ull);  // queue full: keep the FP32 value
-        }
-        if (F > fm[u] || (F == fm[u] && F > 0.f && a.scale < a.idx[q[u]])) {
-          a.fmax[q[u]] = F;
-          a.idx[q[u]] = a.scale;
-          if constexpr (VEL) {
-#pragma unroll
-            for (int cpt = 0; cpt < 3; ++cpt)
-              a.vstate[(size_t)cpt * total + q[u]] = a.psi_out[(size_t)cpt * total + q[u]];
-          }
-        }
-      }
-    }
-  } else {
-  for (int q0 = blockIdx.x * blockDim.x + threadIdx.x; q0 < total; q0 += U * stride) {
-    float lam[U][3], fm[U];
-    bool valid[U];
-    int q[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      q[u] = q0 + u * stride;
-      const bool in = q[u] < total;
-      lam[u][0] = in ? __ldg(L0 + q[u]) : 0.f;
-      lam[u][1] = in ? __ldg(L1 + q[u]) : 0.f;
-      lam[u][2] = in ? __ldg(L2 + q[u]) : 0.f;
-      fm[u] = in ? a.fmax[q[u]] : 0.f;
-      valid[u] = in && !isnan(lam[u][0]);  // NaN: queued by the z pass
-      if (!valid[u]) lam[u][0] = lam[u][1] = lam[u][2] = 0.f;
-    }
-    CollapseState<float> cs[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) collapse_main<float>(lam[u], ccf, cs[u]);
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-      if (cs[u].need[0] || cs[u].need[1]) collapse_rare<float>(cs[u]);
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (!valid[u]) continue;
-      const float F = cs[u].best + cs[u].corr;
-      if (cs[u].kappa < a.tau_root) {
-        atomicAdd(a.counters + 1, 1ull);
-        const unsigned slot = atomicAdd(a.redo_count, 1u);
-        if (slot < a.redo_cap) {
-          RedoEntry e;
-          e.q = q[u];
-          e.h[0] = lam[u][0];
-          e.h[1] = lam[u][1];
-          e.h[2] = lam[u][2];
-          e.h[3] = e.h[4] = e.h[5] = 0.f;
-          e.kind = 1;
-          a.redo_list[slot] = e;
-          continue;  // the redo kernel updates this particle
-        }
-        atomicAdd(a.counters + 2, 1ull);  // queue full: keep the FP32 value
-      }
-      if (F > fm[u] || (F == fm[u] && F > 0.f && a.scale < a.idx[q[u]])) {
-        a.fmax[q[u]] = F;
-        a.idx[q[u]] = a.scale;
-        if constexpr (VEL) {
-#pragma unroll
-          for (int cpt = 0; cpt < 3; ++cpt)
-            a.vstate[(size_t)cpt * total + q[u]] = a.psi_out[(size_t)cpt * total + q[u]];
-        }
-      }
-    }
-  }
-  }
-}
-
-cudaError_t launch_roots(const ArgsZ& a, cudaStream_t st) {
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const long need = ((long)a.npart + 255) / 256;
-  const unsigned grid = (unsigned)std::max<long>(1, std::min<long>(need, (long)sms * 8));
-  if (a.vstate) k_roots<true><<<grid, 256, 0, st>>>(a);
-  else k_roots<false><<<grid, 256, 0, st>>>(a);
-  return cudaGetLastError();
-}
-
 // FP64 redo of the queued particles of one radius (grid-stride; each particle
 // appears once per radius, so the in-place update has no race).
 __global__ void __launch_bounds__(128) k_redo64(ArgsZ a) {
@@ -749,19 +460,13 @@ template <int N> struct Cfg {
 #define PIN_TC_LONG 16
 #endif
   static constexpr int TC = P >= 16 ? PIN_TC_LONG : (P >= 8 ? 16 : (P == 4 ? 32 : 64));
-  // z-pass lines per block: 64 threads' worth of line per pair (at the
-  // three-level sizes one 32-thread line: 768 -> 1, 384 -> 2)
+  // threads' worth of z lines per block and pair (MinBlocks: why): one
+  // 32-thread line at 768, two 16-thread lines at 384 and 512, ...
 #ifndef PIN_Z_LW3
 #define PIN_Z_LW3 32
 #endif
-  static constexpr int LINES = P >= 64 ? 1 : (Shape<N>::P2 > 1 ? PIN_Z_LW3 : 64) / P;
-  // the root solve runs inside the z pass where its transform leaves the
-  // registers for it (three-level lines)
-#ifndef PIN_Z_FUSE
-  static constexpr bool FUSE = Shape<N>::P2 > 1;
-#else
-  static constexpr bool FUSE = PIN_Z_FUSE != 0;
-#endif
+  static constexpr int LW = Shape<N>::P2 > 1 ? PIN_Z_LW3 : (E <= 16 ? 64 : 32);
+  static constexpr int LINES = P >= LW ? 1 : LW / P;
   static constexpr size_t xz = (size_t)XLayoutLines<E, P, 3 * LINES, P1>::kSize * 8;
   static constexpr size_t fz = (size_t)LINES * 6 * field_stride<N>() * 4;
   // the field buffer is followed by the queue of the root solve (one 16-bit
@@ -789,18 +494,18 @@ static cudaError_t set_attrs() {
   using C = Cfg<N>;
   cudaError_t e = set_attrs_xy_all<N, 0>();
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_pass_z<N, C::LINES, false, 3, C::FUSE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  e = cudaFuncSetAttribute(k_pass_z<N, C::LINES, 3, kZCollapse>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)C::smem_z);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_pass_z<N, C::LINES_V, false, 5, C::FUSE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  e = cudaFuncSetAttribute(k_pass_z<N, C::LINES_V, 5, kZCollapse>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)C::smem_zv);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(k_pass_z<N, C::LINES, false, 3, false, true>,
+  e = cudaFuncSetAttribute(k_pass_z<N, C::LINES, 3, kZSource>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_z);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k_fwd_z<N, C::NCF>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_fz);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(k_pass_z<N, C::LINES, true, 3, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  return cudaFuncSetAttribute(k_pass_z<N, C::LINES, 3, kZDump>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               (int)C::smem_z);
 }
 
@@ -829,16 +534,16 @@ static cudaError_t run_z(const ArgsZ& a_in, bool dump, cudaStream_t st) {
   const long nlines = a.nlines;
   // one wave ahead: measured best against none and two waves (384^3 z pass
   // 0.80 -> 0.76 ms, 768^3 5.93 -> 5.89 ms per radius)
-  static const int wave = resident_blocks(k_pass_z<N, C::LINES, false, 3, C::FUSE>, C::threads_z, C::smem_z);
+  static const int wave = resident_blocks(k_pass_z<N, C::LINES, 3, kZCollapse>, C::threads_z, C::smem_z);
   if (!dump && a.nfields <= 6) a.prefetch_blocks = wave;
   if (!dump && a.nfields > 6) {
     const unsigned grid = (unsigned)((nlines + C::LINES_V - 1) / C::LINES_V);
-    k_pass_z<N, C::LINES_V, false, 5, C::FUSE><<<grid, C::threads_zv, C::smem_zv, st>>>(a);
+    k_pass_z<N, C::LINES_V, 5, kZCollapse><<<grid, C::threads_zv, C::smem_zv, st>>>(a);
     return cudaGetLastError();
   }
   const unsigned grid = (unsigned)((nlines + C::LINES - 1) / C::LINES);
-  if (dump) k_pass_z<N, C::LINES, true, 3, false><<<grid, C::threads_z, C::smem_z, st>>>(a);
-  else k_pass_z<N, C::LINES, false, 3, C::FUSE><<<grid, C::threads_z, C::smem_z, st>>>(a);
+  if (dump) k_pass_z<N, C::LINES, 3, kZDump><<<grid, C::threads_z, C::smem_z, st>>>(a);
+  else k_pass_z<N, C::LINES, 3, kZCollapse><<<grid, C::threads_z, C::smem_z, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -846,7 +551,7 @@ template <int N>
 static cudaError_t run_z_source(const ArgsZ& a, cudaStream_t st) {
   using C = Cfg<N>;
   const unsigned grid = (unsigned)((a.nlines + C::LINES - 1) / C::LINES);
-  k_pass_z<N, C::LINES, false, 3, false, true><<<grid, C::threads_z, C::smem_z, st>>>(a);
+  k_pass_z<N, C::LINES, 3, kZSource><<<grid, C::threads_z, C::smem_z, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -862,9 +567,9 @@ static cudaError_t run_fwd_z(const float* src, float2* dst, int nlines, int nhp,
 
 #define PIN_SIZES(X) X(8) X(16) X(32) X(48) X(64) X(96) X(128) X(192) X(256) X(384) X(512) X(768)
 
-bool z_fuses_roots(int n) {
+bool three_level(int n) {
   switch (n) {
-#define CASE(N) case N: return Cfg<N>::FUSE;
+#define CASE(N) case N: return Shape<N>::P2 > 1;
     PIN_SIZES(CASE)
 #undef CASE
     default: return false;

@@ -70,10 +70,10 @@ struct ArgsY {
 };
 
 // A particle whose FP32 collapse is ill-conditioned, finished in FP64 by the
-// redo kernel: kind 0 (near-degenerate eigenvalue pair, queued by the z pass)
-// carries the six FP32 Hessian components; kind 1 (near-tangent or
-// unconverged root, queued by the root kernel) carries the three eigenvalues
-// in h[0..2].
+// redo kernel, both kinds queued by the z pass: kind 0 (near-degenerate
+// eigenvalue pair) carries the six FP32 Hessian components; kind 1
+// (near-tangent or unconverged root) carries the three eigenvalues in
+// h[0..2].
 struct RedoEntry {
   int q;
   float h[6];
@@ -81,9 +81,8 @@ struct RedoEntry {
 };
 
 // z pass: c2r of each field (its z factor already applied by the y pass),
-// then either the eigenvalues of every particle (lam_out, [3][nlines*N];
-// NaN for particles queued for the FP64 redo), or, where z_fuses_roots, the
-// collapse times and running maximum directly, or a dump of the real fields.
+// then the collapse times and running maximum of every particle, or a dump of
+// the real fields.
 struct ArgsZ {
   const float2* src[kMaxFields];
   int nfields;
@@ -92,11 +91,9 @@ struct ArgsZ {
   int prefetch_blocks;  // z pass: prefetch the lines of block + this many into L2 (0: none)
   const float2* tw;
   int nhp;
-  // eigenvalue mode (nfields 6), plus the displacement components (nfields 9)
-  float* lam_out;
-  float* psi_out;   // [3][npart] smoothed displacement of this radius
+  // collapse mode (nfields 6), with the displacement components (nfields 9)
+  float* psi_out;   // [3][npart] smoothed displacement of this radius, for queued particles
   float* vstate;    // [3][npart] displacement at R_max, or null
-  // root and redo kernels
   float* fmax;
   int* idx;
   int scale;
@@ -165,12 +162,9 @@ cudaError_t launch_fwd_z(int n, const float* src, float2* dst, int nlines, int n
                          cudaStream_t st);
 cudaError_t launch_phi2(const float2* T, float2* out, int nx, int ny, int nz, int nhp, double box, float scale,
                         cudaStream_t st);
-// True when the z pass of size n also computes the collapse times and the
-// running maximum (launch_roots is then not called for that size).
-bool z_fuses_roots(int n);
-// Collapse time and running maximum from the eigenvalues the z pass wrote
-// (after it, same stream), then the FP64 redo of every queued particle.
-cudaError_t launch_roots(const ArgsZ& a, cudaStream_t st);
+// True when lines of n points run three-level transforms.
+bool three_level(int n);
+// The FP64 redo of every particle the z pass queued (after it, same stream).
 cudaError_t launch_redo(const ArgsZ& a, cudaStream_t st);
 cudaError_t upload_constant_twiddles();  // per device
 

@@ -196,7 +196,6 @@ extern "C" pin_status pin_collapse_times_noalloc(const void* delta_k, int dtype,
     az.nfields = 6;
     az.nlines = n * n;
     az.npart = n * n * n;
-    az.lam_out = reinterpret_cast<float*>(U);
     az.tw = tw;
     az.nhp = nhp;
     az.fmax = F_max;
@@ -214,7 +213,6 @@ extern "C" pin_status pin_collapse_times_noalloc(const void* delta_k, int dtype,
     if (pin::launch_x(n, tc, 0, ax, cs) != cudaSuccess || pin::launch_y(n, tc, 0, ay, cs) != cudaSuccess ||
         cudaMemsetAsync(redo_count, 0, sizeof(unsigned), cs) != cudaSuccess ||
         pin::launch_z(n, az, false, cs) != cudaSuccess ||
-        (!pin::z_fuses_roots(n) && pin::launch_roots(az, cs) != cudaSuccess) ||
         pin::launch_redo(az, cs) != cudaSuccess)
       return PIN_ECUDA;
   }

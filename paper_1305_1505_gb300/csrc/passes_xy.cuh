@@ -128,13 +128,14 @@ template <int N> struct Stage {
 #ifndef PIN_Y_TMASTORE
 #define PIN_Y_TMASTORE 1
 #endif
-#ifndef PIN_Z_MINB
-#define PIN_Z_MINB 2
-#endif
-// Independent particles per iteration of the collapse loop.
-#ifndef PIN_Z_ILP
-#define PIN_Z_ILP 2
-#endif
+// Two-level lines: with at most 16 values per thread, 192-thread blocks (64
+// threads' worth of lines per pair) six to an SM (56 registers); with more
+// values (48 to 154 registers uncapped), 96-thread blocks eight to an SM.
+// Picoseconds per particle and radius of the whole pass, uncapped 192-thread
+// blocks -> these: 256^3 12.98 -> 11.96, 128^3 14.53 -> 11.30, 64^3 15.49 ->
+// 13.45, 192^3 17.59 -> 12.09, 96^3 18.98 -> 13.82, 512^3 17.17 -> 12.82.
+// With the velocity fields (160 threads): 256^3 19.24 -> 16.20, 64^3 20.13 ->
+// 18.13 (six blocks), 512^3 26.76 -> 17.28 (four).
 // Three-level lines hold half the registers per thread: the z pass is sized
 // for more resident blocks (one line per block, 96 threads, nine blocks per
 // SM at 72 registers: measured against four 192-thread blocks at 80
@@ -151,8 +152,11 @@ template <int N, int TC = 16, int V = 0> struct MinBlocks {
   // resident threads per SM
   static constexpr int xy =
       Shape<N, V>::P2 > 1 ? 512 / (TC * Shape<N, V>::P) : (N >= 384 ? PIN_XY_MINB : 1);
-  static constexpr int z = Shape<N>::P2 > 1 ? PIN_Z_MINB3 : (N >= 384 ? PIN_Z_MINB : 1);
-  static constexpr int zv = Shape<N>::P2 > 1 ? PIN_Z_MINB3V : (N >= 384 ? PIN_Z_MINB : 1);
+  static constexpr int z = Shape<N>::P2 > 1 ? PIN_Z_MINB3 : (Shape<N>::E <= 16 ? 6 : 8);
+  static constexpr int zv = Shape<N>::P2 > 1 ? PIN_Z_MINB3V : (Shape<N>::E <= 16 ? 6 : 4);
+  // the dump and source modes only transform: no cap at the two-level sizes
+  // (192- or 96-thread blocks, at least two or four to an SM at 512)
+  static constexpr int zt = Shape<N>::P2 > 1 ? PIN_Z_MINB3 : (N >= 384 ? 4 : 1);
 };
 
 // ---------------------------------------------------------------- x pass --

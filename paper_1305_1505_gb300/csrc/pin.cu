@@ -534,7 +534,6 @@ pin_status enqueue_radius(pin_plan_t p, int ms, int scale, float* const* dump, f
   az.vstate = (p->velocities && collapse) ? p->vstate : nullptr;
   az.nlines = p->nx * p->ny * p->batch;
   az.npart = az.nlines * p->nz;
-  az.lam_out = reinterpret_cast<float*>(p->U);  // the x-pass spectra are free by now (serial schedule)
   az.tw = p->twz();
   az.nhp = p->nhp;
   az.fmax = p->fmax;
@@ -561,7 +560,6 @@ pin_status enqueue_radius(pin_plan_t p, int ms, int scale, float* const* dump, f
   PIN_CK(p, launch_z(p->nz, az, dump != nullptr, rs.zs));
   PIN_CK(p, mark(5, rs.zs));
   if (!dump) {
-    if (!z_fuses_roots(p->nz)) PIN_CK(p, launch_roots(az, rs.zs));
     PIN_CK(p, launch_redo(az, rs.zs));
   }
   PIN_CK(p, mark(6, rs.zs));
@@ -1208,7 +1206,7 @@ pin_status pin_get_stats(pin_plan_t p, pin_stats* out) {
 
 int pin_kernels_per_call(pin_plan_t p) {
   if (!p) return 0;
-  return (z_fuses_roots(p->nz) ? 4 : 5) * p->nscales;  // x, y, z, [roots,] redo per radius
+  return 4 * p->nscales;  // x, y, z, redo per radius
 }
 
 pin_status pin_profile(pin_plan_t p, int enable) {
@@ -1408,8 +1406,8 @@ pin_status pin_set_schedule(pin_plan_t p, int schedule) {
   pin_status st = check_plan(p);
   if (st != PIN_OK) return st;
   if (schedule < 0 || schedule > 2) return fail(p, PIN_EINVAL, "schedule must be 0, 1 or 2");
-  if (schedule && !z_fuses_roots(p->nz))
-    return fail(p, PIN_EINVAL, "the overlapped schedules need a z pass that computes the collapse times (nz 384, 768)");
+  if (schedule && !three_level(p->nz))
+    return fail(p, PIN_EINVAL, "the overlapped schedules need three-level z lines (nz 384, 768)");
   if (schedule == p->sched) return PIN_OK;
   PIN_CK(p, cudaStreamSynchronize(p->stream));
   if (schedule && !p->s_xy) {
