@@ -722,8 +722,7 @@ static cudaError_t encode(CUtensorMap* tm, int rank, const void* base, const cuu
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-cudaError_t make_tmap_x(CUtensorMap* tm, const float2* src, int nx, int ny, int nhp, int batch, int tc) {
-  const int boxes = (nx + 255) / 256;
+cudaError_t make_tmap_x(CUtensorMap* tm, const float2* src, int nx, int ny, int nhp, int batch, int tc, int boxes) {
   const cuuint64_t dims[2] = {(cuuint64_t)ny * nhp, (cuuint64_t)nx * batch};
   const cuuint64_t strides[1] = {(cuuint64_t)ny * nhp * 8};
   const cuuint32_t box[2] = {(cuuint32_t)tc, (cuuint32_t)(nx / boxes)};
@@ -738,8 +737,7 @@ cudaError_t make_tmap_rows(CUtensorMap* tm, const float2* base, int cols, long l
 }
 
 cudaError_t make_tmap_y(CUtensorMap* tm, const float2* src3, int nx, int ny, int nhp, size_t spec_elems,
-                        int batch, int tc) {
-  const int boxes = (ny + 255) / 256;
+                        int batch, int tc, int boxes) {
   const cuuint64_t dims[4] = {(cuuint64_t)nhp, (cuuint64_t)ny, (cuuint64_t)nx * batch, 3};
   const cuuint64_t strides[3] = {(cuuint64_t)nhp * 8, (cuuint64_t)ny * nhp * 8, (cuuint64_t)spec_elems * 8};
   const cuuint32_t box[4] = {(cuuint32_t)tc, (cuuint32_t)(ny / boxes), 1, 1};

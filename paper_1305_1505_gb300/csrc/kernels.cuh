@@ -19,12 +19,42 @@ namespace pin {
 
 constexpr int kMaxFields = 9;
 
+// Filter support.  W = exp(-k^2 R^2 / 2) underflows: past about kR = 14 the
+// FP32 axis factors {W, k W, k^2 W} / n are exactly zero, and with them every
+// product and every line they multiply.  At 768^3 with 4 Mpc/h cells and 40
+// radii from 120 to 4 Mpc/h, 55 % of the radii have such modes, and 30 % of
+// all z columns, 41 % of all (ky, kz) lines are zero.  A band holds, per
+// radius, the largest |wavenumber index| with a non-zero factor of each axis,
+// {x, y, z, 0}; the x and y passes neither load nor transform what lies
+// outside (per radius of such a run the x pass takes 0.95 instead of 1.62 ms,
+// the y pass 2.35 instead of 3.35).  The z pass reads whole lines: a test per
+// mode costs its issue slots more (3 %) than the loads it saves.  So the
+// columns past a radius's z band have to hold zeros in V; the y pass writes
+// them where the radius before it in the same buffer (prev) had modes, all
+// others are zero already, the radii running from small to large.
+// Nothing but exact zeros is left out, so the results are those of the full
+// passes: a field with a value that is not finite, or so large that an
+// intermediate could overflow (then 0 x inf would make a NaN of a zero), sets
+// *wide, and the passes run full.
+struct BandArgs {
+  const int* band;  // {x, y, z, 0} of this radius; null: full
+  const int* wide;  // non-zero: full
+  const int* prev;  // y pass: the band of the radius before, null: full
+};
+// Band of one radius from the axis factors ([3][n] each).  The z entry of a
+// full axis is nhp - 1, so that it covers the pad columns.
+void fill_band(int* band4, const float* mx, int nx, const float* my, int ny, const float* mz, int nz, int nhp);
+// |Phi0| from which a field runs full: far below where any intermediate of
+// the passes can overflow FP32.
+float wide_limit(int nx, int ny, int nz, double box);
+
 // x pass (lines of length nx): for each output f, dst[f] = IDFT_x(mult[xm[f]]
 // * src).  The source tiles arrive by TMA: tm is a 2D map over src,
 // {ny*nhp columns, batch*nx rows} (realisations stacked along rows), box
 // {tc, nx/boxes}.
 struct ArgsX {
-  CUtensorMap tm;
+  CUtensorMap tm;       // in stage_boxes, for partial bands
+  CUtensorMap tm_full;  // in store_boxes: the fewest, for whole lines
   const float2* src;
   float2* dst[3];
   int xm[3];
@@ -34,6 +64,8 @@ struct ArgsX {
   const float2* tw;   // twiddles: w_N^{p k1} [E][P], then w_P^{p1 k2a} [P2][P1] for three levels
   int nhp;
   int batch;          // realisations stacked back to back (same N, radii)
+  BandArgs band;
+  int col_unit;       // the y pass reads the band's columns in tiles of this many: all of them are stored
   int* err;           // set to 1 if a TMA wait gave up (bounded wait)
   long long wait_cycles;  // budget of a TMA wait in SM clocks; <= 0: the default (2^31)
   CUtensorMap tm_out[3];  // maps of dst[f] (filled at launch when outputs go out by TMA stores)
@@ -46,7 +78,8 @@ struct ArgsX {
 // map over the three source spectra (stored back to back),
 // {nhp, ny, batch*nx, 3}, box {tc, ny/boxes, 1, 1}.
 struct ArgsY {
-  CUtensorMap tm;
+  CUtensorMap tm;       // in stage_boxes, for partial bands
+  CUtensorMap tm_full;  // in store_boxes
   const float2* src[3];
   float2* dst[kMaxFields];
   int sel[kMaxFields];
@@ -64,6 +97,7 @@ struct ArgsY {
   const float2* tw;
   int nhp;
   int batch;
+  BandArgs band;
   int* err;
   long long wait_cycles;
   CUtensorMap tm_out[kMaxFields];  // maps of dst[o] (filled at launch when outputs go out by TMA stores)
@@ -124,11 +158,19 @@ struct PassShape {
 // entry point, so no driver library is linked).  spec_elems is the stride
 // between the spectra the y map spans; tc is the tile width (columns) of the
 // pass that reads the map, one of xy_tile_options.
-cudaError_t make_tmap_x(CUtensorMap* tm, const float2* src, int nx, int ny, int nhp, int batch, int tc);
+// `boxes`: the boxes a tile of rows is moved in (stage_boxes of the pass's
+// schedule for loads, store_boxes for stores).
+cudaError_t make_tmap_x(CUtensorMap* tm, const float2* src, int nx, int ny, int nhp, int batch, int tc, int boxes);
 // 2D map of rows of `cols` complex values (row pitch cols), box {tc, box_rows}
 cudaError_t make_tmap_rows(CUtensorMap* tm, const float2* base, int cols, long long rows, int tc, int box_rows);
 cudaError_t make_tmap_y(CUtensorMap* tm, const float2* src3, int nx, int ny, int nhp, size_t spec_elems,
-                        int batch, int tc);
+                        int batch, int tc, int boxes);
+// Boxes of a staged tile of n rows with E register slots per thread: eighths
+// (quarters where E is no multiple of eight), whole slots each, so that a
+// band's rows are loaded and a band's slots multiplied without a remainder.
+// A TMA box has at most 256 rows, and 768 / 4 rows fit as well.
+constexpr int stage_boxes(int E) { return E % 8 == 0 ? 8 : 4; }
+constexpr int store_boxes(int n) { return (n + 255) / 256; }
 // Radix schedules of the x/y line transforms (fft.cuh ShapeBase<N, V>):
 // 0, the default and the z pass's, and 1.
 constexpr int kRadixVariants = 2;
@@ -176,13 +218,14 @@ cudaError_t upload_constant_twiddles();  // per device
 //   fill_mult        {W, kW, k^2 W} / n of one axis at one radius ([3][n])
 //   fill_twiddles    the line transform's twiddles of one axis
 //   launch_load_phi0 Phi0 = delta / k^2 into the padded layout (C64 or C128
-//                    input, batch realisations back to back)
+//                    input, batch realisations back to back); *wide is set to
+//                    1 where |Phi0| is not below `limit` (the caller clears it)
 int padded_half(int n);
 double correction_dcorr();
 void fill_mult(float* out, int n, double box, double radius);
 void fill_twiddles(float2* t, int n, const PassShape& sh);
 cudaError_t launch_load_phi0(const void* src, int dtype, int nx, int ny, int nz, int nhp, double box, int batch,
-                             float2* phi0, cudaStream_t st);
+                             float2* phi0, int* wide, cudaStream_t st);
 
 // All-FP64 loop of a PIN_FP64 plan (fp64.cu): device bytes of its workspace
 // (FP64 half-spectrum, one full complex cube, the tensor, F_max), the input

@@ -51,10 +51,12 @@ constexpr size_t kOffPhi0 = 0;
 constexpr size_t kOffU = kOffPhi0 + kSpecBytes;
 constexpr size_t kOffV = kOffU + 3 * kSpecBytes;
 constexpr size_t kOffMult = kOffV + 6 * kSpecBytes;
-constexpr size_t kOffTw = kOffMult + kMultBytes;
+constexpr size_t kOffBand = kOffMult + kMultBytes;            // 4 ints per radius
+constexpr size_t kOffTw = kOffBand + kMaxScales * 4 * sizeof(int);
 constexpr size_t kOffCnt = kOffTw + kTwBytes;                 // 3 counters
 constexpr size_t kOffRedoCount = kOffCnt + 4 * sizeof(unsigned long long);
 constexpr size_t kOffErr = kOffRedoCount + 16;                // cleared with the counters
+constexpr size_t kOffWide = kOffErr + 8;                      // as is the word that turns the bands off
 constexpr size_t kStatusBytes = kOffErr + 16 - kOffCnt;      // counters .. error word
 constexpr size_t kOffRedo = (kOffErr + 16 + 255) & ~(size_t)255;
 constexpr size_t kScratchBytes = (kOffRedo + kRedoCap * sizeof(pin::RedoEntry) + 255) & ~(size_t)255;
@@ -72,6 +74,7 @@ unsigned char* g_scratch_ptr[kMaxDevices] = {};
 // pageable host memory has consumed its source when cudaMemcpyAsync returns).
 std::mutex g_stage_mu;
 float g_h_mult[kMultFloats];
+int g_h_band[kMaxScales * 4];
 float2 g_h_tw[kMaxN];
 
 // Once per device, with that device current: the scratch address, the
@@ -126,26 +129,37 @@ extern "C" pin_status pin_collapse_times_noalloc(const void* delta_k, int dtype,
   unsigned long long* cnt = reinterpret_cast<unsigned long long*>(base + kOffCnt);
   unsigned* redo_count = reinterpret_cast<unsigned*>(base + kOffRedoCount);
   int* err = reinterpret_cast<int*>(base + kOffErr);
+  int* band = reinterpret_cast<int*>(base + kOffBand);
+  int* wide = reinterpret_cast<int*>(base + kOffWide);
   pin::RedoEntry* redo_list = reinterpret_cast<pin::RedoEntry*>(base + kOffRedo);
-  CUtensorMap tm_x, tm_y;
+  CUtensorMap tm_x[2], tm_y[2];  // staged and whole-line boxes
   const int tc = sh.tc;  // the default tile width, as a new plan runs
-  if (pin::make_tmap_x(&tm_x, phi0, n, n, nhp, 1, tc) != cudaSuccess ||
-      pin::make_tmap_y(&tm_y, U, n, n, nhp, spec, 1, tc) != cudaSuccess)
-    return PIN_ECUDA;
+  for (int m = 0; m < 2; ++m) {
+    const int boxes = m ? pin::store_boxes(n) : pin::stage_boxes(sh.E);
+    if (pin::make_tmap_x(&tm_x[m], phi0, n, n, nhp, 1, tc, boxes) != cudaSuccess ||
+        pin::make_tmap_y(&tm_y[m], U, n, n, nhp, spec, 1, tc, boxes) != cudaSuccess)
+      return PIN_ECUDA;
+  }
   const double dcorr = pin::correction_dcorr();
   const size_t n3 = (size_t)n * n * n;
   {
     // per radius [3][n] multipliers (cubic grid: one table serves all axes)
     std::lock_guard<std::mutex> lk(g_stage_mu);
-    for (int s = 0; s < nscales; ++s) pin::fill_mult(g_h_mult + (size_t)s * 3 * n, n, box, radii[s]);
+    for (int s = 0; s < nscales; ++s) {
+      float* m = g_h_mult + (size_t)s * 3 * n;
+      pin::fill_mult(m, n, box, radii[s]);
+      pin::fill_band(g_h_band + 4 * s, m, n, m, n, m, n, nhp);
+    }
     pin::fill_twiddles(g_h_tw, n, sh);
     if (cudaMemcpyAsync(mult, g_h_mult, (size_t)nscales * 3 * n * sizeof(float), cudaMemcpyHostToDevice, cs) !=
+            cudaSuccess ||
+        cudaMemcpyAsync(band, g_h_band, (size_t)nscales * 4 * sizeof(int), cudaMemcpyHostToDevice, cs) !=
             cudaSuccess ||
         cudaMemcpyAsync(tw, g_h_tw, (size_t)n * sizeof(float2), cudaMemcpyHostToDevice, cs) != cudaSuccess)
       return PIN_ECUDA;
   }
-  if (pin::launch_load_phi0(delta_k, dtype, n, n, n, nhp, box, 1, phi0, cs) != cudaSuccess) return PIN_ECUDA;
   if (cudaMemsetAsync(cnt, 0, kStatusBytes, cs) != cudaSuccess ||
+      pin::launch_load_phi0(delta_k, dtype, n, n, n, nhp, box, 1, phi0, wide, cs) != cudaSuccess ||
       cudaMemsetAsync(F_max, 0, n3 * sizeof(float), cs) != cudaSuccess ||
       cudaMemsetAsync(scale_idx, 0xFF, n3 * sizeof(int32_t), cs) != cudaSuccess)
     return PIN_ECUDA;
@@ -162,7 +176,8 @@ extern "C" pin_status pin_collapse_times_noalloc(const void* delta_k, int dtype,
     const int s = order[k];
     const float* m = mult + (size_t)s * 3 * n;
     pin::ArgsX ax{};
-    ax.tm = tm_x;
+    ax.tm = tm_x[0];
+    ax.tm_full = tm_x[1];
     ax.src = phi0;
     for (int f = 0; f < 3; ++f) { ax.dst[f] = U + f * spec; ax.xm[f] = f; }
     ax.nout = 3;
@@ -170,10 +185,13 @@ extern "C" pin_status pin_collapse_times_noalloc(const void* delta_k, int dtype,
     ax.mult = m;
     ax.tw = tw;
     ax.nhp = nhp;
+    ax.band = pin::BandArgs{band + 4 * s, wide, nullptr};
+    ax.col_unit = tc;
     ax.batch = 1;
     ax.err = err;
     pin::ArgsY ay{};
-    ay.tm = tm_y;
+    ay.tm = tm_y[0];
+    ay.tm_full = tm_y[1];
     for (int f = 0; f < 3; ++f) ay.src[f] = U + f * spec;
     for (int o = 0; o < 6; ++o) {
       ay.dst[o] = V + vout[o] * spec;
@@ -189,6 +207,7 @@ extern "C" pin_status pin_collapse_times_noalloc(const void* delta_k, int dtype,
     ay.mult_z = m;
     ay.tw = tw;
     ay.nhp = nhp;
+    ay.band = pin::BandArgs{band + 4 * s, wide, k ? band + 4 * order[k - 1] : nullptr};
     ay.batch = 1;
     ay.err = err;
     pin::ArgsZ az{};

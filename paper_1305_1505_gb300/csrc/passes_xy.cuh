@@ -105,37 +105,40 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* tm,
       : "memory");
 }
 
-// Staged-tile geometry of a line length: kBoxes boxes of kRows rows (a box
-// dimension is at most 256).
-template <int N> struct Stage {
-  static constexpr int kBoxes = (N + 255) / 256;
+// Staged-tile geometry of a line: kBoxes boxes of kRows rows, kSlots register
+// slots each.
+template <int N, int V> struct Stage {
+  static constexpr int kBoxes = stage_boxes(Shape<N, V>::E);
+  static constexpr int kRows = N / kBoxes;
+  static constexpr int kSlots = Shape<N, V>::E / kBoxes;
+  static_assert(kRows <= 256 && kSlots * kBoxes == Shape<N, V>::E, "boxes hold whole slots");
+};
+template <int N> struct Store {
+  static constexpr int kBoxes = store_boxes(N);
   static constexpr int kRows = N / kBoxes;
 };
 
-// Resident blocks per SM the register budget is sized for (shared memory
-// already limits the long-line passes to one or two blocks per SM).
-#ifndef PIN_XY_MINB
-#define PIN_XY_MINB 1
-#endif
+// The boxes that hold rows |index| <= b of a line of N points: [0, lo) and
+// [hi, kBoxes).  part: some row of the line lies outside.
+struct BoxRange {
+  int lo, hi;
+  bool part;
+  __device__ __forceinline__ bool has(int box) const { return box < lo || box >= hi; }
+  __device__ __forceinline__ bool edge(int box) const { return part && (box == lo - 1 || box == hi); }
+  __device__ __forceinline__ int count(int boxes) const { return min(boxes, lo + boxes - hi); }
+};
+template <int N, int V>
+__device__ __forceinline__ BoxRange boxes_of(int b) {
+  using G = Stage<N, V>;
+  if (2 * b + 1 >= N) return BoxRange{G::kBoxes, G::kBoxes, false};
+  return BoxRange{b / G::kRows + 1, (N - b) / G::kRows, true};
+}
+
 // Outputs of the x pass, and of the y pass in single-store mode, go out by
 // TMA bulk tensor stores of the output tile (written into the exchange
 // buffer in tile order) instead of per-thread stores: the warps leave the
 // global store queue to the copy engine (x 1.80 -> 1.62 ms, y 3.58 -> 3.36
-// ms per radius at 768^3).  0 selects the per-thread stores.
-#ifndef PIN_X_TMASTORE
-#define PIN_X_TMASTORE 1
-#endif
-#ifndef PIN_Y_TMASTORE
-#define PIN_Y_TMASTORE 1
-#endif
-// Two-level lines: with at most 16 values per thread, 192-thread blocks (64
-// threads' worth of lines per pair) six to an SM (56 registers); with more
-// values (48 to 154 registers uncapped), 96-thread blocks eight to an SM.
-// Picoseconds per particle and radius of the whole pass, uncapped 192-thread
-// blocks -> these: 256^3 12.98 -> 11.96, 128^3 14.53 -> 11.30, 64^3 15.49 ->
-// 13.45, 192^3 17.59 -> 12.09, 96^3 18.98 -> 13.82, 512^3 17.17 -> 12.82.
-// With the velocity fields (160 threads): 256^3 19.24 -> 16.20, 64^3 20.13 ->
-// 18.13 (six blocks), 512^3 26.76 -> 17.28 (four).
+// ms per radius at 768^3).
 // Three-level lines hold half the registers per thread: the z pass is sized
 // for more resident blocks (one line per block, 96 threads, nine blocks per
 // SM at 72 registers: measured against four 192-thread blocks at 80
@@ -148,10 +151,18 @@ template <int N> struct Stage {
 #define PIN_Z_MINB3V 4
 #endif
 template <int N, int TC = 16, int V = 0> struct MinBlocks {
+  using S = Shape<N, V>;
   // three-level x/y blocks (TC columns x P threads) are sized for 512
-  // resident threads per SM
-  static constexpr int xy =
-      Shape<N, V>::P2 > 1 ? 512 / (TC * Shape<N, V>::P) : (N >= 384 ? PIN_XY_MINB : 1);
+  // resident threads per SM; two-level ones for as many blocks as their
+  // shared memory (staged tile, exchange, tables) lets an SM hold, as long as
+  // that leaves a thread registers for its E values and a transform's
+  // temporaries (4 E + 24: uncapped, the band's cases take a third more and
+  // cost the 256^3 y pass a block per SM, 110 -> 131 us)
+  static constexpr int kSmem = 2 * N * TC * 8 + S::kTw * 8 + 12 * N + 1280;
+  static constexpr int kByRegs = 65536 / (TC * S::P * ((4 * S::E + 24 + 7) / 8 * 8));
+  static constexpr int kBySmem = (227 * 1024) / kSmem;
+  static constexpr int kTwo = kBySmem < kByRegs ? kBySmem : kByRegs;
+  static constexpr int xy = S::P2 > 1 ? 512 / (TC * S::P) : (kTwo > 1 ? kTwo : 1);
   static constexpr int z = Shape<N>::P2 > 1 ? PIN_Z_MINB3 : (Shape<N>::E <= 16 ? 6 : 8);
   static constexpr int zv = Shape<N>::P2 > 1 ? PIN_Z_MINB3V : (Shape<N>::E <= 16 ? 6 : 4);
   // the dump and source modes only transform: no cap at the two-level sizes
@@ -159,19 +170,47 @@ template <int N, int TC = 16, int V = 0> struct MinBlocks {
   static constexpr int zt = Shape<N>::P2 > 1 ? PIN_Z_MINB3 : (N >= 384 ? 4 : 1);
 };
 
+// Slots of a staged tile times their axis factors; slots outside the band are
+// zero (their boxes are not loaded).  GUARD: rows of the band's edge boxes
+// that lie outside the band hold whatever an earlier radius or field left
+// there (the x pass stores only the band's ky rows), so they are set to zero
+// instead of being multiplied by their zero factor.
+template <int N, int TC, int V, bool GUARD>
+__device__ __forceinline__ void load_slots(float2 (&v)[Shape<N, V>::E], const float2* s_st, const float* mt,
+                                           const BoxRange& rows, int b0, int p, int c) {
+  using G = Stage<N, V>;
+  constexpr int E = Shape<N, V>::E, P = Shape<N, V>::P;
+  if (!rows.part) {
+#pragma unroll
+    for (int t = 0; t < E; ++t) v[t] = cscale(s_st[(p + P * t) * TC + c], mt[P * t]);
+    return;
+  }
+#pragma unroll
+  for (int b = 0; b < G::kBoxes; ++b) {
+    const bool in = rows.has(b), edge = GUARD && rows.edge(b);
+#pragma unroll
+    for (int i = 0; i < G::kSlots; ++i) {
+      const int t = b * G::kSlots + i, n = p + P * t;
+      v[t] = make_float2(0.f, 0.f);
+      if (in && !(edge && n > b0 && n < N - b0)) v[t] = cscale(s_st[n * TC + c], mt[P * t]);
+    }
+  }
+}
+
 // ---------------------------------------------------------------- x pass --
 // Lines along x: column index col in [0, N*nhp) enumerates (ky, kz); element
 // (kx, col) sits at kx*N*nhp + col, so a row of TC columns is contiguous.  A
 // persistent block walks column tiles; the staged Phi0 tile serves all
 // outputs, and the next tile is requested as soon as the last output has read
 // the current one into registers.  Each output tile leaves by TMA stores
-// (PIN_X_TMASTORE; columns past the last are clipped by the map).
+// (columns past the last are clipped by the map).
 template <int N, int TC, int V>
 __global__ void __launch_bounds__(TC* Shape<N, V>::P, MinBlocks<N, TC, V>::xy)
     k_pass_x(const __grid_constant__ ArgsX a) {
   constexpr int E = Shape<N, V>::E, P = Shape<N, V>::P, NTW = Shape<N, V>::kTw;
   using L = XLayoutCols<E, P, TC, Shape<N, V>::P1>;
-  using G = Stage<N>;
+  using G = Stage<N, V>;
+  using GS = Store<N>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   // staged tile [N][TC]; TMA destinations start on a 128-byte boundary
   float2* s_st = reinterpret_cast<float2*>(smem_raw + ((128 - (smem_u32(smem_raw) & 127)) & 127));
@@ -179,40 +218,57 @@ __global__ void __launch_bounds__(TC* Shape<N, V>::P, MinBlocks<N, TC, V>::xy)
   float2* s_tw = s_x + L::kSize;
   float* s_m = reinterpret_cast<float*>(s_tw + NTW);  // [3][N] multipliers
   __shared__ __align__(8) unsigned long long s_bar;
-  __shared__ float2* s_dst[3];
   __shared__ int s_xm[3];
   const int tid = threadIdx.x, c = tid % TC, p = tid / TC;
   const uint32_t bar = smem_u32(&s_bar);
   for (int i = tid; i < NTW; i += TC * P) s_tw[i] = a.tw[i];
   for (int i = tid; i < 3 * N; i += TC * P) s_m[i] = a.mult[i];
-  if (tid < 3) {
-    s_dst[tid] = a.dst[tid];
-    s_xm[tid] = a.xm[tid];
-  }
+  if (tid < 3) s_xm[tid] = a.xm[tid];
   if (tid == 0) {
     mbar_init(bar, 1);
     mbar_init_fence();
   }
   __syncthreads();
   const int ncols = a.ny * a.nhp;
-  const int tpr = (ncols + TC - 1) / TC;  // tiles per realisation; the last may run past ncols
-  const int ntiles = tpr * a.batch;        // realisation r owns rows [r N, r N + N)
+  // the filter's support (BandArgs): kx boxes, ky rows 0..by and ny-by..ny-1,
+  // columns kz < ncz.  A full plane is walked as one run of columns; a partial
+  // one row by row, ktiles tiles to a row (the last may run past the row's
+  // end: it then computes the first columns of the next row as well, which
+  // come out the same from every tile that holds them).
+  const bool part = a.band.band != nullptr && __ldg(a.band.wide) == 0;
+  const int by = part ? __ldg(a.band.band + 1) : a.ny / 2;
+  const int ncz = part ? min(a.nhp, (__ldg(a.band.band + 2) / a.col_unit + 1) * a.col_unit) : a.nhp;
+  const BoxRange rows = boxes_of<N, V>(part ? __ldg(a.band.band) : N / 2);
+  const bool flat = 2 * by + 1 >= a.ny && ncz >= a.nhp;
+  const int nrows = min(a.ny, 2 * by + 1), ktiles = (ncz + TC - 1) / TC;
+  const int tpr = flat ? (ncols + TC - 1) / TC : nrows * ktiles;  // tiles per realisation; the last may run past ncols
+  const int ntiles = tpr * a.batch;  // realisation r owns rows [r N, r N + N)
+  auto col_of = [&](int t) {  // first column of tile t of a realisation
+    if (flat) return t * TC;
+    const int row = t / ktiles;
+    return (row <= by ? row : a.ny - nrows + row) * a.nhp + (t - row * ktiles) * TC;
+  };
   auto issue = [&](int tile) {
-    const int r = tile / tpr, t = tile % tpr;
-    mbar_expect_tx(bar, N * TC * 8);
+    const int r = tile / tpr, c0 = col_of(tile % tpr);
+    mbar_expect_tx(bar, rows.count(G::kBoxes) * G::kRows * TC * 8);
+    if (!rows.part) {
+#pragma unroll
+      for (int b = 0; b < GS::kBoxes; ++b)
+        tma_load_2d(smem_u32(s_st + b * GS::kRows * TC), &a.tm_full, c0, r * N + b * GS::kRows, bar);
+      return;
+    }
 #pragma unroll
     for (int b = 0; b < G::kBoxes; ++b)
-      tma_load_2d(smem_u32(s_st + b * G::kRows * TC), &a.tm, t * TC, r * N + b * G::kRows, bar);
+      if (rows.has(b)) tma_load_2d(smem_u32(s_st + b * G::kRows * TC), &a.tm, c0, r * N + b * G::kRows, bar);
   };
   if (tid == 0 && (int)blockIdx.x < ntiles) issue(blockIdx.x);
   uint32_t parity = 0;
   // TMA stores: an output tile is written into the exchange buffer in tile
   // order and stored by the copy engine; the next transform's first
   // exchange waits (in the hook) until the engine has read it
-  constexpr bool kStore = PIN_X_TMASTORE != 0;
   bool pending = false;
   auto wait_store = [&] {
-    if (kStore && pending) {
+    if (pending) {
       if (tid == 0) bulk_wait_read();
       __syncthreads();
       pending = false;
@@ -220,19 +276,16 @@ __global__ void __launch_bounds__(TC* Shape<N, V>::P, MinBlocks<N, TC, V>::xy)
   };
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     if (!stage_ready(bar, parity, a.err, a.wait_cycles)) {
-      if (kStore && tid == 0) bulk_wait_all();
+      if (tid == 0) bulk_wait_all();
       return;
     }
     parity ^= 1;
-    const int col = (tile % tpr) * TC + c;
-    const bool ok = col < ncols;
-    const size_t rbase = (size_t)(tile / tpr) * N * ncols;
+    const int col0 = col_of(tile % tpr), row0 = (tile / tpr) * N;
 #pragma unroll 1
     for (int f = 0; f < a.nout; ++f) {
       const float* mt = s_m + s_xm[f] * N + p;
       float2 v[E];
-#pragma unroll
-      for (int t = 0; t < E; ++t) v[t] = cscale(s_st[(p + P * t) * TC + c], mt[P * t]);
+      load_slots<N, TC, V, false>(v, s_st, mt, rows, 0, p, c);
       if (f == a.nout - 1) {
         __syncthreads();  // the tile has been read by every thread
         if (tid == 0 && tile + (int)gridDim.x < ntiles) {
@@ -240,46 +293,36 @@ __global__ void __launch_bounds__(TC* Shape<N, V>::P, MinBlocks<N, TC, V>::xy)
           issue(tile + gridDim.x);
         }
       }
-      if constexpr (kStore) {
-        fft_line<N, L, false, V>(v, p, c, s_x, s_tw, wait_store);
-        __syncthreads();  // every thread has read its last exchange values
+      fft_line<N, L, false, V>(v, p, c, s_x, s_tw, wait_store);
+      __syncthreads();  // every thread has read its last exchange values
 #pragma unroll
-        for (int j = 0; j < E; ++j) s_x[fft_out_index<N, V>(p, j) * TC + c] = v[j];
-        fence_proxy_async();
-        __syncthreads();
-        if (tid == 0) {
-          const int r = tile / tpr, t = tile % tpr;
+      for (int j = 0; j < E; ++j) s_x[fft_out_index<N, V>(p, j) * TC + c] = v[j];
+      fence_proxy_async();
+      __syncthreads();
+      if (tid == 0) {
 #pragma unroll
-          for (int b = 0; b < G::kBoxes; ++b)
-            tma_store_2d(&a.tm_out[f], t * TC, r * N + b * G::kRows, smem_u32(s_x + b * G::kRows * TC));
-          bulk_commit();
-        }
-        pending = true;
-      } else {
-        fft_line<N, L, false, V>(v, p, c, s_x, s_tw);
-        float2* d = s_dst[f] + rbase + (ok ? col : 0);
-#pragma unroll
-        for (int j = 0; j < E; ++j)
-          if (ok) d[(size_t)fft_out_index<N, V>(p, j) * ncols] = v[j];
-        __syncthreads();
+        for (int b = 0; b < GS::kBoxes; ++b)
+          tma_store_2d(&a.tm_out[f], col0, row0 + b * GS::kRows, smem_u32(s_x + b * GS::kRows * TC));
+        bulk_commit();
       }
+      pending = true;
     }
   }
-  if (kStore && tid == 0) bulk_wait_all();
+  if (tid == 0) bulk_wait_all();
 }
 
 // ---------------------------------------------------------------- y pass --
 // Lines along y: a tile is TC consecutive kz of one x plane; element
 // (ky, kz) of plane x sits at (x*N + ky)*nhp + kz.  Columns past nhp are
 // zero-filled by the tensor map and not stored.  Without second stores each
-// output tile leaves by TMA stores (PIN_Y_TMASTORE); with them (DUAL) by
-// per-thread stores.
+// output tile leaves by TMA stores; with them (DUAL) by per-thread stores.
 template <int N, int TC, bool DUAL, int V>
 __global__ void __launch_bounds__(TC* Shape<N, V>::P, MinBlocks<N, TC, V>::xy)
     k_pass_y(const __grid_constant__ ArgsY a) {
   constexpr int E = Shape<N, V>::E, P = Shape<N, V>::P, NTW = Shape<N, V>::kTw;
   using L = XLayoutCols<E, P, TC, Shape<N, V>::P1>;
-  using G = Stage<N>;
+  using G = Stage<N, V>;
+  using GS = Store<N>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   float2* s_st = reinterpret_cast<float2*>(smem_raw + ((128 - (smem_u32(smem_raw) & 127)) & 127));
   float2* s_x = s_st + N * TC;
@@ -310,19 +353,29 @@ __global__ void __launch_bounds__(TC* Shape<N, V>::P, MinBlocks<N, TC, V>::xy)
   }
   __syncthreads();
   const int nhp = a.nhp, nout = a.nout;
-  const int ktiles = (nhp + TC - 1) / TC;
+  // the filter's support (BandArgs): ky boxes and columns kz <= bz
+  const bool part = a.band.band != nullptr && __ldg(a.band.wide) == 0;
+  const int by = part ? __ldg(a.band.band + 1) : N / 2;
+  const BoxRange rows = boxes_of<N, V>(by);
+  const int ktiles = ((part ? __ldg(a.band.band + 2) + 1 : nhp) + TC - 1) / TC;
   const int ntiles = a.nx * a.batch * ktiles;  // x planes of all realisations, back to back
   auto issue = [&](int tile, int src) {
     const int x = tile / ktiles, kz0 = (tile % ktiles) * TC;
-    mbar_expect_tx(bar, N * TC * 8);
+    mbar_expect_tx(bar, rows.count(G::kBoxes) * G::kRows * TC * 8);
+    if (!rows.part) {
+#pragma unroll
+      for (int b = 0; b < GS::kBoxes; ++b)
+        tma_load_4d(smem_u32(s_st + b * GS::kRows * TC), &a.tm_full, kz0, b * GS::kRows, x, src, bar);
+      return;
+    }
 #pragma unroll
     for (int b = 0; b < G::kBoxes; ++b)
-      tma_load_4d(smem_u32(s_st + b * G::kRows * TC), &a.tm, kz0, b * G::kRows, x, src, bar);
+      if (rows.has(b)) tma_load_4d(smem_u32(s_st + b * G::kRows * TC), &a.tm, kz0, b * G::kRows, x, src, bar);
   };
   if (tid == 0 && (int)blockIdx.x < ntiles) issue(blockIdx.x, s_sel[0]);
   uint32_t parity = 0;
   // TMA stores (single-store mode): as in the x pass
-  constexpr bool kStore = PIN_Y_TMASTORE != 0 && !DUAL;
+  constexpr bool kStore = !DUAL;
   bool pending = false;
   auto wait_store = [&] {
     if (kStore && pending) {
@@ -346,8 +399,7 @@ __global__ void __launch_bounds__(TC* Shape<N, V>::P, MinBlocks<N, TC, V>::xy)
       }
       const float* mt = s_m + s_ym[o] * N + p;
       float2 v[E];
-#pragma unroll
-      for (int t = 0; t < E; ++t) v[t] = cscale(s_st[(p + P * t) * TC + c], mt[P * t]);
+      load_slots<N, TC, V, true>(v, s_st, mt, rows, by, p, c);
       const bool last_use = (o == nout - 1) || s_sel[o + 1] != s_sel[o];
       if (last_use) {
         __syncthreads();  // the staged source has been read by every thread
@@ -371,8 +423,8 @@ __global__ void __launch_bounds__(TC* Shape<N, V>::P, MinBlocks<N, TC, V>::xy)
       if constexpr (kStore) fft_line<N, L, false, V>(v, p, c, s_x, s_tw, wait_store);
       else fft_line<N, L, false, V>(v, p, c, s_x, s_tw);
       const bool mi = s_mi[o] != 0;
-      float2* d = s_dst[o] + base;
       if constexpr (DUAL) {
+        float2* d = s_dst[o] + base;
         // outputs with a second store: the same transform with another z
         // factor (displacement components), both stores per register slot so
         // that each slot dies after its two stores
@@ -405,21 +457,45 @@ __global__ void __launch_bounds__(TC* Shape<N, V>::P, MinBlocks<N, TC, V>::xy)
         if (tid == 0) {
           const int kz0 = (tile % ktiles) * TC;
 #pragma unroll
-          for (int b = 0; b < G::kBoxes; ++b)
-            tma_store_2d(&a.tm_out[o], kz0, x * N + b * G::kRows, smem_u32(s_x + b * G::kRows * TC));
+          for (int b = 0; b < GS::kBoxes; ++b)
+            tma_store_2d(&a.tm_out[o], kz0, x * N + b * GS::kRows, smem_u32(s_x + b * GS::kRows * TC));
           bulk_commit();
         }
         pending = true;
         continue;
-      } else {
-#pragma unroll
-        for (int j = 0; j < E; ++j) {
-          float2 w = cscale(v[j], zf);
-          if (mi) w = cmuli(w);
-          if (ok) d[(size_t)fft_out_index<N, V>(p, j) * nhp] = w;
-        }
       }
       __syncthreads();
+    }
+  }
+  // columns past the band that the radius before had: zeros
+  const int zend = part ? ((a.band.prev ? __ldg(a.band.prev + 2) + 1 : nhp) + TC - 1) / TC : ktiles;
+  if (zend > ktiles) {
+    const int zt = zend - ktiles, nz0 = a.nx * a.batch * zt;
+    if constexpr (kStore) {
+      wait_store();
+      for (int i = tid; i < N * TC; i += TC * P) s_x[i] = make_float2(0.f, 0.f);
+      fence_proxy_async();
+      __syncthreads();
+      if (tid == 0)
+        for (int i = blockIdx.x; i < nz0; i += gridDim.x) {
+          const int x = i / zt, kz0 = (ktiles + i % zt) * TC;
+          for (int o = 0; o < nout; ++o)
+#pragma unroll
+            for (int b = 0; b < GS::kBoxes; ++b)
+              tma_store_2d(&a.tm_out[o], kz0, x * N + b * GS::kRows, smem_u32(s_x + b * GS::kRows * TC));
+          bulk_commit();
+        }
+    } else {
+      for (int i = blockIdx.x; i < nz0; i += gridDim.x) {
+        const int x = i / zt, kz = (ktiles + i % zt) * TC + c;
+        if (kz >= nhp) continue;
+        for (int o = 0; o < nout; ++o)
+          for (int r = p; r < N; r += P) {
+            const size_t at = ((size_t)x * N + r) * nhp + kz;
+            s_dst[o][at] = make_float2(0.f, 0.f);
+            if (s_dst2[o] != nullptr) s_dst2[o][at] = make_float2(0.f, 0.f);
+          }
+      }
     }
   }
   if (kStore && tid == 0) bulk_wait_all();
@@ -483,12 +559,10 @@ template <int N, int TC, int V>
 static cudaError_t run_x(const ArgsX& a_in, cudaStream_t st) {
   using C = CfgXY<N, TC, V>;
   ArgsX a = a_in;
-  if (PIN_X_TMASTORE) {
-    // output maps: the same geometry as the source map, one per output
-    for (int f = 0; f < a.nout; ++f) {
-      const cudaError_t e = make_tmap_x(&a.tm_out[f], a.dst[f], N, a.ny, a.nhp, a.batch, TC);
-      if (e != cudaSuccess) return e;
-    }
+  // output maps: the source map's geometry in store boxes, one per output
+  for (int f = 0; f < a.nout; ++f) {
+    const cudaError_t e = make_tmap_x(&a.tm_out[f], a.dst[f], N, a.ny, a.nhp, a.batch, TC, Store<N>::kBoxes);
+    if (e != cudaSuccess) return e;
   }
   const long ntiles = (((long)a.ny * a.nhp + TC - 1) / TC) * a.batch;
   const unsigned grid = persistent_grid(k_pass_x<N, TC, V>, C::threads, C::smem, ntiles);
@@ -502,25 +576,20 @@ static cudaError_t run_y(const ArgsY& a, cudaStream_t st) {
   const long ntiles = (long)a.nx * a.batch * ((a.nhp + TC - 1) / TC);
   bool dual = false;
   for (int o = 0; o < a.nout; ++o) dual = dual || a.dst2[o] != nullptr;
-  if (PIN_Y_TMASTORE && !dual) {
-    // output maps: rows (x, ky) of nhp values, boxes of the staged tile's rows
+  if (!dual) {
+    // output maps: rows (x, ky) of nhp values in store boxes
     ArgsY b = a;
     for (int o = 0; o < b.nout; ++o) {
       const cudaError_t e = make_tmap_rows(&b.tm_out[o], b.dst[o], b.nhp, (long long)b.nx * b.batch * N, TC,
-                                           Stage<N>::kRows);
+                                           Store<N>::kRows);
       if (e != cudaSuccess) return e;
     }
     const unsigned grid = persistent_grid(k_pass_y<N, TC, false, V>, C::threads, C::smem, ntiles);
     k_pass_y<N, TC, false, V><<<grid, C::threads, C::smem, st>>>(b);
     return cudaGetLastError();
   }
-  if (dual) {
-    const unsigned grid = persistent_grid(k_pass_y<N, TC, true, V>, C::threads, C::smem, ntiles);
-    k_pass_y<N, TC, true, V><<<grid, C::threads, C::smem, st>>>(a);
-  } else {
-    const unsigned grid = persistent_grid(k_pass_y<N, TC, false, V>, C::threads, C::smem, ntiles);
-    k_pass_y<N, TC, false, V><<<grid, C::threads, C::smem, st>>>(a);
-  }
+  const unsigned grid = persistent_grid(k_pass_y<N, TC, true, V>, C::threads, C::smem, ntiles);
+  k_pass_y<N, TC, true, V><<<grid, C::threads, C::smem, st>>>(a);
   return cudaGetLastError();
 }
 

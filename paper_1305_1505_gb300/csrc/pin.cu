@@ -28,6 +28,12 @@
 
 using namespace pin;
 
+// multiplier sets of a plan: one per radius (at most 64, pin_set_radii may
+// change the list), then the R = 0 set of the unsmoothed products
+constexpr int kMaxScales = 64;
+constexpr int kBandWide = 4 * (kMaxScales + 1);  // index of the "field runs full" word
+constexpr int kBandInts = kBandWide + 4;
+
 struct pin_plan_s {
   int nx = 0, ny = 0, nz = 0, nhp = 0, nscales = 0, correction = 1, precision = 0;
   int batch = 1;          // realisations sharing the grid and radii
@@ -49,6 +55,7 @@ struct pin_plan_s {
   float* fmax = nullptr;
   int* idx = nullptr;
   float* mult = nullptr;  // kMaxScales + 1 sets of 3 x n; set kMaxScales has R = 0
+  int* band = nullptr;    // behind mult: the filter's support of each set (4 ints), then the word that turns it off
   float2* tw = nullptr;
   unsigned long long* counters = nullptr;  // [0] eig redo, [1] root redo, [2] queue overflow
   RedoEntry* redo_list = nullptr;          // FP64 redo queue, reused by every radius
@@ -56,7 +63,7 @@ struct pin_plan_s {
   unsigned redo_cap = 0;
   int* err = nullptr;                      // set by a pass whose bounded TMA wait gave up
   long long wait_cycles = 0;               // TMA wait budget of the x/y passes (0: default)
-  CUtensorMap tm_x{}, tm_y{};              // Phi0 -> x pass, U[3] -> y pass
+  CUtensorMap tm_x[2]{}, tm_y[2]{};        // Phi0 -> x pass, U[3] -> y pass: staged and whole-line boxes
   int tc_x = 0, tc_y = 0;                  // tile widths (columns per block) of the x and y passes
   int vx = 0, vy = 0;                      // radix schedules of the x and y line transforms
   bool ic_set = false;
@@ -92,6 +99,9 @@ struct pin_plan_s {
   const float* mx(int ms) const { return mult + ms * mult_set(); }
   const float* my(int ms) const { return mx(ms) + 3 * (size_t)nx; }
   const float* mz(int ms) const { return my(ms) + 3 * (size_t)ny; }
+  BandArgs bands(int ms, int prev = -1) const {
+    return BandArgs{band + 4 * ms, band + kBandWide, prev < 0 ? nullptr : band + 4 * prev};
+  }
   const float2* twx() const { return tw + tw_off[0]; }
   const float2* twy() const { return tw + tw_off[1]; }
   const float2* twz() const { return tw + tw_off[2]; }
@@ -138,6 +148,31 @@ void fill_mult(float* out, int n, double box, double radius) {
   }
 }
 
+void fill_band(int* band4, const float* mx, int nx, const float* my, int ny, const float* mz, int nz, int nhp) {
+  const float* m[3] = {mx, my, mz};
+  const int n[3] = {nx, ny, nz};
+  for (int a = 0; a < 3; ++a) {
+    band4[a] = 0;
+    for (int i = 0; i < n[a]; ++i) {
+      const int s = i < n[a] / 2 ? i : n[a] - i;
+      for (int k = 0; k < 3; ++k)
+        if (m[a][(size_t)k * n[a] + i] != 0.0f) band4[a] = std::max(band4[a], s);
+    }
+  }
+  if (band4[2] == nz / 2) band4[2] = nhp - 1;
+  band4[3] = 0;
+}
+
+// Every intermediate is a sum of at most nx ny nz terms |Phi0| times factors
+// whose product over the axes is at most max(1, k)^4 / (nx ny nz), k the
+// largest wavenumber of an axis.
+float wide_limit(int nx, int ny, int nz, double box) {
+  (void)ny;
+  (void)nz;
+  const double k = std::max(1.0, M_PI * nx / box);  // cubic cells: the Nyquist wavenumber of every axis
+  return (float)(1e36 / (k * k * k * k));
+}
+
 // Twiddles of one axis: w_n^{p k1} in [k1][p] order; for a three-level line
 // (P = P1 P2) then w_P^{p1 k2a} in [k2a][p1] order.
 void fill_twiddles(float2* t, int n, const PassShape& sh) {
@@ -159,7 +194,7 @@ void fill_twiddles(float2* t, int n, const PassShape& sh) {
 // zero).  Cubic cells: the side along x is `box`, L_y = box ny / nx,
 // L_z = box nz / nx.
 __global__ void k_load_phi0(const void* src, int dtype, int nx, int ny, int nz, int nhp, double box, int batch,
-                            float2* phi0) {
+                            float limit, float2* phi0, int* wide) {
   const int nh = nz / 2 + 1;
   const size_t total = (size_t)nx * ny * nhp * batch;
   const double kfx = 2.0 * M_PI / box, kfy = 2.0 * M_PI / (ny == nx ? box : box * ny / nx),
@@ -189,6 +224,7 @@ __global__ void k_load_phi0(const void* src, int dtype, int nx, int ny, int nz, 
       }
     }
     phi0[i] = out;
+    if (!(fabsf(out.x) < limit && fabsf(out.y) < limit)) *wide = 1;
   }
 }
 
@@ -225,11 +261,12 @@ cudaError_t copy_to_host(void* host_dst, const void* dev_src, size_t bytes, cuda
 }
 
 cudaError_t launch_load_phi0(const void* src, int dtype, int nx, int ny, int nz, int nhp, double box, int batch,
-                             float2* phi0, cudaStream_t st) {
+                             float2* phi0, int* wide, cudaStream_t st) {
   const size_t total = (size_t)nx * ny * nhp * batch;
   const int threads = 256;
   const unsigned blocks = (unsigned)std::min<size_t>((total + threads - 1) / threads, 152 * 64);
-  k_load_phi0<<<blocks, threads, 0, st>>>(src, dtype, nx, ny, nz, nhp, box, batch, phi0);
+  k_load_phi0<<<blocks, threads, 0, st>>>(src, dtype, nx, ny, nz, nhp, box, batch, wide_limit(nx, ny, nz, box), phi0,
+                                           wide);
   return cudaGetLastError();
 }
 
@@ -310,17 +347,13 @@ unsigned redo_capacity(size_t n3, int batch) {
 
 int batch_of(const pin_plan_desc* d) { return d->batch <= 0 ? 1 : d->batch; }
 
-// multiplier sets of a plan: one per radius (at most 64, pin_set_radii may
-// change the list), then the R = 0 set of the unsmoothed products
-constexpr int kMaxScales = 64;
-
 size_t footprint(int nx, int ny, int nz, int nscales, int batch, bool velocities, bool fp64) {
   (void)nscales;
   const size_t spec = (size_t)nx * ny * padded_half(nz) * batch;
   const size_t n3 = (size_t)nx * ny * nz * batch;
   return (fp64 ? fp64_workspace_bytes(nx, ny, nz) : 0) + spec * 8 * (velocities ? 13 : 10) + n3 * 8 +
          (velocities ? n3 * 24 : 0) +
-         (size_t)(kMaxScales + 1) * 3 * (nx + ny + nz) * 4 + (size_t)(nx + ny + nz + 3 * 64) * 8 + 64 +
+         (size_t)(kMaxScales + 1) * 3 * (nx + ny + nz) * 4 + kBandInts * sizeof(int) + (size_t)(nx + ny + nz + 3 * 64) * 8 + 64 +
          (size_t)redo_capacity((size_t)nx * ny * nz, batch) * sizeof(RedoEntry) + 16 + sizeof(int);
 }
 
@@ -425,16 +458,45 @@ std::vector<float> mult_table(pin_plan_t p) {
   return mult;
 }
 
+// Bands of the plan's multiplier sets, from the host copy of the factors.
+std::vector<int> band_table(pin_plan_t p, const std::vector<float>& mult) {
+  std::vector<int> band((size_t)kBandWide, 0);
+  for (int s = 0; s <= kMaxScales; ++s) {
+    if (s < kMaxScales && s >= p->nscales) continue;
+    const float* m = mult.data() + (size_t)s * p->mult_set();
+    fill_band(band.data() + 4 * s, m, p->nx, m + 3 * (size_t)p->nx, p->ny, m + 3 * (size_t)(p->nx + p->ny), p->nz,
+              p->nhp);
+  }
+  return band;
+}
+
+// Source maps {staged boxes, whole-line boxes} of the x pass over one spectrum
+// and of the y pass over the three spectra at src, for tile width tc.
+cudaError_t source_maps_x(pin_plan_t p, CUtensorMap* tm, const float2* src, int batch, int tc) {
+  cudaError_t e = make_tmap_x(tm, src, p->nx, p->ny, p->nhp, batch, tc, stage_boxes(p->shape_x.E));
+  if (e == cudaSuccess) e = make_tmap_x(tm + 1, src, p->nx, p->ny, p->nhp, batch, tc, store_boxes(p->nx));
+  return e;
+}
+cudaError_t source_maps_y(pin_plan_t p, CUtensorMap* tm, const float2* src, int batch, int tc) {
+  cudaError_t e = make_tmap_y(tm, src, p->nx, p->ny, p->nhp, p->field_elems, batch, tc, stage_boxes(p->shape_y.E));
+  if (e == cudaSuccess)
+    e = make_tmap_y(tm + 1, src, p->nx, p->ny, p->nhp, p->field_elems, batch, tc, store_boxes(p->ny));
+  return e;
+}
+
 // x pass of one radius (mult set `ms`): Phi0 -> U[0..2] with the x factors
 // W, k W, k^2 W.
 ArgsX radius_args_x(pin_plan_t p, int ms) {
   ArgsX ax{};
-  ax.tm = p->tm_x;
+  ax.tm = p->tm_x[0];
+  ax.tm_full = p->tm_x[1];
   ax.src = p->phi0;
   for (int f = 0; f < 3; ++f) { ax.dst[f] = spec(p, p->U, f); ax.xm[f] = f; }
   ax.nout = 3;
   ax.ny = p->ny;
   ax.mult = p->mx(ms);
+  ax.band = p->bands(ms);
+  ax.col_unit = p->tc_y;
   ax.tw = p->twx();
   ax.nhp = p->nhp;
   ax.batch = p->batch;
@@ -449,14 +511,15 @@ ArgsX radius_args_x(pin_plan_t p, int ms) {
 // With the velocities of a collapse call, the smoothed displacement
 // psi = i k W Phi0 shares the y transforms of xz (psi_x: z factor W), zz
 // (psi_z: z factor k W) and yz (psi_y: z factor W).
-ArgsY radius_args_y(pin_plan_t p, int ms, bool collapse, float2* vbuf = nullptr) {
+ArgsY radius_args_y(pin_plan_t p, int ms, bool collapse, float2* vbuf = nullptr, int prev = -1) {
   if (!vbuf) vbuf = p->V;
   static const int vout[6] = {0, 3, 4, 1, 2, 5};
   static const int sel[6] = {2, 1, 1, 0, 0, 0};
   static const int ym[6] = {0, 1, 0, 2, 0, 1};
   static const int zm[6] = {0, 0, 1, 0, 2, 1};
   ArgsY ay{};
-  ay.tm = p->tm_y;
+  ay.tm = p->tm_y[0];
+  ay.tm_full = p->tm_y[1];
   for (int f = 0; f < 3; ++f) ay.src[f] = spec(p, p->U, f);
   for (int o = 0; o < 6; ++o) {
     ay.dst[o] = spec(p, vbuf, vout[o]);
@@ -481,6 +544,7 @@ ArgsY radius_args_y(pin_plan_t p, int ms, bool collapse, float2* vbuf = nullptr)
   ay.nz = p->nz;
   ay.mult = p->my(ms);
   ay.mult_z = p->mz(ms);
+  ay.band = p->bands(ms, prev);
   ay.tw = p->twy();
   ay.nhp = p->nhp;
   ay.batch = p->batch;
@@ -492,12 +556,14 @@ ArgsY radius_args_y(pin_plan_t p, int ms, bool collapse, float2* vbuf = nullptr)
 // Where the passes of one radius of the collapse loop run: the x and y passes
 // on xs, the z pass and the FP64 redo on zs, the y outputs in vbuf; the y pass
 // first waits for y_wait (if set), y_done is recorded after it (and zs waits
-// for it), z_done after the redo.  The serial schedule is xs = zs = the
-// plan's stream, vbuf = V, no events.
+// for it), z_done after the redo.  prev: the multiplier set of the radius
+// that wrote vbuf before in this call, -1 for the first.  The serial schedule
+// is xs = zs = the plan's stream, vbuf = V, no events.
 struct RadiusSched {
   cudaStream_t xs, zs;
   float2* vbuf;
   cudaEvent_t y_wait, y_done, z_done;
+  int prev;
 };
 
 // Filter-and-transform passes of one radius (mult set `ms`), ending in the
@@ -506,7 +572,7 @@ struct RadiusSched {
 pin_status enqueue_radius(pin_plan_t p, int ms, int scale, float* const* dump, float* source = nullptr,
                           const RadiusSched* sched = nullptr) {
   const bool collapse = dump == nullptr && source == nullptr;
-  const RadiusSched rs = sched ? *sched : RadiusSched{p->stream, p->stream, p->V, nullptr, nullptr, nullptr};
+  const RadiusSched rs = sched ? *sched : RadiusSched{p->stream, p->stream, p->V, nullptr, nullptr, nullptr, -1};
   const bool rec = p->profile && collapse && !p->events.empty();
   auto mark = [&](int k, cudaStream_t st) {
     return rec ? cudaEventRecordWithFlags(p->events[7 * scale + k], st, cudaEventRecordExternal) : cudaSuccess;
@@ -518,7 +584,7 @@ pin_status enqueue_radius(pin_plan_t p, int ms, int scale, float* const* dump, f
   if (rs.y_wait) PIN_CK(p, cudaStreamWaitEvent(rs.xs, rs.y_wait, 0));
 
   PIN_CK(p, mark(2, rs.xs));
-  const ArgsY ay = radius_args_y(p, ms, collapse, rs.vbuf);
+  const ArgsY ay = radius_args_y(p, ms, collapse, rs.vbuf, rs.prev);
   PIN_CK(p, launch_y(p->ny, p->tc_y, p->vy, ay, rs.xs));
   PIN_CK(p, mark(3, rs.xs));
   if (rs.y_done) {
@@ -575,7 +641,8 @@ pin_status enqueue_collapse(pin_plan_t p) {
   if (p->sched == 0) {
     for (int k = 0; k < p->nscales; ++k) {
       const int s = p->order[k];
-      pin_status st = enqueue_radius(p, s, s, nullptr);
+      const RadiusSched rs{p->stream, p->stream, p->V, nullptr, nullptr, nullptr, k ? p->order[k - 1] : -1};
+      pin_status st = enqueue_radius(p, s, s, nullptr, nullptr, &rs);
       if (st != PIN_OK) return st;
     }
     return PIN_OK;
@@ -594,7 +661,8 @@ pin_status enqueue_collapse(pin_plan_t p) {
   for (int k = 0; k < p->nscales; ++k) {
     const int s = p->order[k];
     RadiusSched rs{p->s_xy, p->s_z, (nbuf == 2 && (k & 1)) ? p->V2 : p->V,
-                   k >= nbuf ? p->cap_ev[2 + 2 * (k - nbuf)] : nullptr, p->cap_ev[1 + 2 * k], p->cap_ev[2 + 2 * k]};
+                   k >= nbuf ? p->cap_ev[2 + 2 * (k - nbuf)] : nullptr, p->cap_ev[1 + 2 * k], p->cap_ev[2 + 2 * k],
+                   k >= nbuf ? p->order[k - nbuf] : -1};
     pin_status st = enqueue_radius(p, s, s, nullptr, nullptr, &rs);
     if (st != PIN_OK) return st;
   }
@@ -687,6 +755,23 @@ pin_status upload_axis_twiddles(pin_plan_t p, int axis, int v) {
   return PIN_OK;
 }
 
+// Re-encode the plan's tensor maps for new tile widths; the captured graph
+// holds the old maps and launch shapes, so it is dropped (after the stream
+// drains) and captured again by the next call.
+pin_status apply_tiles(pin_plan_t p, int tc_x, int tc_y) {
+  CUtensorMap mx[2], my[2];
+  if (source_maps_x(p, mx, p->phi0, p->batch, tc_x) != cudaSuccess ||
+      source_maps_y(p, my, p->U, p->batch, tc_y) != cudaSuccess)
+    return fail(p, PIN_ECUDA, "tensor map encoding failed");
+  PIN_CK(p, cudaStreamSynchronize(p->stream));
+  drop_graph(p);
+  std::copy(mx, mx + 2, p->tm_x);
+  std::copy(my, my + 2, p->tm_y);
+  p->tc_x = tc_x;
+  p->tc_y = tc_y;
+  return PIN_OK;
+}
+
 // Switches the radix schedules of the x and y passes (twiddles, shapes).
 pin_status apply_radix(pin_plan_t p, int vx, int vy) {
   if (vx == p->vx && vy == p->vy) return PIN_OK;
@@ -699,24 +784,7 @@ pin_status apply_radix(pin_plan_t p, int vx, int vy) {
   p->vy = vy;
   p->shape_x = pass_shape_xy(p->nx, vx);
   p->shape_y = pass_shape_xy(p->ny, vy);
-  return PIN_OK;
-}
-
-// Re-encode the plan's tensor maps for new tile widths; the captured graph
-// holds the old maps and launch shapes, so it is dropped (after the stream
-// drains) and captured again by the next call.
-pin_status apply_tiles(pin_plan_t p, int tc_x, int tc_y) {
-  CUtensorMap mx, my;
-  if (make_tmap_x(&mx, p->phi0, p->nx, p->ny, p->nhp, p->batch, tc_x) != cudaSuccess ||
-      make_tmap_y(&my, p->U, p->nx, p->ny, p->nhp, p->field_elems, p->batch, tc_y) != cudaSuccess)
-    return fail(p, PIN_ECUDA, "tensor map encoding failed");
-  PIN_CK(p, cudaStreamSynchronize(p->stream));
-  drop_graph(p);
-  p->tm_x = mx;
-  p->tm_y = my;
-  p->tc_x = tc_x;
-  p->tc_y = tc_y;
-  return PIN_OK;
+  return apply_tiles(p, p->tc_x, p->tc_y);  // the boxes of the source maps follow the schedule
 }
 
 // Mean device time (ms) of `reps` launches of the first radius's x or y pass
@@ -725,8 +793,11 @@ pin_status apply_tiles(pin_plan_t p, int tc_x, int tc_y) {
 pin_status time_pass(pin_plan_t p, bool y_pass, int tc, int reps, float* ms) {
   ArgsX ax = radius_args_x(p, 0);
   ArgsY ay = radius_args_y(p, 0, true);
-  cudaError_t e = y_pass ? make_tmap_y(&ay.tm, p->U, p->nx, p->ny, p->nhp, p->field_elems, p->batch, tc)
-                         : make_tmap_x(&ax.tm, p->phi0, p->nx, p->ny, p->nhp, p->batch, tc);
+  ax.band = ay.band = BandArgs{};  // full passes, whatever the first radius filters out
+  CUtensorMap tm[2];
+  cudaError_t e = y_pass ? source_maps_y(p, tm, p->U, p->batch, tc) : source_maps_x(p, tm, p->phi0, p->batch, tc);
+  (y_pass ? ay.tm : ax.tm) = tm[0];
+  (y_pass ? ay.tm_full : ax.tm_full) = tm[1];
   if (e != cudaSuccess) return fail(p, PIN_ECUDA, "tensor map encoding failed");
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   PIN_CK(p, cudaEventCreate(&e0));
@@ -813,7 +884,7 @@ pin_status pin_plan(pin_plan_t* out, const pin_plan_desc* d) {
       A(&p->V, (p->velocities ? 9 : 6) * p->field_elems * 8) != cudaSuccess ||
       (p->velocities && (A(&p->psi, 3 * n3 * 4) != cudaSuccess || A(&p->vstate, 3 * n3 * 4) != cudaSuccess)) ||
       A(&p->fmax, n3 * 4) != cudaSuccess || A(&p->idx, n3 * 4) != cudaSuccess ||
-      A(&p->mult, mult_elems * 4) != cudaSuccess || A(&p->tw, tw_elems * 8) != cudaSuccess ||
+      A(&p->mult, mult_elems * 4 + kBandInts * sizeof(int)) != cudaSuccess || A(&p->tw, tw_elems * 8) != cudaSuccess ||
       A(&p->counters, 3 * sizeof(unsigned long long)) != cudaSuccess ||
       A(&p->redo_list, (size_t)p->redo_cap * sizeof(RedoEntry)) != cudaSuccess ||
       A(&p->redo_count, sizeof(unsigned)) != cudaSuccess || A(&p->err, sizeof(int)) != cudaSuccess ||
@@ -824,21 +895,34 @@ pin_status pin_plan(pin_plan_t* out, const pin_plan_desc* d) {
     cudaGetLastError();
     return bail(PIN_ENOMEM);
   }
+  p->band = reinterpret_cast<int*>(p->mult + mult_elems);
   const std::vector<float> mult = mult_table(p);
+  const std::vector<int> band = band_table(p, mult);
   std::vector<float2> tw(tw_elems);
   for (int a = 0; a < 3; ++a) fill_twiddles(tw.data() + p->tw_off[a], ns[a], *shapes[a]);
   if (cudaMemcpy(p->mult, mult.data(), mult_elems * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemset(p->band, 0, kBandInts * sizeof(int)) != cudaSuccess ||
+      cudaMemcpy(p->band, band.data(), band.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(p->tw, tw.data(), tw.size() * 8, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemset(p->counters, 0, 3 * sizeof(unsigned long long)) != cudaSuccess ||
       cudaMemset(p->err, 0, sizeof(int)) != cudaSuccess)
     return bail(PIN_ECUDA);
   p->tc_x = p->shape_x.tc;
   p->tc_y = p->shape_y.tc;
-  if (make_tmap_x(&p->tm_x, p->phi0, p->nx, p->ny, p->nhp, p->batch, p->tc_x) != cudaSuccess ||
-      make_tmap_y(&p->tm_y, p->U, p->nx, p->ny, p->nhp, p->field_elems, p->batch, p->tc_y) != cudaSuccess)
+  if (source_maps_x(p, p->tm_x, p->phi0, p->batch, p->tc_x) != cudaSuccess ||
+      source_maps_y(p, p->tm_y, p->U, p->batch, p->tc_y) != cudaSuccess)
     return bail(PIN_ECUDA);
   *out = p;
   return PIN_OK;
+}
+
+// Phi0 of the field in src (device-readable), and whether the field is one
+// that runs full (BandArgs).
+static cudaError_t load_phi0(pin_plan_t p, const void* src, int dtype) {
+  const cudaError_t e = cudaMemsetAsync(p->band + kBandWide, 0, sizeof(int), p->stream);
+  if (e != cudaSuccess) return e;
+  return launch_load_phi0(src, dtype, p->nx, p->ny, p->nz, p->nhp, p->box, p->batch, p->phi0, p->band + kBandWide,
+                          p->stream);
 }
 
 pin_status pin_set_ic(pin_plan_t p, const void* delta_k, int dtype, int on_device) {
@@ -865,7 +949,7 @@ pin_status pin_set_ic(pin_plan_t p, const void* delta_k, int dtype, int on_devic
       src = p->V;
     }
   }
-  PIN_CK(p, launch_load_phi0(src, dtype, p->nx, p->ny, p->nz, p->nhp, p->box, p->batch, p->phi0, p->stream));
+  PIN_CK(p, load_phi0(p, src, dtype));
   if (p->d64) PIN_CK(p, fp64_load(src, dtype, p->nx, p->ny, p->nz, p->d64, p->stream));
   if (!on_device) PIN_CK(p, cudaStreamSynchronize(p->stream));
   p->ic_set = true;
@@ -889,7 +973,7 @@ pin_status pin_set_ic_seed(pin_plan_t p, uint64_t seed, const pin_spectrum* ps) 
   PIN_CK(p, cudaMemcpyAsync(keys_dev, keys.data(), keys.size() * sizeof(uint64_t), cudaMemcpyHostToDevice,
                             p->stream));
   PIN_CK(p, generate_ic(p->nx, p->box, keys_dev, p->batch, amp, ps->ns, ps->gamma, field, p->stream));
-  PIN_CK(p, launch_load_phi0(field, PIN_C64, p->nx, p->ny, p->nz, p->nhp, p->box, p->batch, p->phi0, p->stream));
+  PIN_CK(p, load_phi0(p, field, PIN_C64));
   if (p->d64) PIN_CK(p, fp64_load(field, PIN_C64, p->nx, p->ny, p->nz, p->d64, p->stream));
   PIN_CK(p, cudaStreamSynchronize(p->stream));  // the host key vector goes out of scope
   p->ic_set = true;
@@ -1024,8 +1108,11 @@ static cudaError_t enqueue_gradient(pin_plan_t p, float2* phi, float2* a0, float
   const size_t n3 = p->n3();
   const int r0 = kMaxScales;  // the R = 0 multiplier set
   ArgsX ax{};
-  cudaError_t e = make_tmap_x(&ax.tm, phi, p->nx, p->ny, p->nhp, 1, p->tc_x);
+  CUtensorMap tm[2];
+  cudaError_t e = source_maps_x(p, tm, phi, 1, p->tc_x);
   if (e != cudaSuccess) return e;
+  ax.tm = tm[0];
+  ax.tm_full = tm[1];
   ax.src = phi;
   ax.dst[0] = a0;
   ax.dst[1] = a0 + p->field_elems;
@@ -1043,8 +1130,10 @@ static cudaError_t enqueue_gradient(pin_plan_t p, float2* phi, float2* a0, float
   if (e != cudaSuccess) return e;
   // psi_x <- a1 (k_x), psi_y <- a0 (k_y), psi_z <- a0 (z: k_z); all times i
   ArgsY ay{};
-  e = make_tmap_y(&ay.tm, a0, p->nx, p->ny, p->nhp, p->field_elems, 1, p->tc_y);
+  e = source_maps_y(p, tm, a0, 1, p->tc_y);
   if (e != cudaSuccess) return e;
+  ay.tm = tm[0];
+  ay.tm_full = tm[1];
   ay.src[0] = a0;
   ay.src[1] = a0 + p->field_elems;
   ay.src[2] = a0 + 2 * p->field_elems;
@@ -1125,7 +1214,10 @@ pin_status pin_displacements_2lpt(pin_plan_t p, float* psi2, int on_device) {
   if (st == PIN_OK && e == cudaSuccess) {
     const int r0 = kMaxScales;
     ArgsY ay{};
-    e = make_tmap_y(&ay.tm, V0, nx, ny, p->nhp, p->field_elems, 1, p->tc_y);
+    CUtensorMap tm[2];
+    e = source_maps_y(p, tm, V0, 1, p->tc_y);
+    ay.tm = tm[0];
+    ay.tm_full = tm[1];
     ay.src[0] = V0;
     ay.src[1] = V0;
     ay.src[2] = V0;
@@ -1142,7 +1234,9 @@ pin_status pin_displacements_2lpt(pin_plan_t p, float* psi2, int on_device) {
     ay.wait_cycles = p->wait_cycles;
     if (e == cudaSuccess) e = launch_y(ny, p->tc_y, p->vy, ay, p->stream);
     ArgsX ax{};
-    if (e == cudaSuccess) e = make_tmap_x(&ax.tm, spec(p, p->V, 1), nx, ny, p->nhp, 1, p->tc_x);
+    if (e == cudaSuccess) e = source_maps_x(p, tm, spec(p, p->V, 1), 1, p->tc_x);
+    ax.tm = tm[0];
+    ax.tm_full = tm[1];
     ax.src = spec(p, p->V, 1);
     ax.dst[0] = spec(p, p->V, 2);
     ax.nout = 1;
@@ -1398,7 +1492,9 @@ pin_status pin_set_radii(pin_plan_t p, int nscales, const double* radii) {
     }
   }
   const std::vector<float> mult = mult_table(p);
+  const std::vector<int> band = band_table(p, mult);
   PIN_CK(p, cudaMemcpy(p->mult, mult.data(), (size_t)nscales * p->mult_set() * sizeof(float), cudaMemcpyHostToDevice));
+  PIN_CK(p, cudaMemcpy(p->band, band.data(), 4 * (size_t)nscales * sizeof(int), cudaMemcpyHostToDevice));
   return PIN_OK;
 }
 
