@@ -31,56 +31,73 @@ __device__ __forceinline__ double bbks(double q) {
   return lead * pow(p, -0.25);
 }
 
-__device__ __forceinline__ void mode_value(int n, double box, uint64_t key, double amp, double ns, double gamma,
-                                           int ix, int iy, int iz, double* re, double* im) {
-  const int nh = n / 2 + 1;
-  const double sx = ix < n / 2 ? ix : ix - n, sy = iy < n / 2 ? iy : iy - n;
-  const double sz = iz < n / 2 ? iz : -(n / 2);
-  const double kk = 2.0 * M_PI / box * sqrt(sx * sx + sy * sy + sz * sz);
-  double P = 0.0;
-  if (kk > 0.0) {
-    const double t = bbks(kk / gamma);
-    P = amp * pow(kk, ns) * t * t;
+// sqrt(n^6 P(k) / box^3) of the modes with sx^2 + sy^2 + sz^2 = s2, for every
+// s2 up to 3 (n/2)^2 (0 at k = 0).  The spectrum takes five pow and a log per
+// evaluation, and a grid has a few hundred modes to every s2.
+__global__ void k_ic_scale(int n, double box, double amp, double ns, double gamma, int count, double* tab) {
+  for (int s2 = blockIdx.x * blockDim.x + threadIdx.x; s2 < count; s2 += gridDim.x * blockDim.x) {
+    const double kk = 2.0 * M_PI / box * sqrt((double)s2);
+    double P = 0.0;
+    if (kk > 0.0) {
+      const double t = bbks(kk / gamma);
+      P = amp * pow(kk, ns) * t * t;
+    }
+    tab[s2] = sqrt((double)n * n * n * (double)n * n * n * P / (box * box * box));
   }
-  const double scale = sqrt((double)n * n * n * (double)n * n * n * P / (box * box * box));
+}
+
+// x / sqrt(2), correctly rounded: the quotient by the rounded reciprocal,
+// corrected by its exact remainder (Markstein's division; the values here are
+// far from the ends of the range).
+__device__ __forceinline__ double over_sqrt2(double x) {
+  constexpr double d = 1.4142135623730951, inv = 0.70710678118654746;  // RN(sqrt 2), RN(1 / d)
+  const double q = x * inv;
+  return fma(fma(-q, d, x), inv, q);
+}
+
+__device__ __forceinline__ void mode_value(int n, uint64_t key, const double* __restrict__ tab, int ix, int iy, int iz,
+                                           double* re, double* im) {
+  const int nh = n / 2 + 1;
+  const int sx = ix < n / 2 ? ix : ix - n, sy = iy < n / 2 ? iy : iy - n;
+  const double scale = __ldg(tab + sx * sx + sy * sy + iz * iz);
   const uint64_t m = ((uint64_t)ix * n + iy) * nh + iz;
   const uint64_t r1 = splitmix64(key + (2 * m + 1) * kGolden);
   const uint64_t r2 = splitmix64(key + (2 * m + 2) * kGolden);
   const double u1 = ((double)((r1 >> 11) + 1)) * 0x1.0p-53;  // (0, 1]
   const double u2 = ((double)(r2 >> 11)) * 0x1.0p-53;        // [0, 1)
   const double rad = sqrt(-2.0 * log(u1));
-  *re = scale * (rad * cos(2.0 * M_PI * u2)) / sqrt(2.0);
-  *im = scale * (rad * sin(2.0 * M_PI * u2)) / sqrt(2.0);
+  double sn, cs;
+  sincos(2.0 * M_PI * u2, &sn, &cs);
+  *re = over_sqrt2(scale * (rad * cs));
+  *im = over_sqrt2(scale * (rad * sn));
 }
 
 // One realisation per blockIdx.y; out holds batch half-spectra [n][n][n/2+1].
-__global__ void k_ic_seed(int n, double box, const uint64_t* keys, double amp, double ns, double gamma,
-                          float2* out) {
-  const int nh = n / 2 + 1;
-  const size_t total = (size_t)n * n * nh;
+// Bound by the FP64 pipe (a log, a square root and a sine-cosine pair per
+// mode, two lanes per SM and clock): 512^3 75 -> 9.9 ms with the table of
+// scales and the two-step division.
+__global__ void k_ic_seed(int n, const uint64_t* keys, const double* __restrict__ tab, float2* out) {
+  const unsigned nh = n / 2 + 1, un = n;
+  const unsigned total = un * un * nh;  // < 2^31: checked at plan creation
   const uint64_t key = keys[blockIdx.y];
   float2* o = out + (size_t)blockIdx.y * total;
-  for (size_t m = blockIdx.x * (size_t)blockDim.x + threadIdx.x; m < total; m += (size_t)gridDim.x * blockDim.x) {
-    const int iz = (int)(m % nh);
-    const size_t r = m / nh;
-    const int iy = (int)(r % n), ix = (int)(r / n);
+  for (unsigned m = blockIdx.x * blockDim.x + threadIdx.x; m < total; m += gridDim.x * blockDim.x) {
+    const unsigned r = m / nh;
+    const int iz = (int)(m - r * nh);
+    const int ix = (int)(r / un), iy = (int)(r % un);
     double re = 0.0, im = 0.0;
-    if (!(ix == 0 && iy == 0 && iz == 0)) {
-      if (iz == 0 || iz == n / 2) {
-        const int jx = (n - ix) % n, jy = (n - iy) % n;
-        const size_t mm = ((size_t)jx * n + jy) * nh + iz;
-        if (mm == m) {
-          mode_value(n, box, key, amp, ns, gamma, ix, iy, iz, &re, &im);
-          re *= sqrt(2.0);
-          im = 0.0;
-        } else if (mm < m) {
-          mode_value(n, box, key, amp, ns, gamma, jx, jy, iz, &re, &im);
-          im = -im;
-        } else {
-          mode_value(n, box, key, amp, ns, gamma, ix, iy, iz, &re, &im);
-        }
-      } else {
-        mode_value(n, box, key, amp, ns, gamma, ix, iy, iz, &re, &im);
+    if (m != 0) {
+      // the kz = 0 and kz = n/2 planes: the mirror with the lower index is
+      // generated, the other one its conjugate
+      const bool plane = iz == 0 || iz == n / 2;
+      const int jx = (n - ix) % n, jy = (n - iy) % n;
+      const unsigned mm = ((unsigned)jx * un + jy) * nh + iz;
+      const bool mirror = plane && mm < m;
+      mode_value(n, key, tab, mirror ? jx : ix, mirror ? jy : iy, iz, &re, &im);
+      if (mirror) im = -im;
+      if (plane && mm == m) {
+        re *= sqrt(2.0);
+        im = 0.0;
       }
     }
     o[m] = make_float2((float)re, (float)im);
@@ -89,15 +106,21 @@ __global__ void k_ic_seed(int n, double box, const uint64_t* keys, double amp, d
 
 }  // namespace
 
-cudaError_t generate_ic(int n, double box, const uint64_t* keys_dev, int batch, double amp, double ns,
+size_t ic_table_count(int n) { return (size_t)3 * (n / 2) * (n / 2) + 1; }
+
+cudaError_t generate_ic(int n, double box, const uint64_t* keys_dev, double* table, int batch, double amp, double ns,
                         double gamma, float2* out, cudaStream_t st) {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int count = (int)ic_table_count(n);
+  k_ic_scale<<<(unsigned)((count + 127) / 128), 128, 0, st>>>(n, box, amp, ns, gamma, count, table);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
   const size_t total = (size_t)n * n * (n / 2 + 1);
   const size_t want = (total + 255) / 256;
   const unsigned gx = (unsigned)(want < (size_t)sms * 16 ? want : (size_t)sms * 16);
-  k_ic_seed<<<dim3(gx, (unsigned)batch), 256, 0, st>>>(n, box, keys_dev, amp, ns, gamma, out);
+  k_ic_seed<<<dim3(gx, (unsigned)batch), 256, 0, st>>>(n, keys_dev, table, out);
   return cudaGetLastError();
 }
 

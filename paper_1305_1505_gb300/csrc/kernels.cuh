@@ -240,8 +240,10 @@ cudaError_t fp64_cast(const double* in, size_t n3, float* out, cudaStream_t st);
 
 // Seeded initial conditions on the device (ic_gpu.cu): batch cubic
 // half-spectra [n][n][n/2+1] complex64 into out, realisation b keyed by
-// keys_dev[b] (the splitmix64 of its seed), amplitude amp of P(k).
-cudaError_t generate_ic(int n, double box, const uint64_t* keys_dev, int batch, double amp, double ns,
+// keys_dev[b] (the splitmix64 of its seed), amplitude amp of P(k); table is
+// scratch for ic_table_count(n) doubles.
+size_t ic_table_count(int n);
+cudaError_t generate_ic(int n, double box, const uint64_t* keys_dev, double* table, int batch, double amp, double ns,
                         double gamma, float2* out, cudaStream_t st);
 
 // Fragmentation front end (fragment.cu): the particles of one nx*ny*nz grid in
