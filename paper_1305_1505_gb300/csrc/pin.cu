@@ -197,39 +197,58 @@ void fill_twiddles(float2* t, int n, const PassShape& sh) {
 // Phi0(k) = delta(k) / k^2 into the padded layout (pad modes and k = 0
 // zero).  Cubic cells: the side along x is `box`, L_y = box ny / nx,
 // L_z = box nz / nx.
-__global__ void k_load_phi0(const void* src, int dtype, int nx, int ny, int nz, int nhp, double box, int batch,
+// 1/k^2 is an FP64 reciprocal (whose pipe has two lanes per SM and clock) and
+// depends on the signs of no index, so a block takes the up to four rows
+// (+-sx, +-sy) of one pair of indices, and every realisation's, with one
+// reciprocal per kz: 768^3 6.9 -> 2.1 ms, 64 x 128^3 2.3 -> 0.35 ms against one
+// per mode.
+template <typename In>
+__global__ void k_load_phi0(const In* __restrict__ src, int nx, int ny, int nz, int nhp, double box, int batch,
                             float limit, float2* phi0, int* wide) {
-  const int nh = nz / 2 + 1;
-  const size_t total = (size_t)nx * ny * nhp * batch;
+  const int nh = nz / 2 + 1, hy = ny / 2 + 1;
   const double kfx = 2.0 * M_PI / box, kfy = 2.0 * M_PI / (ny == nx ? box : box * ny / nx),
                kfz = 2.0 * M_PI / (nz == nx ? box : box * nz / nx);
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total;
-       i += (size_t)gridDim.x * blockDim.x) {
-    const int iz = (int)(i % nhp);
-    const size_t r = i / nhp;
-    const int iy = (int)(r % ny), ix = (int)((r / ny) % nx);  // r runs over realisations too
-    float2 out = make_float2(0.f, 0.f);
-    if (iz < nh) {
-      const size_t j = r * nh + iz;
-      float2 d;
-      if (dtype == PIN_C64) {
-        d = reinterpret_cast<const float2*>(src)[j];
-      } else {
-        const double2 dd = reinterpret_cast<const double2*>(src)[j];
-        d = make_float2((float)dd.x, (float)dd.y);
+  bool big = false;
+  for (int pair = blockIdx.x; pair < (nx / 2 + 1) * hy; pair += gridDim.x) {
+    const int ax = pair / hy, ay = pair - ax * hy;  // |sx|, |sy|
+    const double kx = kfx * ax, ky = kfy * ay;
+    const double kxy2 = __fma_rn(kx, kx, __dmul_rn(ky, ky));
+    int row[4];  // rows ix ny + iy with these |sx|, |sy|; repeated where a sign has no twin
+    const int mx = ax == 0 || 2 * ax == nx ? ax : nx - ax, my = ay == 0 || 2 * ay == ny ? ay : ny - ay;
+    row[0] = ax * ny + ay;
+    row[1] = ax * ny + my;
+    row[2] = mx * ny + ay;
+    row[3] = mx * ny + my;
+    const int nr = mx == ax ? (my == ay ? 1 : 2) : 4, step = (mx != ax && my == ay) ? 2 : 1;
+    for (int iz = threadIdx.x; iz < nhp; iz += blockDim.x) {
+      float inv = 0.f;
+      if (iz < nh) {
+        const double kz = kfz * iz;
+        const double k2 = __fma_rn(kz, kz, kxy2);
+        if (k2 > 0.0) inv = (float)__drcp_rn(k2);
       }
-      const double sx = ix < nx / 2 ? ix : ix - nx, sy = iy < ny / 2 ? iy : iy - ny;
-      const double sz = iz < nz / 2 ? iz : -(nz / 2);
-      const double kx = kfx * sx, ky = kfy * sy, kz = kfz * sz;
-      const double k2 = kx * kx + ky * ky + kz * kz;
-      if (k2 > 0.0) {
-        const float inv = (float)(1.0 / k2);
-        out = make_float2(d.x * inv, d.y * inv);
+      for (int b = 0; b < batch; ++b) {
+        float2 d[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          d[q] = make_float2(0.f, 0.f);
+          if (iz < nh && q < nr && q % step == 0) {
+            const In v = src[((size_t)b * nx * ny + row[q]) * nh + iz];
+            d[q] = make_float2((float)v.x, (float)v.y);
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (q >= nr || q % step != 0) continue;
+          float2 out = make_float2(0.f, 0.f);
+          if (inv > 0.f) out = make_float2(d[q].x * inv, d[q].y * inv);
+          phi0[((size_t)b * nx * ny + row[q]) * nhp + iz] = out;
+          big |= !(fabsf(out.x) < limit && fabsf(out.y) < limit);
+        }
       }
     }
-    phi0[i] = out;
-    if (!(fabsf(out.x) < limit && fabsf(out.y) < limit)) *wide = 1;
   }
+  if (big) *wide = 1;
 }
 
 // Plain copy by a kernel (16-byte words when both ends and the size allow,
@@ -266,11 +285,15 @@ cudaError_t copy_to_host(void* host_dst, const void* dev_src, size_t bytes, cuda
 
 cudaError_t launch_load_phi0(const void* src, int dtype, int nx, int ny, int nz, int nhp, double box, int batch,
                              float2* phi0, int* wide, cudaStream_t st) {
-  const size_t total = (size_t)nx * ny * nhp * batch;
-  const int threads = 256;
-  const unsigned blocks = (unsigned)std::min<size_t>((total + threads - 1) / threads, 152 * 64);
-  k_load_phi0<<<blocks, threads, 0, st>>>(src, dtype, nx, ny, nz, nhp, box, batch, wide_limit(nx, ny, nz, box), phi0,
-                                           wide);
+  const int threads = std::min(256, (nhp + 31) / 32 * 32);
+  const unsigned blocks = (unsigned)std::min((nx / 2 + 1) * (ny / 2 + 1), 152 * 64);
+  const float limit = wide_limit(nx, ny, nz, box);
+  if (dtype == PIN_C64)
+    k_load_phi0<<<blocks, threads, 0, st>>>(static_cast<const float2*>(src), nx, ny, nz, nhp, box, batch, limit, phi0,
+                                            wide);
+  else
+    k_load_phi0<<<blocks, threads, 0, st>>>(static_cast<const double2*>(src), nx, ny, nz, nhp, box, batch, limit, phi0,
+                                            wide);
   return cudaGetLastError();
 }
 
