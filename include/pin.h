@@ -201,14 +201,17 @@ pin_status pin_sync(pin_plan_t p, int64_t timeout_ns);
 pin_status pin_get_stats(pin_plan_t p, pin_stats* out);
 
 /* Number of kernels one pin_collapse_times call launches (for accounting):
- * per radius the x, y and z passes and the FP64 redo. */
+ * per radius the x, y and z passes and the FP64 redo; on small grids (lines of
+ * at most 128 points, no velocities, spectra of two or more radii within 320
+ * MB) a launch covers a group of radii, and one more kernel unpacks the
+ * running maximum at the end. */
 int pin_kernels_per_call(pin_plan_t p);
 
 /* Measurement hooks.  pin_profile(p, 1) makes later pin_collapse_times calls
  * record CUDA events around each pass of each radius (on the plan's stream,
  * inside its graph); pin_pass_times() then waits for the plan's work and
  * returns, for the last completed call, the device time in milliseconds summed
- * over radii of: ms4[0] the x pass (filter + transform), ms4[1] the y pass,
+ * over radii (or groups of radii) of: ms4[0] the x pass (filter + transform), ms4[1] the y pass,
  * ms4[2] the z pass (c2r, eigenvalues, collapse time and running max), ms4[3]
  * the FP64 redo of the queued ill-conditioned particles.  Each is measured on the stream its pass runs on; under an
  * overlapped schedule (pin_set_schedule) the passes overlap, so the four sums

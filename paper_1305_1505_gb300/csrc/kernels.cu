@@ -47,9 +47,16 @@ template <int N> __host__ __device__ constexpr int field_stride() {
 // (z and roots together), this kernel 12.0 and 11.3; it is bound by
 // instruction issue.  The two-level sizes use the fma-contracted eigenvalue
 // form, which keeps their results to the last bit.
+// Running maximum of a particle in a radius group (ArgsZ::state).
+__device__ __forceinline__ unsigned long long pack_state(float F, int scale) {
+  return (unsigned long long)__float_as_uint(F) << 32 | (unsigned)~scale;
+}
+__device__ __forceinline__ float state_f(unsigned long long s) { return __uint_as_float((unsigned)(s >> 32)); }
+
 enum ZMode { kZCollapse, kZDump, kZSource };
 
-template <int N, int LINES, int NP, ZMode MODE>
+// GROUP: the launch covers a group of radii (ArgsZ::state), blockIdx.y the radius.
+template <int N, int LINES, int NP, ZMode MODE, bool GROUP = false>
 __global__ void __launch_bounds__(NP * LINES * Shape<N>::P, MODE != kZCollapse ? MinBlocks<N>::zt
                                                             : NP == 5          ? MinBlocks<N>::zv
                                                                                : MinBlocks<N>::z)
@@ -77,6 +84,11 @@ __global__ void __launch_bounds__(NP * LINES * Shape<N>::P, MODE != kZCollapse ?
     }
   }
 
+  const int gr = GROUP ? blockIdx.y : 0;
+  const size_t goff = GROUP ? gr * a.gstride : 0;
+  const int scale = GROUP ? a.ms[gr] : a.scale;
+  RedoEntry* redo_list = GROUP ? a.redo_list + (size_t)gr * a.redo_cap : a.redo_list;
+  unsigned* redo_count = GROUP ? a.redo_count + gr : a.redo_count;
   const int npairs = (a.nfields + 1) / 2;
   const int c = tid / P, p = tid % P;
   const int ln = c / NP, pair = c % NP;
@@ -89,8 +101,8 @@ __global__ void __launch_bounds__(NP * LINES * Shape<N>::P, MODE != kZCollapse ?
 
   float2 v[E];
   {
-    const float2* A = active ? a.src[fa] + (size_t)line * nhp : nullptr;
-    const float2* B = hasb ? a.src[fb] + (size_t)line * nhp : nullptr;
+    const float2* A = active ? a.src[fa] + goff + (size_t)line * nhp : nullptr;
+    const float2* B = hasb ? a.src[fb] + goff + (size_t)line * nhp : nullptr;
 #pragma unroll
     for (int t = 0; t < E; ++t) {
       const int n = p + P * t;
@@ -188,7 +200,7 @@ __global__ void __launch_bounds__(NP * LINES * Shape<N>::P, MODE != kZCollapse ?
           const float F = cs.best + cs.corr;
           if (cs.kappa < a.tau_root) {
             atomicAdd(a.counters + 1, 1ull);
-            const unsigned slot = atomicAdd(a.redo_count, 1u);
+            const unsigned slot = atomicAdd(redo_count, 1u);
             if (slot < a.redo_cap) {
               RedoEntry e;
               e.q = qq;
@@ -196,7 +208,7 @@ __global__ void __launch_bounds__(NP * LINES * Shape<N>::P, MODE != kZCollapse ?
               for (int k = 0; k < 3; ++k) e.h[k] = u ? lm[k].y : lm[k].x;
               e.h[3] = e.h[4] = e.h[5] = 0.f;
               e.kind = 1;
-              a.redo_list[slot] = e;
+              redo_list[slot] = e;
               if constexpr (NP == 5) {
 #pragma unroll
                 for (int cpt = 0; cpt < 3; ++cpt) a.psi_out[cpt * total + qq] = s_f[lzv[u] + (6 + cpt) * kFS];
@@ -205,9 +217,11 @@ __global__ void __launch_bounds__(NP * LINES * Shape<N>::P, MODE != kZCollapse ?
             }
             atomicAdd(a.counters + 2, 1ull);  // queue full: keep the FP32 value
           }
-          if (F > fmv[u] || (F == fmv[u] && F > 0.f && a.scale < a.idx[qq])) {
+          if constexpr (GROUP) {
+            if (F > 0.f && F >= fmv[u]) atomicMax(a.state + qq, pack_state(F, scale));
+          } else if (F > fmv[u] || (F == fmv[u] && F > 0.f && scale < a.idx[qq])) {
             a.fmax[qq] = F;
-            a.idx[qq] = a.scale;
+            a.idx[qq] = scale;
             if constexpr (NP == 5) {
 #pragma unroll
               for (int cpt = 0; cpt < 3; ++cpt) a.vstate[cpt * total + qq] = s_f[lzv[u] + (6 + cpt) * kFS];
@@ -238,7 +252,7 @@ __global__ void __launch_bounds__(NP * LINES * Shape<N>::P, MODE != kZCollapse ?
         const float2 rabs = eig3_x2<(Shape<N>::P2 == 1)>(h, lam);
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-          fm[u] = valid[u] ? a.fmax[q[u]] : 0.f;
+          fm[u] = !valid[u] ? 0.f : GROUP ? state_f(a.state[q[u]]) : a.fmax[q[u]];
           if (valid[u] && (u ? rabs.y : rabs.x) > 1.f - a.tau_eig) {
             // a near-degenerate pair: the FP32 eigenvalues are not trusted,
             // but the invariant bound (no eigenvalues) may already show that
@@ -252,14 +266,14 @@ __global__ void __launch_bounds__(NP * LINES * Shape<N>::P, MODE != kZCollapse ?
               continue;
             }
             atomicAdd(a.counters + 0, 1ull);
-            const unsigned slot = atomicAdd(a.redo_count, 1u);
+            const unsigned slot = atomicAdd(redo_count, 1u);
             if (slot < a.redo_cap) {
               RedoEntry e;
               e.q = q[u];
 #pragma unroll
               for (int f = 0; f < 6; ++f) e.h[f] = u ? h[f].y : h[f].x;
               e.kind = 0;
-              a.redo_list[slot] = e;
+              redo_list[slot] = e;
               if constexpr (NP == 5) {
 #pragma unroll
                 for (int cpt = 0; cpt < 3; ++cpt) a.psi_out[cpt * total + q[u]] = s_f[lz[u] + (6 + cpt) * kFS];
@@ -410,20 +424,28 @@ __global__ void k_phi2(const float2* __restrict__ T, float2* out, int nx, int ny
 }
 
 // FP64 redo of the queued particles of one radius (grid-stride; each particle
-// appears once per radius, so the in-place update has no race).
+// appears once per radius, so the in-place update has no race) or of a group
+// of radii (a particle may appear once per radius: atomic maxima).
 __global__ void __launch_bounds__(128) k_redo64(ArgsZ a) {
-  const unsigned cnt = *a.redo_count;
-  const unsigned n = cnt < a.redo_cap ? cnt : a.redo_cap;
   CollapseConsts<double> ccd{a.dcorr_d, a.correction};
-  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const RedoEntry e = a.redo_list[i];
+  // the queues of a group's radii one after the other
+  const bool group = a.state != nullptr;
+  unsigned before = 0, n = 0;
+  int g = -1;
+  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x;; i += gridDim.x * blockDim.x) {
+    while (i >= before + n) {
+      before += n;
+      if (++g >= (group ? a.nrad : 1)) return;
+      n = min(a.redo_count[g], a.redo_cap);
+    }
+    const RedoEntry e = a.redo_list[(size_t)g * a.redo_cap + (i - before)];
     double h[6], lam[3], kap;
 #pragma unroll
     for (int f = 0; f < 6; ++f) h[f] = (double)e.h[f];
     // the invariant bound (the six components, or diag(lambda) for kind 1)
     // first: below F_max by more than the FP32 rounding of F, the particle
     // cannot be updated, and the FP64 eigenvalues and roots are skipped
-    const float fm0 = a.fmax[e.q];
+    const float fm0 = group ? state_f(a.state[e.q]) : a.fmax[e.q];
     if ((double)fm0 * (1.0 - 1e-6) > collapse_bound<double>(h, ccd)) continue;
     if (e.kind == 0) {
       eig3<double>(h, lam);
@@ -433,6 +455,10 @@ __global__ void __launch_bounds__(128) k_redo64(ArgsZ a) {
       lam[2] = h[2];
     }
     const float F = (float)collapse_from_eigs<double>(lam, ccd, kap);
+    if (group) {
+      if (F > 0.f) atomicMax(a.state + e.q, pack_state(F, a.ms[g]));
+      continue;
+    }
     const float fm = a.fmax[e.q];
     if (F > fm || (F == fm && F > 0.f && a.scale < a.idx[e.q])) {
       a.fmax[e.q] = F;
@@ -444,6 +470,19 @@ __global__ void __launch_bounds__(128) k_redo64(ArgsZ a) {
       }
     }
   }
+}
+
+__global__ void k_unpack(const unsigned long long* __restrict__ state, size_t n, float* fmax, int* idx) {
+  for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < n; q += (size_t)gridDim.x * blockDim.x) {
+    const unsigned long long s = state[q];
+    fmax[q] = state_f(s);
+    idx[q] = s ? (int)~(unsigned)s : -1;
+  }
+}
+
+cudaError_t launch_unpack(const unsigned long long* state, size_t n, float* fmax, int* idx, cudaStream_t st) {
+  k_unpack<<<(unsigned)std::min<size_t>((n + 255) / 256, 152 * 16), 256, 0, st>>>(state, n, fmax, idx);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_redo(const ArgsZ& a, cudaStream_t st) {
@@ -497,6 +536,11 @@ static cudaError_t set_attrs() {
   e = cudaFuncSetAttribute(k_pass_z<N, C::LINES, 3, kZCollapse>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)C::smem_z);
   if (e != cudaSuccess) return e;
+  if constexpr (kMultiRad<N>) {
+    e = cudaFuncSetAttribute(k_pass_z<N, C::LINES, 3, kZCollapse, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)C::smem_z);
+    if (e != cudaSuccess) return e;
+  }
   e = cudaFuncSetAttribute(k_pass_z<N, C::LINES_V, 5, kZCollapse>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)C::smem_zv);
   if (e != cudaSuccess) return e;
@@ -542,6 +586,15 @@ static cudaError_t run_z(const ArgsZ& a_in, bool dump, cudaStream_t st) {
     return cudaGetLastError();
   }
   const unsigned grid = (unsigned)((nlines + C::LINES - 1) / C::LINES);
+  if (a.state) {
+    if constexpr (kMultiRad<N>) {
+      a.prefetch_blocks = 0;  // the group's spectra are in L2
+      k_pass_z<N, C::LINES, 3, kZCollapse, true><<<dim3(grid, a.nrad), C::threads_z, C::smem_z, st>>>(a);
+      return cudaGetLastError();
+    } else {
+      return cudaErrorInvalidValue;
+    }
+  }
   if (dump) k_pass_z<N, C::LINES, 3, kZDump><<<grid, C::threads_z, C::smem_z, st>>>(a);
   else k_pass_z<N, C::LINES, 3, kZCollapse><<<grid, C::threads_z, C::smem_z, st>>>(a);
   return cudaGetLastError();
@@ -736,12 +789,12 @@ cudaError_t make_tmap_rows(CUtensorMap* tm, const float2* base, int cols, long l
   return encode(tm, 2, base, dims, strides, box);
 }
 
-cudaError_t make_tmap_y(CUtensorMap* tm, const float2* src3, int nx, int ny, int nhp, size_t spec_elems,
+cudaError_t make_tmap_y(CUtensorMap* tm, const float2* src, int nx, int ny, int nhp, size_t spec_elems, int nspec,
                         int batch, int tc, int boxes) {
-  const cuuint64_t dims[4] = {(cuuint64_t)nhp, (cuuint64_t)ny, (cuuint64_t)nx * batch, 3};
+  const cuuint64_t dims[4] = {(cuuint64_t)nhp, (cuuint64_t)ny, (cuuint64_t)nx * batch, (cuuint64_t)nspec};
   const cuuint64_t strides[3] = {(cuuint64_t)nhp * 8, (cuuint64_t)ny * nhp * 8, (cuuint64_t)spec_elems * 8};
   const cuuint32_t box[4] = {(cuuint32_t)tc, (cuuint32_t)(ny / boxes), 1, 1};
-  return encode(tm, 4, src3, dims, strides, box);
+  return encode(tm, 4, src, dims, strides, box);
 }
 
 cudaError_t upload_constant_twiddles() {

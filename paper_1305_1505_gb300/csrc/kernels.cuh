@@ -30,16 +30,27 @@ constexpr int kMaxFields = 9;
 // the y pass 2.35 instead of 3.35).  The z pass reads whole lines: a test per
 // mode costs its issue slots more (3 %) than the loads it saves.  So the
 // columns past a radius's z band have to hold zeros in V; the y pass writes
-// them where the radius before it in the same buffer (prev) had modes, all
-// others are zero already, the radii running from small to large.
+// them where the radius before it in the same buffer (RadGroup::prev) had
+// modes, all others are zero already, the radii running from small to large.
 // Nothing but exact zeros is left out, so the results are those of the full
 // passes: a field with a value that is not finite, or so large that an
 // intermediate could overflow (then 0 x inf would make a NaN of a zero), sets
 // *wide, and the passes run full.
-struct BandArgs {
-  const int* band;  // {x, y, z, 0} of this radius; null: full
-  const int* wide;  // non-zero: full
-  const int* prev;  // y pass: the band of the radius before, null: full
+//
+// Radius groups.  A small grid's pass over one radius is a few microseconds of
+// work on a part of the SMs, so its launches cover several radii at once: U
+// and V hold n sets of spectra back to back, the x and y passes walk the tiles
+// of all of them, the z pass has a grid row per radius and keeps its running
+// maximum in one 64-bit word per particle.  Lines of at most kGroupMaxN points.
+constexpr int kMaxGroup = 16;
+constexpr int kGroupMaxN = 128;
+struct RadGroup {
+  int n;                // radii of this launch (1 where a line has more than kGroupMaxN points)
+  int ms[kMaxGroup];    // their multiplier sets
+  int prev[kMaxGroup];  // y pass: the set whose spectra the V buffer held before; -1: anything
+  int mult_set;         // floats from one set's multipliers to the next
+  const int* band;      // {x, y, z, 0} of set 0, sets back to back; null: full
+  const int* wide;      // non-zero: full
 };
 // Band of one radius from the axis factors ([3][n] each).  The z entry of a
 // full axis is nhp - 1, so that it covers the pad columns.
@@ -60,11 +71,11 @@ struct ArgsX {
   int xm[3];
   int nout;
   int ny;             // rows of a plane: the columns are (ky, kz), ny * nhp of them
-  const float* mult;  // [3][nx] multipliers of this radius (W, kW, k^2W, each / nx)
+  const float* mult;  // [3][nx] multipliers of set 0 (W, kW, k^2W, each / nx)
   const float2* tw;   // twiddles: w_N^{p k1} [E][P], then w_P^{p1 k2a} [P2][P1] for three levels
   int nhp;
   int batch;          // realisations stacked back to back (same N, radii)
-  BandArgs band;
+  RadGroup rad;       // radius g's outputs: dst[f] + g * 3 spectra (of all realisations)
   int col_unit;       // the y pass reads the band's columns in tiles of this many: all of them are stored
   int* err;           // set to 1 if a TMA wait gave up (bounded wait)
   long long wait_cycles;  // budget of a TMA wait in SM clocks; <= 0: the default (2^31)
@@ -76,7 +87,7 @@ struct ArgsX {
 // constant along a y line.  Outputs are processed in the given order;
 // consecutive outputs with the same source share one staged tile.  tm is a 4D
 // map over the three source spectra (stored back to back),
-// {nhp, ny, batch*nx, 3}, box {tc, ny/boxes, 1, 1}.
+// {nhp, ny, batch*nx, 3 per radius}, box {tc, ny/boxes, 1, 1}.
 struct ArgsY {
   CUtensorMap tm;       // in stage_boxes, for partial bands
   CUtensorMap tm_full;  // in store_boxes
@@ -92,12 +103,12 @@ struct ArgsY {
   int muli2[kMaxFields];
   int nout;
   int nx, nz;           // x planes per realisation; z line length (z factors for kz <= nz/2)
-  const float* mult;    // [3][ny] y multipliers
-  const float* mult_z;  // [3][nz] z multipliers
+  const float* mult;    // [3][ny] y multipliers of set 0
+  const float* mult_z;  // [3][nz] z multipliers of set 0
   const float2* tw;
   int nhp;
   int batch;
-  BandArgs band;
+  RadGroup rad;         // radius g: sources src + g * 3 spectra, outputs dst[o] + g * 6
   int* err;
   long long wait_cycles;
   CUtensorMap tm_out[kMaxFields];  // maps of dst[o] (filled at launch when outputs go out by TMA stores)
@@ -131,6 +142,14 @@ struct ArgsZ {
   float* fmax;
   int* idx;
   int scale;
+  // radius groups: state != null.  Radius g < nrad (index ms[g]) reads src[f]
+  // + g * gstride and queues into redo_list + g * redo_cap, redo_count[g];
+  // state[q] = bits of F << 32 | ~index, 0 before any F > 0: its maximum is
+  // the larger F and among equal ones the lower index.  fmax, idx, scale unused.
+  unsigned long long* state;
+  int nrad;
+  int ms[kMaxGroup];
+  size_t gstride;
   int correction;
   float dcorr_f;
   double dcorr_d;
@@ -163,7 +182,7 @@ struct PassShape {
 cudaError_t make_tmap_x(CUtensorMap* tm, const float2* src, int nx, int ny, int nhp, int batch, int tc, int boxes);
 // 2D map of rows of `cols` complex values (row pitch cols), box {tc, box_rows}
 cudaError_t make_tmap_rows(CUtensorMap* tm, const float2* base, int cols, long long rows, int tc, int box_rows);
-cudaError_t make_tmap_y(CUtensorMap* tm, const float2* src3, int nx, int ny, int nhp, size_t spec_elems,
+cudaError_t make_tmap_y(CUtensorMap* tm, const float2* src, int nx, int ny, int nhp, size_t spec_elems, int nspec,
                         int batch, int tc, int boxes);
 // Boxes of a staged tile of n rows with E register slots per thread: eighths
 // (quarters where E is no multiple of eight), whole slots each, so that a
@@ -208,6 +227,8 @@ cudaError_t launch_phi2(const float2* T, float2* out, int nx, int ny, int nz, in
 bool three_level(int n);
 // The FP64 redo of every particle the z pass queued (after it, same stream).
 cudaError_t launch_redo(const ArgsZ& a, cudaStream_t st);
+// state -> F_max and index of every particle (after the last group's redo)
+cudaError_t launch_unpack(const unsigned long long* state, size_t n, float* fmax, int* idx, cudaStream_t st);
 cudaError_t upload_constant_twiddles();  // per device
 
 // Host helpers shared by the plan path (pin.cu) and the allocation-free entry

@@ -37,29 +37,49 @@ namespace {
 
 constexpr int kMaxN = PIN_NOALLOC_MAX_N;
 constexpr int kMaxScales = 64;
-constexpr int kMaxNhp = (kMaxN / 2 + 1 + 3) & ~3;  // padded_half(kMaxN)
-constexpr size_t kSpecElems = (size_t)kMaxN * kMaxN * kMaxNhp;  // one padded half-spectrum
-constexpr size_t kSpecBytes = kSpecElems * sizeof(float2);
-constexpr size_t kMultFloats = (size_t)kMaxScales * 3 * kMaxN;
-constexpr size_t kMultBytes = kMultFloats * sizeof(float);
-constexpr size_t kTwBytes = (size_t)kMaxN * sizeof(float2);
-// FP64 redo queue: the plan path's capacity, max(65536, N^3 / 64), which is
-// 65536 entries for every N this entry point accepts
+// FP64 redo queue per radius: the plan path's capacity, max(65536, N^3 / 64),
+// which is 65536 entries for every N this entry point accepts
 constexpr size_t kRedoCap = 65536;
 static_assert((size_t)kMaxN * kMaxN * kMaxN / 64 <= kRedoCap, "redo capacity below the plan path's rule");
-constexpr size_t kOffPhi0 = 0;
-constexpr size_t kOffU = kOffPhi0 + kSpecBytes;
-constexpr size_t kOffV = kOffU + 3 * kSpecBytes;
-constexpr size_t kOffMult = kOffV + 6 * kSpecBytes;
-constexpr size_t kOffBand = kOffMult + kMultBytes;            // 4 ints per radius
-constexpr size_t kOffTw = kOffBand + kMaxScales * 4 * sizeof(int);
-constexpr size_t kOffCnt = kOffTw + kTwBytes;                 // 3 counters
-constexpr size_t kOffRedoCount = kOffCnt + 4 * sizeof(unsigned long long);
-constexpr size_t kOffErr = kOffRedoCount + 16;                // cleared with the counters
-constexpr size_t kOffWide = kOffErr + 8;                      // as is the word that turns the bands off
-constexpr size_t kStatusBytes = kOffErr + 16 - kOffCnt;      // counters .. error word
-constexpr size_t kOffRedo = (kOffErr + 16 + 255) & ~(size_t)255;
-constexpr size_t kScratchBytes = (kOffRedo + kRedoCap * sizeof(pin::RedoEntry) + 255) & ~(size_t)255;
+
+constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
+constexpr size_t spec_bytes(int n) { return (size_t)n * n * ((n / 2 + 1 + 3) & ~3) * sizeof(float2); }
+
+// Where things lie in the workspace for grids of n points a side and groups of
+// `group` radii (RadGroup): Phi0, U and V, the running maximum of a group, the
+// tables, {counters, queue counts, error word, the word that turns the bands
+// off} (cleared by every call), the redo queues.
+struct Layout {
+  int group;
+  size_t cap;  // redo entries per radius
+  size_t phi0, U, V, state, mult, band, tw, cnt, redo_count, err, wide, redo, end;
+  constexpr Layout(int n, int g)
+      : group(g), cap(), phi0(), U(), V(), state(), mult(), band(), tw(), cnt(), redo_count(), err(), wide(), redo(),
+        end() {
+    const size_t n3 = (size_t)n * n * n;
+    cap = g > 1 && n3 < kRedoCap ? n3 : kRedoCap;
+    U = spec_bytes(n);
+    V = U + 3 * spec_bytes(n) * g;
+    state = V + 6 * spec_bytes(n) * g;
+    mult = state + (g > 1 ? n3 * 8 : 0);
+    band = mult + (size_t)kMaxScales * 3 * n * sizeof(float);
+    tw = band + (size_t)kMaxScales * 4 * sizeof(int);
+    cnt = tw + (size_t)n * sizeof(float2);
+    redo_count = cnt + 4 * sizeof(unsigned long long);
+    err = redo_count + pin::kMaxGroup * sizeof(unsigned);
+    wide = err + 8;
+    redo = align256(err + 16);
+    end = align256(redo + cap * g * sizeof(pin::RedoEntry));
+  }
+};
+// One radius at a time at the largest grid: 13.9 MB; smaller grids use the
+// same space for groups of radii (48^3: one, 32^3: five, 16^3: sixteen).
+constexpr size_t kScratchBytes = Layout(kMaxN, 1).end;
+constexpr int group_of(int n) {
+  int g = 1;
+  while (g < pin::kMaxGroup && Layout(n, g + 1).end <= kScratchBytes) ++g;
+  return g;
+}
 
 // The whole device workspace of this entry point (13.9 MB for
 // N <= 64).  In host code this name is only a stand-in for the symbol, never
@@ -69,11 +89,13 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 constexpr int kMaxDevices = 64;
 std::mutex g_setup_mu;
 unsigned char* g_scratch_ptr[kMaxDevices] = {};
+size_t g_last_cnt[kMaxDevices] = {};  // counters and error word of the last call
+size_t g_last_err[kMaxDevices] = {};
 
 // Host staging of the tables (filled and copied under g_stage_mu; a copy from
 // pageable host memory has consumed its source when cudaMemcpyAsync returns).
 std::mutex g_stage_mu;
-float g_h_mult[kMultFloats];
+float g_h_mult[(size_t)kMaxScales * 3 * kMaxN];
 int g_h_band[kMaxScales * 4];
 float2 g_h_tw[kMaxN];
 
@@ -121,23 +143,30 @@ extern "C" pin_status pin_collapse_times_noalloc(const void* delta_k, int dtype,
   const pin::PassShape sh = pin::pass_shape(n);
   const int nhp = pin::padded_half(n);
   const size_t spec = (size_t)n * n * nhp;
-  float2* phi0 = reinterpret_cast<float2*>(base + kOffPhi0);
-  float2* U = reinterpret_cast<float2*>(base + kOffU);
-  float2* V = reinterpret_cast<float2*>(base + kOffV);
-  float* mult = reinterpret_cast<float*>(base + kOffMult);
-  float2* tw = reinterpret_cast<float2*>(base + kOffTw);
-  unsigned long long* cnt = reinterpret_cast<unsigned long long*>(base + kOffCnt);
-  unsigned* redo_count = reinterpret_cast<unsigned*>(base + kOffRedoCount);
-  int* err = reinterpret_cast<int*>(base + kOffErr);
-  int* band = reinterpret_cast<int*>(base + kOffBand);
-  int* wide = reinterpret_cast<int*>(base + kOffWide);
-  pin::RedoEntry* redo_list = reinterpret_cast<pin::RedoEntry*>(base + kOffRedo);
+  const Layout at(n, group_of(n));
+  {
+    std::lock_guard<std::mutex> lk(g_setup_mu);
+    g_last_cnt[dev] = at.cnt;
+    g_last_err[dev] = at.err;
+  }
+  float2* phi0 = reinterpret_cast<float2*>(base + at.phi0);
+  float2* U = reinterpret_cast<float2*>(base + at.U);
+  float2* V = reinterpret_cast<float2*>(base + at.V);
+  unsigned long long* state = at.group > 1 ? reinterpret_cast<unsigned long long*>(base + at.state) : nullptr;
+  float* mult = reinterpret_cast<float*>(base + at.mult);
+  float2* tw = reinterpret_cast<float2*>(base + at.tw);
+  unsigned long long* cnt = reinterpret_cast<unsigned long long*>(base + at.cnt);
+  unsigned* redo_count = reinterpret_cast<unsigned*>(base + at.redo_count);
+  int* err = reinterpret_cast<int*>(base + at.err);
+  int* band = reinterpret_cast<int*>(base + at.band);
+  int* wide = reinterpret_cast<int*>(base + at.wide);
+  pin::RedoEntry* redo_list = reinterpret_cast<pin::RedoEntry*>(base + at.redo);
   CUtensorMap tm_x[2], tm_y[2];  // staged and whole-line boxes
   const int tc = sh.tc;  // the default tile width, as a new plan runs
   for (int m = 0; m < 2; ++m) {
     const int boxes = m ? pin::store_boxes(n) : pin::stage_boxes(sh.E);
     if (pin::make_tmap_x(&tm_x[m], phi0, n, n, nhp, 1, tc, boxes) != cudaSuccess ||
-        pin::make_tmap_y(&tm_y[m], U, n, n, nhp, spec, 1, tc, boxes) != cudaSuccess)
+        pin::make_tmap_y(&tm_y[m], U, n, n, nhp, spec, 3 * at.group, 1, tc, boxes) != cudaSuccess)
       return PIN_ECUDA;
   }
   const double dcorr = pin::correction_dcorr();
@@ -158,10 +187,11 @@ extern "C" pin_status pin_collapse_times_noalloc(const void* delta_k, int dtype,
         cudaMemcpyAsync(tw, g_h_tw, (size_t)n * sizeof(float2), cudaMemcpyHostToDevice, cs) != cudaSuccess)
       return PIN_ECUDA;
   }
-  if (cudaMemsetAsync(cnt, 0, kStatusBytes, cs) != cudaSuccess ||
+  if (cudaMemsetAsync(cnt, 0, at.err + 16 - at.cnt, cs) != cudaSuccess ||
       pin::launch_load_phi0(delta_k, dtype, n, n, n, nhp, box, 1, phi0, wide, cs) != cudaSuccess ||
-      cudaMemsetAsync(F_max, 0, n3 * sizeof(float), cs) != cudaSuccess ||
-      cudaMemsetAsync(scale_idx, 0xFF, n3 * sizeof(int32_t), cs) != cudaSuccess)
+      (state ? cudaMemsetAsync(state, 0, n3 * sizeof(*state), cs) != cudaSuccess
+             : cudaMemsetAsync(F_max, 0, n3 * sizeof(float), cs) != cudaSuccess ||
+                   cudaMemsetAsync(scale_idx, 0xFF, n3 * sizeof(int32_t), cs) != cudaSuccess))
     return PIN_ECUDA;
 
   static const int vout[6] = {0, 3, 4, 1, 2, 5};
@@ -172,9 +202,17 @@ extern "C" pin_status pin_collapse_times_noalloc(const void* delta_k, int dtype,
   int order[kMaxScales];
   for (int s = 0; s < nscales; ++s) order[s] = s;
   std::stable_sort(order, order + nscales, [&](int a, int b) { return radii[a] < radii[b]; });
-  for (int k = 0; k < nscales; ++k) {
+  for (int k = 0; k < nscales; k += at.group) {
     const int s = order[k];
-    const float* m = mult + (size_t)s * 3 * n;
+    pin::RadGroup rad{};
+    rad.n = std::min(at.group, nscales - k);
+    rad.mult_set = 3 * n;
+    for (int g = 0; g < rad.n; ++g) {
+      rad.ms[g] = order[k + g];
+      rad.prev[g] = k + g >= at.group ? order[k + g - at.group] : -1;
+    }
+    rad.band = band;
+    rad.wide = wide;
     pin::ArgsX ax{};
     ax.tm = tm_x[0];
     ax.tm_full = tm_x[1];
@@ -182,10 +220,10 @@ extern "C" pin_status pin_collapse_times_noalloc(const void* delta_k, int dtype,
     for (int f = 0; f < 3; ++f) { ax.dst[f] = U + f * spec; ax.xm[f] = f; }
     ax.nout = 3;
     ax.ny = n;
-    ax.mult = m;
+    ax.mult = mult;
+    ax.rad = rad;
     ax.tw = tw;
     ax.nhp = nhp;
-    ax.band = pin::BandArgs{band + 4 * s, wide, nullptr};
     ax.col_unit = tc;
     ax.batch = 1;
     ax.err = err;
@@ -203,11 +241,11 @@ extern "C" pin_status pin_collapse_times_noalloc(const void* delta_k, int dtype,
     ay.nout = 6;
     ay.nx = n;
     ay.nz = n;
-    ay.mult = m;
-    ay.mult_z = m;
+    ay.mult = mult;
+    ay.mult_z = mult;
+    ay.rad = rad;
     ay.tw = tw;
     ay.nhp = nhp;
-    ay.band = pin::BandArgs{band + 4 * s, wide, k ? band + 4 * order[k - 1] : nullptr};
     ay.batch = 1;
     ay.err = err;
     pin::ArgsZ az{};
@@ -220,6 +258,12 @@ extern "C" pin_status pin_collapse_times_noalloc(const void* delta_k, int dtype,
     az.fmax = F_max;
     az.idx = scale_idx;
     az.scale = s;
+    if (state) {
+      az.state = state;
+      az.nrad = rad.n;
+      for (int g = 0; g < rad.n; ++g) az.ms[g] = rad.ms[g];
+      az.gstride = 6 * spec;
+    }
     az.correction = correction;
     az.dcorr_d = dcorr;
     az.dcorr_f = (float)dcorr;
@@ -228,13 +272,14 @@ extern "C" pin_status pin_collapse_times_noalloc(const void* delta_k, int dtype,
     az.counters = cnt;
     az.redo_list = redo_list;
     az.redo_count = redo_count;
-    az.redo_cap = (unsigned)kRedoCap;
+    az.redo_cap = (unsigned)at.cap;
     if (pin::launch_x(n, tc, 0, ax, cs) != cudaSuccess || pin::launch_y(n, tc, 0, ay, cs) != cudaSuccess ||
-        cudaMemsetAsync(redo_count, 0, sizeof(unsigned), cs) != cudaSuccess ||
+        cudaMemsetAsync(redo_count, 0, rad.n * sizeof(unsigned), cs) != cudaSuccess ||
         pin::launch_z(n, az, false, cs) != cudaSuccess ||
         pin::launch_redo(az, cs) != cudaSuccess)
       return PIN_ECUDA;
   }
+  if (state && pin::launch_unpack(state, n3, F_max, scale_idx, cs) != cudaSuccess) return PIN_ECUDA;
   return PIN_OK;
 }
 
@@ -243,15 +288,18 @@ extern "C" pin_status pin_noalloc_status(int* wait_failed, uint64_t* counters3) 
   const int dev = current_device();
   if (dev < 0) return PIN_ECUDA;
   unsigned char* base = nullptr;
+  size_t off_cnt = 0, off_err = 0;
   {
     std::lock_guard<std::mutex> lk(g_setup_mu);
     base = g_scratch_ptr[dev];
+    off_cnt = g_last_cnt[dev];
+    off_err = g_last_err[dev];
   }
-  if (!base) return PIN_ESTATE;  // no call has run on this device
+  if (!base || !off_cnt) return PIN_ESTATE;  // no call has run on this device
   unsigned long long c[3] = {0, 0, 0};
   int e = 0;
-  if (cudaMemcpy(c, base + kOffCnt, sizeof(c), cudaMemcpyDeviceToHost) != cudaSuccess ||
-      cudaMemcpy(&e, base + kOffErr, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
+  if (cudaMemcpy(c, base + off_cnt, sizeof(c), cudaMemcpyDeviceToHost) != cudaSuccess ||
+      cudaMemcpy(&e, base + off_err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
     return PIN_ECUDA;
   *wait_failed = e != 0;
   for (int i = 0; i < 3; ++i) counters3[i] = c[i];

@@ -197,6 +197,78 @@ __device__ __forceinline__ void load_slots(float2 (&v)[Shape<N, V>::E], const fl
   }
 }
 
+// Lines short enough for radius groups (RadGroup).
+template <int N> constexpr bool kMultiRad = N <= kGroupMaxN;
+
+// Walk over the x pass's tiles: radius by radius, realisation by realisation,
+// the columns of the filter's support: ky rows 0..by and ny-by..ny-1, columns
+// kz < ncz (the y pass's tiles are read whole).  A full plane is walked as one
+// run of columns; a partial one row by row, ktiles tiles to a row (the last
+// may run past the row's end: it then computes the first columns of the next
+// row as well, which come out the same from every tile that holds them).
+template <int N, int TC, int V>
+struct WalkX {
+  int g, base;     // radius of the launch, its first tile
+  int by, nrows, ktiles, tpr, ntiles;  // tiles of a realisation and of the radius; the last may run past the columns
+  bool flat;
+  BoxRange rows;   // kx boxes
+  __device__ __forceinline__ explicit WalkX(const ArgsX& a) : g(0), base(0) { init(a); }
+  __device__ __forceinline__ void init(const ArgsX& a) {
+    const int* b = a.rad.band ? a.rad.band + 4 * a.rad.ms[g] : nullptr;
+    const bool part = b != nullptr && __ldg(a.rad.wide) == 0;
+    by = part ? __ldg(b + 1) : a.ny / 2;
+    const int ncz = part ? min(a.nhp, (__ldg(b + 2) / a.col_unit + 1) * a.col_unit) : a.nhp;
+    rows = boxes_of<N, V>(part ? __ldg(b) : N / 2);
+    flat = 2 * by + 1 >= a.ny && ncz >= a.nhp;
+    nrows = min(a.ny, 2 * by + 1);
+    ktiles = (ncz + TC - 1) / TC;
+    tpr = flat ? (a.ny * a.nhp + TC - 1) / TC : nrows * ktiles;
+    ntiles = tpr * a.batch;
+  }
+  // to the radius of `tile` (not before the current one); false past the last
+  __device__ __forceinline__ bool seek(const ArgsX& a, int tile) {
+    if constexpr (!kMultiRad<N>) return tile < ntiles;
+    while (tile >= base + ntiles) {
+      if (g + 1 >= a.rad.n) return false;
+      base += ntiles;
+      ++g;
+      init(a);
+    }
+    return true;
+  }
+  __device__ __forceinline__ int col(const ArgsX& a, int t) const {  // first column of tile t of a realisation
+    if (flat) return t * TC;
+    const int row = t / ktiles;
+    return (row <= by ? row : a.ny - nrows + row) * a.nhp + (t - row * ktiles) * TC;
+  }
+};
+
+// The same for the y pass: radius by radius, plane by plane, columns kz <= bz.
+template <int N, int TC, int V>
+struct WalkY {
+  int g, base, by, ktiles, ntiles;
+  BoxRange rows;  // ky boxes
+  __device__ __forceinline__ explicit WalkY(const ArgsY& a) : g(0), base(0) { init(a); }
+  __device__ __forceinline__ void init(const ArgsY& a) {
+    const int* b = a.rad.band ? a.rad.band + 4 * a.rad.ms[g] : nullptr;
+    const bool part = b != nullptr && __ldg(a.rad.wide) == 0;
+    by = part ? __ldg(b + 1) : N / 2;
+    rows = boxes_of<N, V>(by);
+    ktiles = ((part ? __ldg(b + 2) + 1 : a.nhp) + TC - 1) / TC;
+    ntiles = a.nx * a.batch * ktiles;
+  }
+  __device__ __forceinline__ bool seek(const ArgsY& a, int tile) {
+    if constexpr (!kMultiRad<N>) return tile < ntiles;
+    while (tile >= base + ntiles) {
+      if (g + 1 >= a.rad.n) return false;
+      base += ntiles;
+      ++g;
+      init(a);
+    }
+    return true;
+  }
+};
+
 // ---------------------------------------------------------------- x pass --
 // Lines along x: column index col in [0, N*nhp) enumerates (ky, kz); element
 // (kx, col) sits at kx*N*nhp + col, so a row of TC columns is contiguous.  A
@@ -222,7 +294,8 @@ __global__ void __launch_bounds__(TC* Shape<N, V>::P, MinBlocks<N, TC, V>::xy)
   const int tid = threadIdx.x, c = tid % TC, p = tid / TC;
   const uint32_t bar = smem_u32(&s_bar);
   for (int i = tid; i < NTW; i += TC * P) s_tw[i] = a.tw[i];
-  for (int i = tid; i < 3 * N; i += TC * P) s_m[i] = a.mult[i];
+  int g_m = 0;  // radius whose multipliers s_m holds
+  for (int i = tid; i < 3 * N; i += TC * P) s_m[i] = a.mult[(size_t)a.rad.ms[0] * a.rad.mult_set + i];
   if (tid < 3) s_xm[tid] = a.xm[tid];
   if (tid == 0) {
     mbar_init(bar, 1);
@@ -230,28 +303,12 @@ __global__ void __launch_bounds__(TC* Shape<N, V>::P, MinBlocks<N, TC, V>::xy)
   }
   __syncthreads();
   const int ncols = a.ny * a.nhp;
-  // the filter's support (BandArgs): kx boxes, ky rows 0..by and ny-by..ny-1,
-  // columns kz < ncz.  A full plane is walked as one run of columns; a partial
-  // one row by row, ktiles tiles to a row (the last may run past the row's
-  // end: it then computes the first columns of the next row as well, which
-  // come out the same from every tile that holds them).
-  const bool part = a.band.band != nullptr && __ldg(a.band.wide) == 0;
-  const int by = part ? __ldg(a.band.band + 1) : a.ny / 2;
-  const int ncz = part ? min(a.nhp, (__ldg(a.band.band + 2) / a.col_unit + 1) * a.col_unit) : a.nhp;
-  const BoxRange rows = boxes_of<N, V>(part ? __ldg(a.band.band) : N / 2);
-  const bool flat = 2 * by + 1 >= a.ny && ncz >= a.nhp;
-  const int nrows = min(a.ny, 2 * by + 1), ktiles = (ncz + TC - 1) / TC;
-  const int tpr = flat ? (ncols + TC - 1) / TC : nrows * ktiles;  // tiles per realisation; the last may run past ncols
-  const int ntiles = tpr * a.batch;  // realisation r owns rows [r N, r N + N)
-  auto col_of = [&](int t) {  // first column of tile t of a realisation
-    if (flat) return t * TC;
-    const int row = t / ktiles;
-    return (row <= by ? row : a.ny - nrows + row) * a.nhp + (t - row * ktiles) * TC;
-  };
-  auto issue = [&](int tile) {
-    const int r = tile / tpr, c0 = col_of(tile % tpr);
-    mbar_expect_tx(bar, rows.count(G::kBoxes) * G::kRows * TC * 8);
-    if (!rows.part) {
+  WalkX<N, TC, V> cur(a);
+  WalkX<N, TC, V> nxt = cur;
+  auto issue = [&](const WalkX<N, TC, V>& w, int tile) {
+    const int t = tile - w.base, r = t / w.tpr, c0 = w.col(a, t % w.tpr);
+    mbar_expect_tx(bar, w.rows.count(G::kBoxes) * G::kRows * TC * 8);
+    if (!w.rows.part) {
 #pragma unroll
       for (int b = 0; b < GS::kBoxes; ++b)
         tma_load_2d(smem_u32(s_st + b * GS::kRows * TC), &a.tm_full, c0, r * N + b * GS::kRows, bar);
@@ -259,9 +316,9 @@ __global__ void __launch_bounds__(TC* Shape<N, V>::P, MinBlocks<N, TC, V>::xy)
     }
 #pragma unroll
     for (int b = 0; b < G::kBoxes; ++b)
-      if (rows.has(b)) tma_load_2d(smem_u32(s_st + b * G::kRows * TC), &a.tm, c0, r * N + b * G::kRows, bar);
+      if (w.rows.has(b)) tma_load_2d(smem_u32(s_st + b * G::kRows * TC), &a.tm, c0, r * N + b * G::kRows, bar);
   };
-  if (tid == 0 && (int)blockIdx.x < ntiles) issue(blockIdx.x);
+  if (tid == 0 && nxt.seek(a, blockIdx.x)) issue(nxt, blockIdx.x);
   uint32_t parity = 0;
   // TMA stores: an output tile is written into the exchange buffer in tile
   // order and stored by the copy engine; the next transform's first
@@ -274,13 +331,20 @@ __global__ void __launch_bounds__(TC* Shape<N, V>::P, MinBlocks<N, TC, V>::xy)
       pending = false;
     }
   };
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+  for (int tile = blockIdx.x; cur.seek(a, tile); tile += gridDim.x) {
     if (!stage_ready(bar, parity, a.err, a.wait_cycles)) {
       if (tid == 0) bulk_wait_all();
       return;
     }
     parity ^= 1;
-    const int col0 = col_of(tile % tpr), row0 = (tile / tpr) * N;
+    if (kMultiRad<N> && cur.g != g_m) {  // every thread is past its last read of s_m
+      g_m = cur.g;
+      for (int i = tid; i < 3 * N; i += TC * P) s_m[i] = a.mult[(size_t)a.rad.ms[g_m] * a.rad.mult_set + i];
+      __syncthreads();
+    }
+    const int tt = tile - cur.base;
+    const int col0 = cur.col(a, tt % cur.tpr), row0 = (tt / cur.tpr + cur.g * 3 * a.batch) * N;
+    const BoxRange rows = cur.rows;
 #pragma unroll 1
     for (int f = 0; f < a.nout; ++f) {
       const float* mt = s_m + s_xm[f] * N + p;
@@ -288,9 +352,9 @@ __global__ void __launch_bounds__(TC* Shape<N, V>::P, MinBlocks<N, TC, V>::xy)
       load_slots<N, TC, V, false>(v, s_st, mt, rows, 0, p, c);
       if (f == a.nout - 1) {
         __syncthreads();  // the tile has been read by every thread
-        if (tid == 0 && tile + (int)gridDim.x < ntiles) {
+        if (tid == 0 && nxt.seek(a, tile + gridDim.x)) {
           fence_proxy_async();
-          issue(tile + gridDim.x);
+          issue(nxt, tile + gridDim.x);
         }
       }
       fft_line<N, L, false, V>(v, p, c, s_x, s_tw, wait_store);
@@ -336,7 +400,8 @@ __global__ void __launch_bounds__(TC* Shape<N, V>::P, MinBlocks<N, TC, V>::xy)
   const int tid = threadIdx.x, c = tid % TC, p = tid / TC;
   const uint32_t bar = smem_u32(&s_bar);
   for (int i = tid; i < NTW; i += TC * P) s_tw[i] = a.tw[i];
-  for (int i = tid; i < 3 * N; i += TC * P) s_m[i] = a.mult[i];
+  int g_m = 0;  // radius whose multipliers s_m holds
+  for (int i = tid; i < 3 * N; i += TC * P) s_m[i] = a.mult[(size_t)a.rad.ms[0] * a.rad.mult_set + i];
   if (tid < kMaxFields) {
     s_dst[tid] = a.dst[tid];
     s_sel[tid] = a.sel[tid] < 3 ? a.sel[tid] : 0;
@@ -353,26 +418,22 @@ __global__ void __launch_bounds__(TC* Shape<N, V>::P, MinBlocks<N, TC, V>::xy)
   }
   __syncthreads();
   const int nhp = a.nhp, nout = a.nout;
-  // the filter's support (BandArgs): ky boxes and columns kz <= bz
-  const bool part = a.band.band != nullptr && __ldg(a.band.wide) == 0;
-  const int by = part ? __ldg(a.band.band + 1) : N / 2;
-  const BoxRange rows = boxes_of<N, V>(by);
-  const int ktiles = ((part ? __ldg(a.band.band + 2) + 1 : nhp) + TC - 1) / TC;
-  const int ntiles = a.nx * a.batch * ktiles;  // x planes of all realisations, back to back
-  auto issue = [&](int tile, int src) {
-    const int x = tile / ktiles, kz0 = (tile % ktiles) * TC;
-    mbar_expect_tx(bar, rows.count(G::kBoxes) * G::kRows * TC * 8);
-    if (!rows.part) {
+  WalkY<N, TC, V> cur(a);
+  WalkY<N, TC, V> nxt = cur;
+  auto issue = [&](const WalkY<N, TC, V>& w, int tile, int src) {
+    const int t = tile - w.base, x = t / w.ktiles, kz0 = (t - x * w.ktiles) * TC, sp = src + 3 * w.g;
+    mbar_expect_tx(bar, w.rows.count(G::kBoxes) * G::kRows * TC * 8);
+    if (!w.rows.part) {
 #pragma unroll
       for (int b = 0; b < GS::kBoxes; ++b)
-        tma_load_4d(smem_u32(s_st + b * GS::kRows * TC), &a.tm_full, kz0, b * GS::kRows, x, src, bar);
+        tma_load_4d(smem_u32(s_st + b * GS::kRows * TC), &a.tm_full, kz0, b * GS::kRows, x, sp, bar);
       return;
     }
 #pragma unroll
     for (int b = 0; b < G::kBoxes; ++b)
-      if (rows.has(b)) tma_load_4d(smem_u32(s_st + b * G::kRows * TC), &a.tm, kz0, b * G::kRows, x, src, bar);
+      if (w.rows.has(b)) tma_load_4d(smem_u32(s_st + b * G::kRows * TC), &a.tm, kz0, b * G::kRows, x, sp, bar);
   };
-  if (tid == 0 && (int)blockIdx.x < ntiles) issue(blockIdx.x, s_sel[0]);
+  if (tid == 0 && nxt.seek(a, blockIdx.x)) issue(nxt, blockIdx.x, s_sel[0]);
   uint32_t parity = 0;
   // TMA stores (single-store mode): as in the x pass
   constexpr bool kStore = !DUAL;
@@ -384,10 +445,14 @@ __global__ void __launch_bounds__(TC* Shape<N, V>::P, MinBlocks<N, TC, V>::xy)
       pending = false;
     }
   };
-  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int x = tile / ktiles, kz = (tile % ktiles) * TC + c;
+  for (int tile = blockIdx.x; cur.seek(a, tile); tile += gridDim.x) {
+    const int tt = tile - cur.base, x = tt / cur.ktiles, kz0 = (tt - x * cur.ktiles) * TC, kz = kz0 + c;
     const bool ok = kz < nhp;
     const size_t base = (size_t)x * N * nhp + (ok ? kz : 0);
+    const float* mult_z = a.mult_z + (size_t)a.rad.ms[cur.g] * a.rad.mult_set;
+    const int row0 = (cur.g * 6 * a.nx * a.batch + x) * N;
+    const BoxRange rows = cur.rows;
+    const int by = cur.by;
 #pragma unroll 1
     for (int o = 0; o < nout; ++o) {
       if (o == 0 || s_sel[o] != s_sel[o - 1]) {
@@ -396,6 +461,11 @@ __global__ void __launch_bounds__(TC* Shape<N, V>::P, MinBlocks<N, TC, V>::xy)
           return;
         }
         parity ^= 1;
+        if (kMultiRad<N> && cur.g != g_m) {  // every thread is past its last read of s_m
+          g_m = cur.g;
+          for (int i = tid; i < 3 * N; i += TC * P) s_m[i] = a.mult[(size_t)a.rad.ms[g_m] * a.rad.mult_set + i];
+          __syncthreads();
+        }
       }
       const float* mt = s_m + s_ym[o] * N + p;
       float2 v[E];
@@ -406,20 +476,20 @@ __global__ void __launch_bounds__(TC* Shape<N, V>::P, MinBlocks<N, TC, V>::xy)
         if (tid == 0) {
           if (o < nout - 1) {
             fence_proxy_async();
-            issue(tile, s_sel[o + 1]);
-          } else if (tile + (int)gridDim.x < ntiles) {
+            issue(cur, tile, s_sel[o + 1]);
+          } else if (nxt.seek(a, tile + gridDim.x)) {
             fence_proxy_async();
-            issue(tile + gridDim.x, s_sel[0]);
+            issue(nxt, tile + gridDim.x, s_sel[0]);
           }
         }
       }
       // z factors of this column (kz <= nz/2; pad columns carry zeros anyway),
       // requested before the transform so that their latency is hidden
       const int nz = a.nz;
-      const float zf = (ok && kz <= nz / 2) ? __ldg(a.mult_z + s_zm[o] * nz + kz) : 0.f;
+      const float zf = (ok && kz <= nz / 2) ? __ldg(mult_z + s_zm[o] * nz + kz) : 0.f;
       float zf2 = 0.f;
       if constexpr (DUAL)
-        zf2 = (ok && s_dst2[o] != nullptr && kz <= nz / 2) ? __ldg(a.mult_z + s_zm2[o] * nz + kz) : 0.f;
+        zf2 = (ok && s_dst2[o] != nullptr && kz <= nz / 2) ? __ldg(mult_z + s_zm2[o] * nz + kz) : 0.f;
       if constexpr (kStore) fft_line<N, L, false, V>(v, p, c, s_x, s_tw, wait_store);
       else fft_line<N, L, false, V>(v, p, c, s_x, s_tw);
       const bool mi = s_mi[o] != 0;
@@ -455,10 +525,9 @@ __global__ void __launch_bounds__(TC* Shape<N, V>::P, MinBlocks<N, TC, V>::xy)
         fence_proxy_async();
         __syncthreads();
         if (tid == 0) {
-          const int kz0 = (tile % ktiles) * TC;
 #pragma unroll
           for (int b = 0; b < GS::kBoxes; ++b)
-            tma_store_2d(&a.tm_out[o], kz0, x * N + b * GS::kRows, smem_u32(s_x + b * GS::kRows * TC));
+            tma_store_2d(&a.tm_out[o], kz0, row0 + b * GS::kRows, smem_u32(s_x + b * GS::kRows * TC));
           bulk_commit();
         }
         pending = true;
@@ -468,26 +537,33 @@ __global__ void __launch_bounds__(TC* Shape<N, V>::P, MinBlocks<N, TC, V>::xy)
     }
   }
   // columns past the band that the radius before had: zeros
-  const int zend = part ? ((a.band.prev ? __ldg(a.band.prev + 2) + 1 : nhp) + TC - 1) / TC : ktiles;
-  if (zend > ktiles) {
-    const int zt = zend - ktiles, nz0 = a.nx * a.batch * zt;
+  bool cleared = false;
+  for (int g = 0; g < (kMultiRad<N> ? a.rad.n : 1); ++g) {
+    if (a.rad.band == nullptr || __ldg(a.rad.wide) != 0) break;
+    const int had = a.rad.prev[g] < 0 ? nhp : __ldg(a.rad.band + 4 * a.rad.prev[g] + 2) + 1;
+    const int k0 = (__ldg(a.rad.band + 4 * a.rad.ms[g] + 2) + TC) / TC, zt = (had + TC - 1) / TC - k0;
+    if (zt <= 0) continue;
+    const int nz0 = a.nx * a.batch * zt;
     if constexpr (kStore) {
-      wait_store();
-      for (int i = tid; i < N * TC; i += TC * P) s_x[i] = make_float2(0.f, 0.f);
-      fence_proxy_async();
-      __syncthreads();
+      if (!cleared) {
+        wait_store();
+        for (int i = tid; i < N * TC; i += TC * P) s_x[i] = make_float2(0.f, 0.f);
+        fence_proxy_async();
+        __syncthreads();
+        cleared = true;
+      }
       if (tid == 0)
         for (int i = blockIdx.x; i < nz0; i += gridDim.x) {
-          const int x = i / zt, kz0 = (ktiles + i % zt) * TC;
+          const int x = i / zt, kz0 = (k0 + i - x * zt) * TC, row0 = (g * 6 * a.nx * a.batch + x) * N;
           for (int o = 0; o < nout; ++o)
 #pragma unroll
             for (int b = 0; b < GS::kBoxes; ++b)
-              tma_store_2d(&a.tm_out[o], kz0, x * N + b * GS::kRows, smem_u32(s_x + b * GS::kRows * TC));
+              tma_store_2d(&a.tm_out[o], kz0, row0 + b * GS::kRows, smem_u32(s_x + b * GS::kRows * TC));
           bulk_commit();
         }
     } else {
       for (int i = blockIdx.x; i < nz0; i += gridDim.x) {
-        const int x = i / zt, kz = (ktiles + i % zt) * TC + c;
+        const int x = i / zt, kz = (k0 + i - x * zt) * TC + c;
         if (kz >= nhp) continue;
         for (int o = 0; o < nout; ++o)
           for (int r = p; r < N; r += P) {
@@ -559,12 +635,14 @@ template <int N, int TC, int V>
 static cudaError_t run_x(const ArgsX& a_in, cudaStream_t st) {
   using C = CfgXY<N, TC, V>;
   ArgsX a = a_in;
+  if (a.rad.n < 1 || (a.rad.n > 1 && !kMultiRad<N>)) return cudaErrorInvalidValue;
   // output maps: the source map's geometry in store boxes, one per output
   for (int f = 0; f < a.nout; ++f) {
-    const cudaError_t e = make_tmap_x(&a.tm_out[f], a.dst[f], N, a.ny, a.nhp, a.batch, TC, Store<N>::kBoxes);
+    const cudaError_t e = make_tmap_x(&a.tm_out[f], a.dst[f], N, a.ny, a.nhp, a.batch * (3 * a.rad.n - 2), TC,
+                                      Store<N>::kBoxes);
     if (e != cudaSuccess) return e;
   }
-  const long ntiles = (((long)a.ny * a.nhp + TC - 1) / TC) * a.batch;
+  const long ntiles = (((long)a.ny * a.nhp + TC - 1) / TC) * a.batch * a.rad.n;
   const unsigned grid = persistent_grid(k_pass_x<N, TC, V>, C::threads, C::smem, ntiles);
   k_pass_x<N, TC, V><<<grid, C::threads, C::smem, st>>>(a);
   return cudaGetLastError();
@@ -573,15 +651,16 @@ static cudaError_t run_x(const ArgsX& a_in, cudaStream_t st) {
 template <int N, int TC, int V>
 static cudaError_t run_y(const ArgsY& a, cudaStream_t st) {
   using C = CfgXY<N, TC, V>;
-  const long ntiles = (long)a.nx * a.batch * ((a.nhp + TC - 1) / TC);
+  const long ntiles = (long)a.nx * a.batch * ((a.nhp + TC - 1) / TC) * a.rad.n;
   bool dual = false;
   for (int o = 0; o < a.nout; ++o) dual = dual || a.dst2[o] != nullptr;
+  if (a.rad.n < 1 || (a.rad.n > 1 && (dual || !kMultiRad<N>))) return cudaErrorInvalidValue;
   if (!dual) {
     // output maps: rows (x, ky) of nhp values in store boxes
     ArgsY b = a;
     for (int o = 0; o < b.nout; ++o) {
-      const cudaError_t e = make_tmap_rows(&b.tm_out[o], b.dst[o], b.nhp, (long long)b.nx * b.batch * N, TC,
-                                           Store<N>::kRows);
+      const cudaError_t e = make_tmap_rows(&b.tm_out[o], b.dst[o], b.nhp, (long long)b.nx * b.batch * N * (6 * b.rad.n - 5),
+                                           TC, Store<N>::kRows);
       if (e != cudaSuccess) return e;
     }
     const unsigned grid = persistent_grid(k_pass_y<N, TC, false, V>, C::threads, C::smem, ntiles);

@@ -48,8 +48,10 @@ struct pin_plan_s {
   size_t spec_elems = 0;  // complex elements of one padded half-spectrum
   size_t field_elems = 0; // batch * spec_elems: one field of every realisation
   float2* phi0 = nullptr;
-  float2* U = nullptr;    // 3 spectra
-  float2* V = nullptr;    // 6 spectra (9 with velocities)
+  int group = 1;          // radii the passes of one launch cover (radius_group)
+  float2* U = nullptr;    // 3 spectra per radius of a group
+  float2* V = nullptr;    // 6 spectra per radius of a group (9 with velocities)
+  unsigned long long* state = nullptr;  // behind V, groups: the running maximum (ArgsZ::state)
   float* psi = nullptr;   // [3][npart] displacement of the current radius (velocities)
   float* vstate = nullptr;  // [3][npart] displacement at R_max (velocities)
   float* fmax = nullptr;
@@ -103,8 +105,31 @@ struct pin_plan_s {
   const float* mx(int ms) const { return mult + ms * mult_set(); }
   const float* my(int ms) const { return mx(ms) + 3 * (size_t)nx; }
   const float* mz(int ms) const { return my(ms) + 3 * (size_t)ny; }
-  BandArgs bands(int ms, int prev = -1) const {
-    return BandArgs{band + 4 * ms, band + kBandWide, prev < 0 ? nullptr : band + 4 * prev};
+  // radii k0 .. k0 + n - 1 of a list of multiplier sets as one launch; the
+  // sets `group` places before them wrote the same V buffers
+  RadGroup radii_of(const int* ms, int k0, int n, int group) const {
+    RadGroup r{};
+    r.n = n;
+    r.mult_set = (int)mult_set();
+    for (int g = 0; g < n; ++g) {
+      r.ms[g] = ms[k0 + g];
+      r.prev[g] = k0 + g >= group ? ms[k0 + g - group] : -1;
+    }
+    r.band = band;
+    r.wide = band + kBandWide;
+    return r;
+  }
+  // radii per launch, the plan's groups evened out (20 radii in groups of at
+  // most 9: 7, 7, 6)
+  int even_group() const {
+    const int launches = (nscales + group - 1) / group;
+    return (nscales + launches - 1) / launches;
+  }
+  // one multiplier set, whole lines whatever it filters out
+  RadGroup full_set(int ms) const {
+    RadGroup r = radii_of(&ms, 0, 1, 1);
+    r.band = nullptr;
+    return r;
   }
   const float2* twx() const { return tw + tw_off[0]; }
   const float2* twy() const { return tw + tw_off[1]; }
@@ -372,16 +397,45 @@ unsigned redo_capacity(size_t n3, int batch) {
   return (unsigned)std::max<size_t>(65536, n3 * batch / 64);
 }
 
+// Radii per launch (RadGroup): as many as fit in kGroupBytes of spectra (9
+// padded ones each), 16 up to 64^3, 9 at 96^3, 4 at 128^3.  Larger groups than
+// L2 holds still pay, because they fill the SMs: 96^3 x 20 takes 1412 us one
+// radius at a time, 960 in twos (72 MB), 759 in fours, 564 in nines; 128^3 x 25
+// 2215 us singly, 1701 in twos, 1381 in fours; 64^3 x 20 916 us singly, 541 in
+// twos, 275 in sixes, 239 in tens.  Beyond, the memory is better left to the
+// caller.  Without velocities; lines of at most kGroupMaxN points.
+#ifndef PIN_GROUP_MB
+#define PIN_GROUP_MB 320
+#endif
+constexpr size_t kGroupBytes = (size_t)PIN_GROUP_MB << 20;
+int radius_group(int nx, int ny, int nz, int batch, bool velocities) {
+  if (velocities || std::max(nx, std::max(ny, nz)) > kGroupMaxN) return 1;
+  const size_t set = (size_t)9 * 8 * nx * ny * padded_half(nz) * batch;
+  return (int)std::max<size_t>(1, std::min<size_t>(kMaxGroup, kGroupBytes / set));
+}
+// Spectra of V, with the running maximum of a group behind them.
+size_t v_bytes(size_t field_elems, size_t npart, int group, bool velocities) {
+  return field_elems * 8 * (velocities ? 9 : 6) * group + (group > 1 ? npart * 8 : 0);
+}
+// A particle is queued at most once per radius: a group's queues need no more
+// than one entry per particle each.
+unsigned group_redo_cap(unsigned cap, size_t npart, int group) {
+  return group > 1 ? (unsigned)std::min<size_t>(cap, npart) : cap;
+}
+
 int batch_of(const pin_plan_desc* d) { return d->batch <= 0 ? 1 : d->batch; }
 
 size_t footprint(int nx, int ny, int nz, int nscales, int batch, bool velocities, bool fp64) {
   (void)nscales;
   const size_t spec = (size_t)nx * ny * padded_half(nz) * batch;
   const size_t n3 = (size_t)nx * ny * nz * batch;
-  return (fp64 ? fp64_workspace_bytes(nx, ny, nz) : 0) + spec * 8 * (velocities ? 13 : 10) + n3 * 8 +
-         (velocities ? n3 * 24 : 0) +
-         (size_t)(kMaxScales + 1) * 3 * (nx + ny + nz) * 4 + kBandInts * sizeof(int) + (size_t)(nx + ny + nz + 3 * 64) * 8 + 64 +
-         (size_t)redo_capacity((size_t)nx * ny * nz, batch) * sizeof(RedoEntry) + 16 + sizeof(int);
+  const int group = radius_group(nx, ny, nz, batch, velocities);
+  const size_t cap = group_redo_cap(redo_capacity((size_t)nx * ny * nz, batch), n3, group);
+  return (fp64 ? fp64_workspace_bytes(nx, ny, nz) : 0) + spec * 8 * (1 + 3 * group) +
+         v_bytes(spec, n3, group, velocities) + n3 * 8 + (velocities ? n3 * 24 : 0) +
+         (size_t)(kMaxScales + 1) * 3 * (nx + ny + nz) * 4 + kBandInts * sizeof(int) +
+         (size_t)(nx + ny + nz + 3 * 64) * 8 + 64 + cap * group * sizeof(RedoEntry) +
+         kMaxGroup * sizeof(unsigned) + 16 + sizeof(int);
 }
 
 pin_status ensure_device_init(pin_plan_t p) {
@@ -498,22 +552,23 @@ std::vector<int> band_table(pin_plan_t p, const std::vector<float>& mult) {
 }
 
 // Source maps {staged boxes, whole-line boxes} of the x pass over one spectrum
-// and of the y pass over the three spectra at src, for tile width tc.
+// and of the y pass over the spectra at src (three per radius of a group; a
+// launch names the ones it reads), for tile width tc.
 cudaError_t source_maps_x(pin_plan_t p, CUtensorMap* tm, const float2* src, int batch, int tc) {
   cudaError_t e = make_tmap_x(tm, src, p->nx, p->ny, p->nhp, batch, tc, stage_boxes(p->shape_x.E));
   if (e == cudaSuccess) e = make_tmap_x(tm + 1, src, p->nx, p->ny, p->nhp, batch, tc, store_boxes(p->nx));
   return e;
 }
 cudaError_t source_maps_y(pin_plan_t p, CUtensorMap* tm, const float2* src, int batch, int tc) {
-  cudaError_t e = make_tmap_y(tm, src, p->nx, p->ny, p->nhp, p->field_elems, batch, tc, stage_boxes(p->shape_y.E));
+  cudaError_t e = make_tmap_y(tm, src, p->nx, p->ny, p->nhp, p->field_elems, 3 * p->group, batch, tc,
+                              stage_boxes(p->shape_y.E));
   if (e == cudaSuccess)
-    e = make_tmap_y(tm + 1, src, p->nx, p->ny, p->nhp, p->field_elems, batch, tc, store_boxes(p->ny));
+    e = make_tmap_y(tm + 1, src, p->nx, p->ny, p->nhp, p->field_elems, 3 * p->group, batch, tc, store_boxes(p->ny));
   return e;
 }
 
-// x pass of one radius (mult set `ms`): Phi0 -> U[0..2] with the x factors
-// W, k W, k^2 W.
-ArgsX radius_args_x(pin_plan_t p, int ms) {
+// x pass of a group of radii: Phi0 -> U[0..2] with the x factors W, k W, k^2 W.
+ArgsX radius_args_x(pin_plan_t p, const RadGroup& rad) {
   ArgsX ax{};
   ax.tm = p->tm_x[0];
   ax.tm_full = p->tm_x[1];
@@ -521,8 +576,8 @@ ArgsX radius_args_x(pin_plan_t p, int ms) {
   for (int f = 0; f < 3; ++f) { ax.dst[f] = spec(p, p->U, f); ax.xm[f] = f; }
   ax.nout = 3;
   ax.ny = p->ny;
-  ax.mult = p->mx(ms);
-  ax.band = p->bands(ms);
+  ax.mult = p->mx(0);
+  ax.rad = rad;
   ax.col_unit = p->tc_y;
   ax.tw = p->twx();
   ax.nhp = p->nhp;
@@ -532,13 +587,13 @@ ArgsX radius_args_x(pin_plan_t p, int ms) {
   return ax;
 }
 
-// y pass of one radius, outputs grouped by source so that each staged tile
+// y pass of a group of radii, outputs grouped by source so that each staged tile
 // serves them in a row: V[xx] <- U2; V[xy] <- U1 (k_y), V[xz] <- U1 (z: k_z);
 // V[yy] <- U0 (k_y^2), V[zz] <- U0 (z: k_z^2), V[yz] <- U0 (k_y; z: k_z).
 // With the velocities of a collapse call, the smoothed displacement
 // psi = i k W Phi0 shares the y transforms of xz (psi_x: z factor W), zz
 // (psi_z: z factor k W) and yz (psi_y: z factor W).
-ArgsY radius_args_y(pin_plan_t p, int ms, bool collapse, float2* vbuf = nullptr, int prev = -1) {
+ArgsY radius_args_y(pin_plan_t p, const RadGroup& rad, bool collapse, float2* vbuf = nullptr) {
   if (!vbuf) vbuf = p->V;
   static const int vout[6] = {0, 3, 4, 1, 2, 5};
   static const int sel[6] = {2, 1, 1, 0, 0, 0};
@@ -569,9 +624,9 @@ ArgsY radius_args_y(pin_plan_t p, int ms, bool collapse, float2* vbuf = nullptr,
   ay.nout = 6;
   ay.nx = p->nx;
   ay.nz = p->nz;
-  ay.mult = p->my(ms);
-  ay.mult_z = p->mz(ms);
-  ay.band = p->bands(ms, prev);
+  ay.mult = p->my(0);
+  ay.mult_z = p->mz(0);
+  ay.rad = rad;
   ay.tw = p->twy();
   ay.nhp = p->nhp;
   ay.batch = p->batch;
@@ -580,38 +635,39 @@ ArgsY radius_args_y(pin_plan_t p, int ms, bool collapse, float2* vbuf = nullptr,
   return ay;
 }
 
-// Where the passes of one radius of the collapse loop run: the x and y passes
-// on xs, the z pass and the FP64 redo on zs, the y outputs in vbuf; the y pass
-// first waits for y_wait (if set), y_done is recorded after it (and zs waits
-// for it), z_done after the redo.  prev: the multiplier set of the radius
-// that wrote vbuf before in this call, -1 for the first.  The serial schedule
+// Where the passes of one radius (or group of radii) of the collapse loop run:
+// the x and y passes on xs, the z pass and the FP64 redo on zs, the y outputs
+// in vbuf; the y pass first waits for y_wait (if set), y_done is recorded
+// after it (and zs waits for it), z_done after the redo.  The serial schedule
 // is xs = zs = the plan's stream, vbuf = V, no events.
 struct RadiusSched {
   cudaStream_t xs, zs;
   float2* vbuf;
   cudaEvent_t y_wait, y_done, z_done;
-  int prev;
 };
 
-// Filter-and-transform passes of one radius (mult set `ms`), ending in the
-// collapse update (dump and source null), a dump of the six real components,
-// or the 2LPT source field S of every particle (source, batch 1).
-pin_status enqueue_radius(pin_plan_t p, int ms, int scale, float* const* dump, float* source = nullptr,
-                          const RadiusSched* sched = nullptr) {
+// Filter-and-transform passes of a group of radii (one, unless the plan runs
+// groups and this is the collapse loop), ending in the collapse update (dump
+// and source null), a dump of the six real components, or the 2LPT source
+// field S of every particle (source, batch 1).  A multiplier set is the index
+// of its radius.
+pin_status enqueue_radii(pin_plan_t p, const RadGroup& rad, float* const* dump, float* source = nullptr,
+                         const RadiusSched* sched = nullptr) {
   const bool collapse = dump == nullptr && source == nullptr;
-  const RadiusSched rs = sched ? *sched : RadiusSched{p->stream, p->stream, p->V, nullptr, nullptr, nullptr, -1};
+  const int scale = rad.ms[0];
+  const RadiusSched rs = sched ? *sched : RadiusSched{p->stream, p->stream, p->V, nullptr, nullptr, nullptr};
   const bool rec = p->profile && collapse && !p->events.empty();
   auto mark = [&](int k, cudaStream_t st) {
     return rec ? cudaEventRecordWithFlags(p->events[7 * scale + k], st, cudaEventRecordExternal) : cudaSuccess;
   };
   PIN_CK(p, mark(0, rs.xs));
-  const ArgsX ax = radius_args_x(p, ms);
+  const ArgsX ax = radius_args_x(p, rad);
   PIN_CK(p, launch_x(p->nx, p->tc_x, p->vx, ax, rs.xs));
   PIN_CK(p, mark(1, rs.xs));
   if (rs.y_wait) PIN_CK(p, cudaStreamWaitEvent(rs.xs, rs.y_wait, 0));
 
   PIN_CK(p, mark(2, rs.xs));
-  const ArgsY ay = radius_args_y(p, ms, collapse, rs.vbuf, rs.prev);
+  const ArgsY ay = radius_args_y(p, rad, collapse, rs.vbuf);
   PIN_CK(p, launch_y(p->ny, p->tc_y, p->vy, ay, rs.xs));
   PIN_CK(p, mark(3, rs.xs));
   if (rs.y_done) {
@@ -632,6 +688,12 @@ pin_status enqueue_radius(pin_plan_t p, int ms, int scale, float* const* dump, f
   az.fmax = p->fmax;
   az.idx = p->idx;
   az.scale = scale;
+  if (collapse && p->group > 1) {
+    az.state = p->state;
+    az.nrad = rad.n;
+    for (int g = 0; g < rad.n; ++g) az.ms[g] = rad.ms[g];
+    az.gstride = 6 * p->field_elems;
+  }
   az.correction = p->correction;
   az.dcorr_d = p->dcorr;
   az.dcorr_f = (float)p->dcorr;
@@ -649,27 +711,39 @@ pin_status enqueue_radius(pin_plan_t p, int ms, int scale, float* const* dump, f
     return PIN_OK;
   }
   PIN_CK(p, mark(4, rs.zs));
-  if (!dump) PIN_CK(p, cudaMemsetAsync(p->redo_count, 0, sizeof(unsigned), rs.zs));
+  if (!dump) PIN_CK(p, cudaMemsetAsync(p->redo_count, 0, rad.n * sizeof(unsigned), rs.zs));
   PIN_CK(p, launch_z(p->nz, az, dump != nullptr, rs.zs));
   PIN_CK(p, mark(5, rs.zs));
-  if (!dump) {
-    PIN_CK(p, launch_redo(az, rs.zs));
-  }
+  if (!dump) PIN_CK(p, launch_redo(az, rs.zs));
   PIN_CK(p, mark(6, rs.zs));
   if (rs.z_done) PIN_CK(p, cudaEventRecord(rs.z_done, rs.zs));
   return PIN_OK;
 }
 
+// The unfused products of one radius (or of the R = 0 set).
+pin_status enqueue_radius(pin_plan_t p, int ms, float* const* dump, float* source = nullptr) {
+  return enqueue_radii(p, p->radii_of(&ms, 0, 1, 1), dump, source);
+}
+
 pin_status enqueue_collapse(pin_plan_t p) {
   const size_t n3 = p->n3() * p->batch;
+  const int* order = p->order.data();
+  if (p->group > 1) {
+    PIN_CK(p, cudaMemsetAsync(p->state, 0, n3 * sizeof(*p->state), p->stream));
+    const int group = p->even_group();
+    for (int k = 0; k < p->nscales; k += group) {
+      pin_status st = enqueue_radii(p, p->radii_of(order, k, std::min(group, p->nscales - k), group), nullptr);
+      if (st != PIN_OK) return st;
+    }
+    PIN_CK(p, launch_unpack(p->state, n3, p->fmax, p->idx, p->stream));
+    return PIN_OK;
+  }
   PIN_CK(p, cudaMemsetAsync(p->fmax, 0, n3 * sizeof(float), p->stream));
   PIN_CK(p, cudaMemsetAsync(p->idx, 0xFF, n3 * sizeof(int), p->stream));
   if (p->velocities) PIN_CK(p, cudaMemsetAsync(p->vstate, 0, 3 * n3 * sizeof(float), p->stream));
   if (p->sched == 0) {
     for (int k = 0; k < p->nscales; ++k) {
-      const int s = p->order[k];
-      const RadiusSched rs{p->stream, p->stream, p->V, nullptr, nullptr, nullptr, k ? p->order[k - 1] : -1};
-      pin_status st = enqueue_radius(p, s, s, nullptr, nullptr, &rs);
+      pin_status st = enqueue_radii(p, p->radii_of(order, k, 1, 1), nullptr);
       if (st != PIN_OK) return st;
     }
     return PIN_OK;
@@ -686,11 +760,10 @@ pin_status enqueue_collapse(pin_plan_t p) {
   PIN_CK(p, cudaStreamWaitEvent(p->s_xy, p->cap_ev[0], 0));
   PIN_CK(p, cudaStreamWaitEvent(p->s_z, p->cap_ev[0], 0));
   for (int k = 0; k < p->nscales; ++k) {
-    const int s = p->order[k];
-    RadiusSched rs{p->s_xy, p->s_z, (nbuf == 2 && (k & 1)) ? p->V2 : p->V,
-                   k >= nbuf ? p->cap_ev[2 + 2 * (k - nbuf)] : nullptr, p->cap_ev[1 + 2 * k], p->cap_ev[2 + 2 * k],
-                   k >= nbuf ? p->order[k - nbuf] : -1};
-    pin_status st = enqueue_radius(p, s, s, nullptr, nullptr, &rs);
+    const RadiusSched rs{p->s_xy, p->s_z, (nbuf == 2 && (k & 1)) ? p->V2 : p->V,
+                         k >= nbuf ? p->cap_ev[2 + 2 * (k - nbuf)] : nullptr, p->cap_ev[1 + 2 * k],
+                         p->cap_ev[2 + 2 * k]};
+    pin_status st = enqueue_radii(p, p->radii_of(order, k, 1, nbuf), nullptr, nullptr, &rs);
     if (st != PIN_OK) return st;
   }
   // join: the plan's stream continues after the last redo and the last y pass
@@ -818,9 +891,8 @@ pin_status apply_radix(pin_plan_t p, int vx, int vy) {
 // at tile width tc with the plan's current radix schedules, after one
 // untimed launch, on the plan's stream.
 pin_status time_pass(pin_plan_t p, bool y_pass, int tc, int reps, float* ms) {
-  ArgsX ax = radius_args_x(p, 0);
-  ArgsY ay = radius_args_y(p, 0, true);
-  ax.band = ay.band = BandArgs{};  // full passes, whatever the first radius filters out
+  ArgsX ax = radius_args_x(p, p->full_set(0));
+  ArgsY ay = radius_args_y(p, p->full_set(0), true);
   CUtensorMap tm[2];
   cudaError_t e = y_pass ? source_maps_y(p, tm, p->U, p->batch, tc) : source_maps_x(p, tm, p->phi0, p->batch, tc);
   (y_pass ? ay.tm : ax.tm) = tm[0];
@@ -880,7 +952,8 @@ pin_status pin_plan(pin_plan_t* out, const pin_plan_desc* d) {
   p->spec_elems = (size_t)p->nx * p->ny * p->nhp;
   p->field_elems = p->spec_elems * p->batch;
   p->dcorr = correction_dcorr();
-  p->redo_cap = redo_capacity(p->n3(), p->batch);
+  p->group = radius_group(p->nx, p->ny, p->nz, p->batch, p->velocities);
+  p->redo_cap = group_redo_cap(redo_capacity(p->n3(), p->batch), p->n3() * p->batch, p->group);
   auto bail = [&](pin_status s) {
     release(p);
     delete p;
@@ -907,14 +980,14 @@ pin_status pin_plan(pin_plan_t* out, const pin_plan_desc* d) {
     tw_elems += (size_t)ns[a] + (a < 2 ? 64 : (shapes[a]->P2 > 1 ? shapes[a]->P : 0));
   }
   auto A = [](auto** ptr, size_t bytes) { return plan_alloc(reinterpret_cast<void**>(ptr), bytes); };
-  if (A(&p->phi0, p->field_elems * 8) != cudaSuccess || A(&p->U, 3 * p->field_elems * 8) != cudaSuccess ||
-      A(&p->V, (p->velocities ? 9 : 6) * p->field_elems * 8) != cudaSuccess ||
+  if (A(&p->phi0, p->field_elems * 8) != cudaSuccess || A(&p->U, 3 * p->group * p->field_elems * 8) != cudaSuccess ||
+      A(&p->V, v_bytes(p->field_elems, n3, p->group, p->velocities)) != cudaSuccess ||
       (p->velocities && (A(&p->psi, 3 * n3 * 4) != cudaSuccess || A(&p->vstate, 3 * n3 * 4) != cudaSuccess)) ||
       A(&p->fmax, n3 * 4) != cudaSuccess || A(&p->idx, n3 * 4) != cudaSuccess ||
       A(&p->mult, mult_elems * 4 + kBandInts * sizeof(int)) != cudaSuccess || A(&p->tw, tw_elems * 8) != cudaSuccess ||
       A(&p->counters, 3 * sizeof(unsigned long long)) != cudaSuccess ||
-      A(&p->redo_list, (size_t)p->redo_cap * sizeof(RedoEntry)) != cudaSuccess ||
-      A(&p->redo_count, sizeof(unsigned)) != cudaSuccess || A(&p->err, sizeof(int)) != cudaSuccess ||
+      A(&p->redo_list, (size_t)p->redo_cap * p->group * sizeof(RedoEntry)) != cudaSuccess ||
+      A(&p->redo_count, kMaxGroup * sizeof(unsigned)) != cudaSuccess || A(&p->err, sizeof(int)) != cudaSuccess ||
       (p->precision == PIN_FP64 &&
        (A(&p->d64, (size_t)p->nx * p->ny * (p->nz / 2 + 1) * 16) != cudaSuccess ||
         A(&p->w64, n3 * 16) != cudaSuccess || A(&p->h64, 6 * n3 * 8) != cudaSuccess ||
@@ -923,6 +996,7 @@ pin_status pin_plan(pin_plan_t* out, const pin_plan_desc* d) {
     return bail(PIN_ENOMEM);
   }
   p->band = reinterpret_cast<int*>(p->mult + mult_elems);
+  if (p->group > 1) p->state = reinterpret_cast<unsigned long long*>(p->V + 6 * p->group * p->field_elems);
   const std::vector<float> mult = mult_table(p);
   const std::vector<int> band = band_table(p, mult);
   std::vector<float2> tw(tw_elems);
@@ -944,7 +1018,7 @@ pin_status pin_plan(pin_plan_t* out, const pin_plan_desc* d) {
 }
 
 // Phi0 of the field in src (device-readable), and whether the field is one
-// that runs full (BandArgs).
+// that runs full (RadGroup::wide).
 static cudaError_t load_phi0(pin_plan_t p, const void* src, int dtype) {
   const cudaError_t e = cudaMemsetAsync(p->band + kBandWide, 0, sizeof(int), p->stream);
   if (e != cudaSuccess) return e;
@@ -1122,7 +1196,7 @@ pin_status pin_hessian(pin_plan_t p, int scale, float* out6, int on_device) {
   if (!on_device) PIN_CK(p, cudaMallocAsync((void**)&dev, 6 * n3 * 4, p->stream));
   float* outs[6];
   for (int f = 0; f < 6; ++f) outs[f] = dev + (size_t)f * n3;
-  st = enqueue_radius(p, scale, scale, outs);
+  st = enqueue_radius(p, scale, outs);
   if (st == PIN_OK && !on_device) {
     cudaError_t e = cudaMemcpyAsync(out6, dev, 6 * n3 * 4, cudaMemcpyDeviceToHost, p->stream);
     if (e != cudaSuccess) st = cuda_fail(p, e, "cudaMemcpyAsync");
@@ -1154,7 +1228,8 @@ static cudaError_t enqueue_gradient(pin_plan_t p, float2* phi, float2* a0, float
   ax.xm[1] = 1;
   ax.nout = 2;
   ax.ny = p->ny;
-  ax.mult = p->mx(r0);
+  ax.mult = p->mx(0);
+  ax.rad = p->full_set(r0);
   ax.tw = p->twx();
   ax.nhp = p->nhp;
   ax.batch = 1;
@@ -1182,8 +1257,9 @@ static cudaError_t enqueue_gradient(pin_plan_t p, float2* phi, float2* a0, float
   ay.nout = 3;
   ay.nx = p->nx;
   ay.nz = p->nz;
-  ay.mult = p->my(r0);
-  ay.mult_z = p->mz(r0);
+  ay.mult = p->my(0);
+  ay.mult_z = p->mz(0);
+  ay.rad = p->full_set(r0);
   ay.tw = p->twy();
   ay.nhp = p->nhp;
   ay.batch = 1;
@@ -1239,7 +1315,7 @@ pin_status pin_displacements_2lpt(pin_plan_t p, float* psi2, int on_device) {
   float2* V0 = spec(p, p->V, 0);
   float* S = reinterpret_cast<float*>(U0);  // nx ny nz floats fit in one padded spectrum
   // 1) the unsmoothed deformation tensor, reduced per particle to the source S
-  st = enqueue_radius(p, kMaxScales, 0, nullptr, S);
+  st = enqueue_radius(p, kMaxScales, nullptr, S);
   // 2) T = inverse-sign transform of S: z into V0, y into V1, x into V2; the
   //    R = 0 multipliers scale each y line by 1/ny, each x line by 1/nx and
   //    the y outputs by 1/nz (z factor), so T / (nx ny nz) arrives in V2
@@ -1259,8 +1335,9 @@ pin_status pin_displacements_2lpt(pin_plan_t p, float* psi2, int on_device) {
     ay.nout = 1;
     ay.nx = nx;
     ay.nz = nz;
-    ay.mult = p->my(r0);
-    ay.mult_z = p->mz(r0);
+    ay.mult = p->my(0);
+    ay.mult_z = p->mz(0);
+    ay.rad = p->full_set(r0);
     ay.tw = p->twy();
     ay.nhp = p->nhp;
     ay.batch = 1;
@@ -1275,7 +1352,8 @@ pin_status pin_displacements_2lpt(pin_plan_t p, float* psi2, int on_device) {
     ax.dst[0] = spec(p, p->V, 2);
     ax.nout = 1;
     ax.ny = ny;
-    ax.mult = p->mx(r0);
+    ax.mult = p->mx(0);
+    ax.rad = p->full_set(r0);
     ax.tw = p->twx();
     ax.nhp = p->nhp;
     ax.batch = 1;
@@ -1334,7 +1412,8 @@ pin_status pin_get_stats(pin_plan_t p, pin_stats* out) {
 
 int pin_kernels_per_call(pin_plan_t p) {
   if (!p) return 0;
-  return 4 * p->nscales;  // x, y, z, redo per radius
+  // x, y, z, redo per radius or group of radii; groups end in one unpack
+  return 4 * ((p->nscales + p->group - 1) / p->group) + (p->group > 1 ? 1 : 0);
 }
 
 pin_status pin_profile(pin_plan_t p, int enable) {
@@ -1490,8 +1569,9 @@ pin_status pin_pass_times(pin_plan_t p, double* ms4) {
   ms4[0] = ms4[1] = ms4[2] = ms4[3] = 0.0;
   // events per radius: x begin/end, y begin/end, z begin/end, redo end
   static const int from[4] = {0, 2, 4, 5}, to[4] = {1, 3, 5, 6};
-  for (int s = 0; s < p->nscales; ++s)
+  for (int j = 0; j < p->nscales; j += p->even_group())
     for (int k = 0; k < 4; ++k) {
+      const int s = p->order[j];  // a group's events are its first radius's
       float ms = 0.f;
       PIN_CK(p, cudaEventElapsedTime(&ms, p->events[7 * s + from[k]], p->events[7 * s + to[k]]));
       ms4[k] += ms;
