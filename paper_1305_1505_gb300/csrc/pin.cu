@@ -88,6 +88,8 @@ struct pin_plan_s {
   // radius s on a second stream while the x pass of s + 1 runs; 2 also the y
   // pass of s + 1, into a second set of V spectra
   int sched = 0;
+  cudaStream_t s_redo = nullptr;               // the FP64 redo's branch of the captured loop
+  cudaEvent_t redo_ev[2] = {nullptr, nullptr};
   cudaStream_t s_xy = nullptr, s_z = nullptr;  // high / low priority streams of the overlapped schedule
   float2* V2 = nullptr;                        // second V buffer (schedule 2)
   // PIN_FP64 plans: FP64 half-spectrum, one full complex cube, the tensor,
@@ -491,6 +493,9 @@ void release(pin_plan_t p) {
   p->fmax64 = nullptr;
   for (cudaEvent_t e : p->cap_ev) cudaEventDestroy(e);
   p->cap_ev.clear();
+  for (cudaEvent_t e : p->redo_ev)
+    if (e) cudaEventDestroy(e);
+  if (p->s_redo) cudaStreamDestroy(p->s_redo);
   if (p->s_xy) cudaStreamDestroy(p->s_xy);
   if (p->s_z) cudaStreamDestroy(p->s_z);
   p->s_xy = p->s_z = nullptr;
@@ -640,10 +645,18 @@ ArgsY radius_args_y(pin_plan_t p, const RadGroup& rad, bool collapse, float2* vb
 // in vbuf; the y pass first waits for y_wait (if set), y_done is recorded
 // after it (and zs waits for it), z_done after the redo.  The serial schedule
 // is xs = zs = the plan's stream, vbuf = V, no events.
+//
+// The serial loop of a captured call runs the redo on a stream of its own
+// (rs), beside the x and y passes of the next radius: 25 us of FP64 latency
+// for a few thousand particles.  It has to be over before the next z pass,
+// which refills its queue and updates the same particles: z_wait, recorded as
+// redo_done after the redo; z_end marks the end of the z pass for rs.
 struct RadiusSched {
   cudaStream_t xs, zs;
   float2* vbuf;
   cudaEvent_t y_wait, y_done, z_done;
+  cudaStream_t rs = nullptr;
+  cudaEvent_t z_wait = nullptr, z_end = nullptr, redo_done = nullptr;
 };
 
 // Filter-and-transform passes of a group of radii (one, unless the plan runs
@@ -710,12 +723,20 @@ pin_status enqueue_radii(pin_plan_t p, const RadGroup& rad, float* const* dump, 
     PIN_CK(p, launch_z_source(p->nz, az, rs.zs));
     return PIN_OK;
   }
+  if (rs.z_wait) PIN_CK(p, cudaStreamWaitEvent(rs.zs, rs.z_wait, 0));
   PIN_CK(p, mark(4, rs.zs));
   if (!dump) PIN_CK(p, cudaMemsetAsync(p->redo_count, 0, rad.n * sizeof(unsigned), rs.zs));
   PIN_CK(p, launch_z(p->nz, az, dump != nullptr, rs.zs));
   PIN_CK(p, mark(5, rs.zs));
-  if (!dump) PIN_CK(p, launch_redo(az, rs.zs));
-  PIN_CK(p, mark(6, rs.zs));
+  cudaStream_t redo_stream = rs.zs;
+  if (rs.rs) {
+    redo_stream = rs.rs;
+    PIN_CK(p, cudaEventRecord(rs.z_end, rs.zs));
+    PIN_CK(p, cudaStreamWaitEvent(rs.rs, rs.z_end, 0));
+  }
+  if (!dump) PIN_CK(p, launch_redo(az, redo_stream));
+  PIN_CK(p, mark(6, redo_stream));
+  if (rs.rs) PIN_CK(p, cudaEventRecord(rs.redo_done, rs.rs));
   if (rs.z_done) PIN_CK(p, cudaEventRecord(rs.z_done, rs.zs));
   return PIN_OK;
 }
@@ -728,26 +749,30 @@ pin_status enqueue_radius(pin_plan_t p, int ms, float* const* dump, float* sourc
 pin_status enqueue_collapse(pin_plan_t p) {
   const size_t n3 = p->n3() * p->batch;
   const int* order = p->order.data();
+  // the serial loop, in groups of `group` radii
+  auto serial = [&](int group) -> pin_status {
+    RadiusSched rs{p->stream, p->stream, p->V, nullptr, nullptr, nullptr, p->s_redo, nullptr, p->redo_ev[0],
+                   p->redo_ev[1]};
+    for (int k = 0; k < p->nscales; k += group) {
+      pin_status st =
+          enqueue_radii(p, p->radii_of(order, k, std::min(group, p->nscales - k), group), nullptr, nullptr, &rs);
+      if (st != PIN_OK) return st;
+      rs.z_wait = rs.redo_done;
+    }
+    PIN_CK(p, cudaStreamWaitEvent(p->stream, rs.redo_done, 0));
+    return PIN_OK;
+  };
   if (p->group > 1) {
     PIN_CK(p, cudaMemsetAsync(p->state, 0, n3 * sizeof(*p->state), p->stream));
-    const int group = p->even_group();
-    for (int k = 0; k < p->nscales; k += group) {
-      pin_status st = enqueue_radii(p, p->radii_of(order, k, std::min(group, p->nscales - k), group), nullptr);
-      if (st != PIN_OK) return st;
-    }
+    pin_status st = serial(p->even_group());
+    if (st != PIN_OK) return st;
     PIN_CK(p, launch_unpack(p->state, n3, p->fmax, p->idx, p->stream));
     return PIN_OK;
   }
   PIN_CK(p, cudaMemsetAsync(p->fmax, 0, n3 * sizeof(float), p->stream));
   PIN_CK(p, cudaMemsetAsync(p->idx, 0xFF, n3 * sizeof(int), p->stream));
   if (p->velocities) PIN_CK(p, cudaMemsetAsync(p->vstate, 0, 3 * n3 * sizeof(float), p->stream));
-  if (p->sched == 0) {
-    for (int k = 0; k < p->nscales; ++k) {
-      pin_status st = enqueue_radii(p, p->radii_of(order, k, 1, 1), nullptr);
-      if (st != PIN_OK) return st;
-    }
-    return PIN_OK;
-  }
+  if (p->sched == 0) return serial(1);
   // Overlapped schedule: the x and y passes of radius s + 1 run on s_xy while
   // the z pass and the redo of radius s run on s_z.  The y pass of radius s
   // overwrites the V buffer that the z pass of radius s - nbuf read, so it
@@ -774,6 +799,10 @@ pin_status enqueue_collapse(pin_plan_t p) {
 
 pin_status ensure_graph(pin_plan_t p) {
   if (p->graph_exec) return PIN_OK;
+  if (!p->s_redo) {
+    PIN_CK(p, cudaStreamCreateWithFlags(&p->s_redo, cudaStreamNonBlocking));
+    for (auto& e : p->redo_ev) PIN_CK(p, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  }
   PIN_CK(p, cudaStreamBeginCapture(p->stream, cudaStreamCaptureModeThreadLocal));
   pin_status st = enqueue_collapse(p);
   cudaGraph_t g = nullptr;
