@@ -1421,7 +1421,10 @@ pin_status pin_sync(pin_plan_t p, int64_t timeout_ns) {
                           std::chrono::steady_clock::now() - t0).count();
       if (dt >= timeout_ns) return fail(p, PIN_ETIMEOUT, "pin_sync timed out");
     }
-    std::this_thread::sleep_for(std::chrono::microseconds(20));
+    // a sleep takes at least 50 us of timer slack, as long as a small call:
+    // poll without it for the first millisecond
+    if (std::chrono::steady_clock::now() - t0 > std::chrono::milliseconds(1))
+      std::this_thread::sleep_for(std::chrono::microseconds(20));
   }
 }
 
