@@ -194,39 +194,64 @@ struct CollapseStateX2 {
   unsigned need;   // bit (2 a + lane): axis a + 1 of that lane may collapse first
 };
 
-// First part of collapse_main<float> for two particles: the coefficients of
-// the three axes (c0 for the axis of the largest eigenvalue, st.c for the
-// others) and the quasi-spherical correction term st.corr.
-__device__ __forceinline__ void collapse_prep_x2(const float2 lam[3], const CollapseConsts<float>& cc,
-                                                 CollapseStateX2& st, float2 c0[3]) {
+// Invariants, half products e_i and the coefficients of the axis of the largest
+// eigenvalue.
+struct AxisZeroX2 {
+  float2 mu1, nmu3, s12, s02, s01, e0, e1, e2, c[3];
+};
+__device__ __forceinline__ AxisZeroX2 axis_zero_x2(const float2 lam[3]) {
   using namespace x2;
-  const float2 mu1 = add(add(lam[0], lam[1]), lam[2]);
-  const float2 mu3 = mul(mul(lam[0], lam[1]), lam[2]);
-  const float2 s12 = add(lam[1], lam[2]), s02 = add(lam[0], lam[2]), s01 = add(lam[0], lam[1]);
+  AxisZeroX2 a;
   const float2 half = splat(0.5f);
-  const float2 e0 = mul(mul(half, lam[0]), s12);
-  const float2 e1 = mul(mul(half, lam[1]), s02);
-  const float2 e2 = mul(mul(half, lam[2]), s01);
-  const float2 k37 = splat(3.0f / 7.0f), k1084 = splat(10.0f / 84.0f);
-  const float2 nmu3 = mul(mu3, splat(-1.0f / 9.0f));
+  a.mu1 = add(add(lam[0], lam[1]), lam[2]);
+  const float2 mu3 = mul(mul(lam[0], lam[1]), lam[2]);
+  a.s12 = add(lam[1], lam[2]);
+  a.s02 = add(lam[0], lam[2]);
+  a.s01 = add(lam[0], lam[1]);
+  a.e0 = mul(mul(half, lam[0]), a.s12);
+  a.e1 = mul(mul(half, lam[1]), a.s02);
+  a.e2 = mul(mul(half, lam[2]), a.s01);
+  a.nmu3 = mul(mu3, splat(-1.0f / 9.0f));
   // axis i: c1 = lam_i, c2 = (3/7) e_i, c3 = (10/84)(lam_i (e_j + e_k) + e_i (lam_j + lam_k)) - mu3/9
-  c0[0] = lam[0];
-  c0[1] = mul(k37, e0);
-  c0[2] = fma(k1084, fma(e0, s12, mul(lam[0], add(e1, e2))), nmu3);
-  st.c[0][0] = lam[1];
-  st.c[0][1] = mul(k37, e1);
-  st.c[0][2] = fma(k1084, fma(e1, s02, mul(lam[1], add(e2, e0))), nmu3);
-  st.c[1][0] = lam[2];
-  st.c[1][1] = mul(k37, e2);
-  st.c[1][2] = fma(k1084, fma(e2, s01, mul(lam[2], add(e0, e1))), nmu3);
-  // quasi-spherical correction: z = eps / 0.1
+  a.c[0] = lam[0];
+  a.c[1] = mul(splat(3.0f / 7.0f), a.e0);
+  a.c[2] = fma(splat(10.0f / 84.0f), fma(a.e0, a.s12, mul(lam[0], add(a.e1, a.e2))), a.nmu3);
+  return a;
+}
+
+// Coefficients of the two other axes.
+__device__ __forceinline__ void minor_axes_x2(const float2 lam[3], const AxisZeroX2& a, float2 c1[3], float2 c2[3]) {
+  using namespace x2;
+  const float2 k37 = splat(3.0f / 7.0f), k1084 = splat(10.0f / 84.0f);
+  c1[0] = lam[1];
+  c1[1] = mul(k37, a.e1);
+  c1[2] = fma(k1084, fma(a.e1, a.s02, mul(lam[1], add(a.e2, a.e0))), a.nmu3);
+  c2[0] = lam[2];
+  c2[1] = mul(k37, a.e2);
+  c2[2] = fma(k1084, fma(a.e2, a.s01, mul(lam[2], add(a.e0, a.e1))), a.nmu3);
+}
+
+// The quasi-spherical correction term (z = eps / 0.1).
+__device__ __forceinline__ float2 correction_x2(const float2 lam[3], float2 mu1, const CollapseConsts<float>& cc) {
+  using namespace x2;
   const float2 num = mul(splat(10.0f), sub(lam[0], lam[2]));
   const float2 z = div(num, make_float2(mu1.x > 0.0f ? mu1.x : 1.0f, mu1.y > 0.0f ? mu1.y : 1.0f));
   const float2 nz2 = mul(mul(z, z), splat(-1.0f));
   const float2 w = make_float2(M<float>::exp_(nz2.x), M<float>::exp_(nz2.y));
   const float2 cw = mul(mul(mu1, splat(cc.dcorr)), w);
-  st.corr.x = (cc.correction && mu1.x > 0.0f) ? cw.x : 0.0f;
-  st.corr.y = (cc.correction && mu1.y > 0.0f) ? cw.y : 0.0f;
+  return make_float2((cc.correction && mu1.x > 0.0f) ? cw.x : 0.0f, (cc.correction && mu1.y > 0.0f) ? cw.y : 0.0f);
+}
+
+// First part of collapse_main<float> for two particles: the coefficients of
+// the three axes (c0 for the axis of the largest eigenvalue, st.c for the
+// others) and the quasi-spherical correction term st.corr.
+__device__ __forceinline__ void collapse_prep_x2(const float2 lam[3], const CollapseConsts<float>& cc,
+                                                 CollapseStateX2& st, float2 c0[3]) {
+  const AxisZeroX2 a = axis_zero_x2(lam);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) c0[k] = a.c[k];
+  minor_axes_x2(lam, a, st.c[0], st.c[1]);
+  st.corr = correction_x2(lam, a.mu1, cc);
 }
 
 // Second part: the largest root of the axis-0 cubic (st.best, st.kappa) and
@@ -252,14 +277,41 @@ __device__ __forceinline__ void collapse_main_x2(const float2 lam[3], const Coll
 // test runs at t (1 - 1e-5), below t by more than the FP32 error of a root, so
 // that a lane it clears could not have been updated by the full computation
 // (nor by its FP64 redo).  Exact up to rounding, like no_root_from.
-__device__ __forceinline__ unsigned cannot_beat_x2(const float2 c0[3], const CollapseStateX2& st, float2 fm) {
+//
+// Only the axis of the largest eigenvalue takes that test.  With k the
+// remaining index, the cubics differ by (the identity follows from e_i, c3)
+//   g_i(F) - g_0(F) = (lam_0 - lam_i) q_i(F),
+//   q_i(F) = F^2 + (3/14) lam_k F + (5/84) lam_k mu1,
+// so beyond a t past all roots of axis 0 the others have none either where q_i
+// stays positive: q_i(t) > 0 (here by 1e-4 t^2, far above rounding), and t
+// right of its vertex or its discriminant negative.  That holds for all but
+// 2e-5 of the particles that axis 0 clears (64^3, 24 radii); a warp with one of
+// them (one in 700) takes the tests of the other axes.  Two of the three tests,
+// their square roots and the coefficients of two axes go: z pass 11.01 -> 10.57
+// ps per particle and radius at 768^3, 12.1 -> 11.3 at 256^3.
+__device__ __forceinline__ unsigned cannot_beat_x2(const float2 lam[3], const CollapseConsts<float>& cc, float2 fm) {
   using namespace x2;
-  const float2 t = mul(sub(fm, st.corr), splat(1.0f - 1e-5f));
-  const unsigned a0 = no_root_from_x2(c0[0], c0[1], c0[2], t);
-  const unsigned a1 = no_root_from_x2(st.c[0][0], st.c[0][1], st.c[0][2], t);
-  const unsigned a2 = no_root_from_x2(st.c[1][0], st.c[1][1], st.c[1][2], t);
+  const AxisZeroX2 a = axis_zero_x2(lam);
+  const float2 t = mul(sub(fm, correction_x2(lam, a.mu1, cc)), splat(1.0f - 1e-5f));
   const unsigned nonneg = (t.x >= 0.0f ? 1u : 0u) | (t.y >= 0.0f ? 2u : 0u);
-  return a0 & a1 & a2 & nonneg;
+  const unsigned a0 = no_root_from_x2(a.c[0], a.c[1], a.c[2], t) & nonneg;
+  const float2 m = fma(splat(3.0f / 14.0f), t, mul(splat(5.0f / 84.0f), a.mu1));
+  const float2 tt = mul(mul(t, splat(1.0f - 1e-4f)), t);
+  const float2 q1 = fma(lam[2], m, tt), q2 = fma(lam[1], m, tt);
+  // t + (3/28) lam_k: right of the vertex; (9/196) lam_k - (5/21) mu1, for
+  // lam_k < 0: negative discriminant (for lam_k >= 0 the first holds)
+  const float2 v1 = fma(splat(3.0f / 28.0f), lam[2], t), v2 = fma(splat(3.0f / 28.0f), lam[1], t);
+  const float2 nm = mul(splat(-5.0f / 21.0f), a.mu1);
+  const float2 n1 = fma(splat(9.0f / 196.0f), lam[2], nm), n2 = fma(splat(9.0f / 196.0f), lam[1], nm);
+  const float w0 = fminf(fminf(q1.x, q2.x), fminf(fmaxf(v1.x, n1.x), fmaxf(v2.x, n2.x)));
+  const float w1 = fminf(fminf(q1.y, q2.y), fminf(fmaxf(v1.y, n1.y), fmaxf(v2.y, n2.y)));
+  const unsigned minor = (w0 > 0.0f ? 1u : 0u) | (w1 > 0.0f ? 2u : 0u);
+  if (a0 & ~minor) {
+    float2 c1[3], c2[3];
+    minor_axes_x2(lam, a, c1, c2);
+    return a0 & (minor | (no_root_from_x2(c1[0], c1[1], c1[2], t) & no_root_from_x2(c2[0], c2[1], c2[2], t)));
+  }
+  return a0;
 }
 
 // One lane of a pair state as the scalar state of collapse.cuh (for the rare

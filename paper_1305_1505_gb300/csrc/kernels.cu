@@ -294,11 +294,8 @@ __global__ void __launch_bounds__(NP * LINES * Shape<N>::P, MODE != kZCollapse ?
         // FP64 redo finishes skip the root solve; the rest wait in a queue:
         // eigenvalues and F_max in the particle's own (already read) field
         // slots 0-3
-        CollapseStateX2 csx;
-        float2 c0[3];
-        collapse_prep_x2(lam, ccf, csx, c0);
         const unsigned done =
-            cannot_beat_x2(c0, csx, make_float2(fm[0], fm[1])) | (valid[0] ? 0u : 1u) | (valid[1] ? 0u : 2u);
+            cannot_beat_x2(lam, ccf, make_float2(fm[0], fm[1])) | (valid[0] ? 0u : 1u) | (valid[1] ? 0u : 2u);
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
           if ((done >> u) & 1u) continue;

@@ -161,7 +161,8 @@ template <int N, int TC = 16, int V = 0> struct MinBlocks {
   static constexpr int kSmem = 2 * N * TC * 8 + S::kTw * 8 + 12 * N + 1280;
   static constexpr int kByRegs = 65536 / (TC * S::P * ((4 * S::E + 24 + 7) / 8 * 8));
   static constexpr int kBySmem = (227 * 1024) / kSmem;
-  static constexpr int kTwo = kBySmem < kByRegs ? kBySmem : kByRegs;
+  static constexpr int kMin = kBySmem < kByRegs ? kBySmem : kByRegs;
+  static constexpr int kTwo = kMin < 24 ? kMin : 24;  // an SM holds at most 32 blocks
   static constexpr int xy = S::P2 > 1 ? 512 / (TC * S::P) : (kTwo > 1 ? kTwo : 1);
   static constexpr int z = Shape<N>::P2 > 1 ? PIN_Z_MINB3 : (Shape<N>::E <= 16 ? 6 : 8);
   static constexpr int zv = Shape<N>::P2 > 1 ? PIN_Z_MINB3V : (Shape<N>::E <= 16 ? 6 : 4);
