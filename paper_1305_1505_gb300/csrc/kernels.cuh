@@ -273,7 +273,7 @@ cudaError_t generate_ic(int n, double box, const uint64_t* keys_dev, double* tab
 // output may be null.  `scratch` holds fragment_scratch_bytes(N^3) bytes.
 size_t fragment_scratch_bytes(long n3);
 cudaError_t fragment_order(const float* fmax, int nx, int ny, int nz, void* scratch, int32_t* order,
-                           uint8_t* n_before, cudaStream_t st);
+                           uint8_t* n_before, int* err, cudaStream_t st);
 int fragment_kernels(bool order, bool counts);  // launches of one fragment_order call
 
 }  // namespace pin

@@ -228,14 +228,17 @@ struct WalkX {
   }
   // to the radius of `tile` (not before the current one); false past the last
   __device__ __forceinline__ bool seek(const ArgsX& a, int tile) {
-    if constexpr (!kMultiRad<N>) return tile < ntiles;
-    while (tile >= base + ntiles) {
-      if (g + 1 >= a.rad.n) return false;
-      base += ntiles;
-      ++g;
-      init(a);
+    if constexpr (kMultiRad<N>) {
+      while (tile >= base + ntiles) {
+        if (g + 1 >= a.rad.n) return false;
+        base += ntiles;
+        ++g;
+        init(a);
+      }
+      return true;
+    } else {
+      return tile < ntiles;
     }
-    return true;
   }
   __device__ __forceinline__ int col(const ArgsX& a, int t) const {  // first column of tile t of a realisation
     if (flat) return t * TC;
@@ -259,14 +262,17 @@ struct WalkY {
     ntiles = a.nx * a.batch * ktiles;
   }
   __device__ __forceinline__ bool seek(const ArgsY& a, int tile) {
-    if constexpr (!kMultiRad<N>) return tile < ntiles;
-    while (tile >= base + ntiles) {
-      if (g + 1 >= a.rad.n) return false;
-      base += ntiles;
-      ++g;
-      init(a);
+    if constexpr (kMultiRad<N>) {
+      while (tile >= base + ntiles) {
+        if (g + 1 >= a.rad.n) return false;
+        base += ntiles;
+        ++g;
+        init(a);
+      }
+      return true;
+    } else {
+      return tile < ntiles;
     }
-    return true;
   }
 };
 
@@ -303,7 +309,6 @@ __global__ void __launch_bounds__(TC* Shape<N, V>::P, MinBlocks<N, TC, V>::xy)
     mbar_init_fence();
   }
   __syncthreads();
-  const int ncols = a.ny * a.nhp;
   WalkX<N, TC, V> cur(a);
   WalkX<N, TC, V> nxt = cur;
   auto issue = [&](const WalkX<N, TC, V>& w, int tile) {

@@ -1192,19 +1192,19 @@ pin_status pin_fragment_order(pin_plan_t p, int32_t* order, uint8_t* n_before, i
   // the y-pass spectra are free once the radius loop is done: sort scratch,
   // and (for host outputs) the device copies of the results after it
   const size_t need = fragment_scratch_bytes(n3);
-  const size_t have = (size_t)(p->velocities ? 9 : 6) * p->field_elems * sizeof(float2);
-  const size_t tail = (need + 255) & ~(size_t)255;
-  if (tail + (size_t)n3 > have) return fail(p, PIN_ECUDA, "fragment scratch does not fit the plan's workspace");
+  const size_t have = v_bytes(p->field_elems, n3, p->group, p->velocities);
+  auto aligned = [](size_t x) { return (x + 255) & ~(size_t)255; };
+  const size_t at_nb = aligned(need), at_order = aligned(at_nb + (on_device ? 0 : (size_t)n3));
+  if (at_order + (on_device ? 0 : (size_t)n3 * 4) > have)
+    return fail(p, PIN_ECUDA, "fragment scratch does not fit the plan's workspace");
   char* scratch = reinterpret_cast<char*>(p->V);
   int32_t* order_dev = order;
   uint8_t* nb_dev = n_before;
   if (!on_device) {
-    // the last radix pass reads keys and values A and writes only values:
-    // the second value array is free for the order
-    if (order) order_dev = reinterpret_cast<int32_t*>(scratch + (size_t)3 * n3 * 4);
-    if (n_before) nb_dev = reinterpret_cast<uint8_t*>(scratch + tail);
+    if (order) order_dev = reinterpret_cast<int32_t*>(scratch + at_order);
+    if (n_before) nb_dev = reinterpret_cast<uint8_t*>(scratch + at_nb);
   }
-  PIN_CK(p, fragment_order(p->fmax, p->nx, p->ny, p->nz, scratch, order_dev, nb_dev, p->stream));
+  PIN_CK(p, fragment_order(p->fmax, p->nx, p->ny, p->nz, scratch, order_dev, nb_dev, p->err, p->stream));
   if (!on_device) {
     if (order) PIN_CK(p, cudaMemcpyAsync(order, order_dev, (size_t)n3 * 4, cudaMemcpyDeviceToHost, p->stream));
     if (n_before) PIN_CK(p, cudaMemcpyAsync(n_before, nb_dev, (size_t)n3, cudaMemcpyDeviceToHost, p->stream));
