@@ -150,7 +150,15 @@ __global__ void k_z64(const double2* __restrict__ half, int nx, int ny, int nz, 
     const int sx = ix < nx / 2 ? ix : ix - nx, sy = iy < ny / 2 ? iy : iy - ny;
     const bool qx = sx == -nx / 2, qy = sy == -ny / 2;
     const double kx = kfx * sx, ky = kfy * sy;
-    const double2 d = half[((size_t)ix * ny + iy) * nh + iz];
+    double2 d = half[((size_t)ix * ny + iy) * nh + iz];
+    if (iz == 0 || iz == nz / 2) {
+      // the planes that are their own mirror: the Hermitian part, whose
+      // transform is the real part of the input's (an input rounded to FP32 is
+      // Hermitian there to 1e-8 only, and the paired transform would hand the
+      // imaginary part of one component to the other)
+      const double2 m = half[((size_t)((nx - ix) % nx) * ny + (ny - iy) % ny) * nh + iz];
+      d = make_double2(0.5 * (d.x + m.x), 0.5 * (d.y - m.y));
+    }
     const double az = kfz * iz;  // |kz|
     const double k2 = kx * kx + ky * ky + az * az;
     const double g = k2 > 0.0 ? exp(-0.5 * k2 * radius * radius) / k2 : 0.0;
