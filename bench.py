@@ -96,26 +96,35 @@ class ClockSampler:
                 "samples": len(sm)}
 
 
-def algorithmic_bytes(n, fused, velocities):
-    """Bytes each pass must move per launch (one launch per radius).
-    A half-spectrum is H = N^2 (N/2+1) complex64 values (8H bytes, ~4 B per
-    particle).  x: read Phi0, write 3 spectra.  y: read 3, write 6 (+3 psi
-    spectra with velocities).  z: read those spectra; split layout: write 3
-    eigenvalue floats per particle (+3 psi floats), then the root pass reads
-    them; the running-maximum state is an F_max read plus F_max and index
-    writes, 12 B per particle (writes are an upper bound: only where F rises),
-    +12 B for the velocity state (+12 B psi read in the split layout)."""
-    H = n * n * (n // 2 + 1)
+def filter_support(n, box, radius):
+    """(modes, half_modes): along an axis of n points, the number of
+    wavenumber indices (of n, and of the n/2 + 1 of the half axis) whose
+    filter factors {W, k W, k^2 W} / n are not exactly zero in FP32."""
+    s = np.arange(n // 2 + 1, dtype=np.float64)
+    k = 2.0 * np.pi * s / box
+    w = np.exp(-0.5 * (k * radius) ** 2) / n
+    live = (w.astype(np.float32) != 0) | ((k * w).astype(np.float32) != 0) | ((k * k * w).astype(np.float32) != 0)
+    m = int(s[live].max())
+    return min(n, 2 * m + 1), m + 1
+
+
+def algorithmic_bytes(n, velocities, box, radii):
+    """Bytes each pass must move per radius, averaged over the radii.  A value
+    of a spectrum is 8 bytes; modes whose filter factors are exactly zero in
+    FP32 need not be moved by the x and y passes.  x: read Phi0 within the
+    support, write 3 spectra of its (ky, kz) columns.  y: read those, write 6
+    spectra (+3 psi with velocities) of its kz columns.  z: read every column
+    (zeros past the support) and the running maximum, write F_max and the
+    index, 12 B per particle (writes are an upper bound: only where F rises),
+    +12 B for the velocity state."""
     N3 = n ** 3
     v = 1 if velocities else 0
-    state = 12 * N3 + 12 * N3 * v
-    alg = {"x": 4 * 8 * H, "y": (9 + 3 * v) * 8 * H}
-    if fused:
-        alg["z"] = (6 + 3 * v) * 8 * H + state
-        alg["redo"] = 0
-    else:
-        alg["z"] = (6 + 3 * v) * 8 * H + 12 * N3 + 12 * N3 * v
-        alg["roots"] = 12 * N3 + 12 * N3 * v + state
+    H = n * n * (n // 2 + 1)
+    alg = {"x": 0.0, "y": 0.0, "z": (6 + 3 * v) * 8 * H + 12 * N3 + 12 * N3 * v, "redo": 0}
+    for r in radii:
+        m, h = filter_support(n, box, r)
+        alg["x"] += 8 * (m * m * h + 3 * n * m * h) / len(radii)
+        alg["y"] += 8 * (3 * n * m * h + (6 + 3 * v) * n * n * h) / len(radii)
     return alg
 
 
@@ -279,8 +288,7 @@ def measure_config(c, steps, warmup, tune=True):
         evs[i + 1].record(stream)
     torch.cuda.synchronize()
     ms = evs[0].elapsed_time(evs[-1]) / steps
-    fused = pin.pin_kernels_per_call(plan.handle) == 4 * S
-    alg = algorithmic_bytes(n, fused, False)
+    alg = algorithmic_bytes(n, False, c["box"], radii)
     peak, peak_kind = _peaks()
     step_bytes = S * sum(alg.values())
     out = {"workload": "%d^3 grid, box %.0f Mpc/h, seed %d, %d radii %.4g->%.4g Mpc/h (log)"
@@ -498,13 +506,10 @@ def run_ours(args):
     pin_schedule = pin.pin_get_schedule(plan.handle)
     radix = plan.radix()
 
-    # roofline of the dominant pass (algorithmic bytes per launch, one launch per radius)
-    fused = kernels_per_call == 4 * S
+    # roofline of the dominant pass (algorithmic bytes per radius)
     per_launch_ms = pass_ms / S
-    alg = algorithmic_bytes(n, fused, bool(args.velocities))
-    names = ["x", "y", "z", "roots"]
-    if fused:
-        names[3] = "redo"  # the z pass computes the collapse times; only the FP64 redo follows
+    alg = algorithmic_bytes(n, bool(args.velocities), w["box"], radii)
+    names = ["x", "y", "z", "redo"]
     dom = int(np.argmax(per_launch_ms))
     peak, peak_kind = _peaks()
     achieved = alg[names[dom]] / (per_launch_ms[dom] / 1e3) / 1e9
@@ -541,7 +546,7 @@ def run_ours(args):
                                                    "y": pin.pin_radix_shape(n, radix[1])},
                                   "tuned": not (args.no_tune or args.tiles or args.radix)},
                            schedule=pin_schedule),
-            "roofline": dict(roofline(names[dom], per_launch_ms[dom], n, bool(args.velocities), fused,
+            "roofline": dict(roofline(names[dom], per_launch_ms[dom], n, bool(args.velocities), True,
                                       achieved, peak, peak_kind, clocks, passes), step=whole_step),
             "cpu_baseline": cb,
             "e2e": None if args.no_e2e else {"value": updates * ws / e2e_s, "unit": UNIT,
@@ -641,11 +646,11 @@ def run_ensemble(args):
     return 0
 
 
-# bytes each particle costs the fragmentation front end: four radix passes
-# (histogram key read 4 B each; scatter: pass 0 reads F 4 B and writes key +
-# index 8 B, passes 1-2 read and write 8 B, pass 3 reads 8 B and writes the
-# index 4 B) and the neighbour count (F read 4 B, count write 1 B)
-FRAGMENT_BYTES = 4 * 4 + (4 + 8) + 2 * (8 + 8) + (8 + 4) + (4 + 1)
+# bytes each particle costs the fragmentation front end: the key range and the
+# digit counts (F read 4 B each), three radix passes (pass 0 reads F 4 B and
+# writes key + index 8 B, pass 1 reads and writes 8 B, pass 2 reads 8 B and
+# writes the index 4 B) and the neighbour count (F read 4 B, count write 1 B)
+FRAGMENT_BYTES = 2 * 4 + (4 + 8) + (8 + 8) + (8 + 4) + (4 + 1)
 
 
 def run_fragment(args):
@@ -719,7 +724,7 @@ def run_fragment(args):
                          "frac": achieved / peak, "traffic": None,
                          "alg_bytes_per_particle": FRAGMENT_BYTES},
             "cpu_baseline": cb, "e2e": e2e,
-            "gpu_launches": int(args.steps * 21), "clocks": clk.summary()}
+            "gpu_launches": int(args.steps * 10), "clocks": clk.summary()}
     print(json.dumps(line), flush=True)
     plan.close()
     return 0

@@ -557,17 +557,6 @@ static PassShape shape_of() {
                    CfgXY<N, C::TC, 0>::threads, C::threads_z};
 }
 
-// Blocks of a z-pass launch resident on the device at once: the distance of
-// its L2 prefetch.
-template <class K>
-static int resident_blocks(K kernel, int threads, size_t smem) {
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
-  return std::max(1, sms) * std::max(1, per_sm);
-}
-
 template <int N>
 static cudaError_t run_z(const ArgsZ& a_in, bool dump, cudaStream_t st) {
   using C = Cfg<N>;
@@ -575,8 +564,8 @@ static cudaError_t run_z(const ArgsZ& a_in, bool dump, cudaStream_t st) {
   const long nlines = a.nlines;
   // one wave ahead: measured best against none and two waves (384^3 z pass
   // 0.80 -> 0.76 ms, 768^3 5.93 -> 5.89 ms per radius)
-  static const int wave = resident_blocks(k_pass_z<N, C::LINES, 3, kZCollapse>, C::threads_z, C::smem_z);
-  if (!dump && a.nfields <= 6) a.prefetch_blocks = wave;
+  if (!dump && a.nfields <= 6)
+    a.prefetch_blocks = (int)resident<k_pass_z<N, C::LINES, 3, kZCollapse>>(C::threads_z, C::smem_z);
   if (!dump && a.nfields > 6) {
     const unsigned grid = (unsigned)((nlines + C::LINES_V - 1) / C::LINES_V);
     k_pass_z<N, C::LINES_V, 5, kZCollapse><<<grid, C::threads_zv, C::smem_zv, st>>>(a);

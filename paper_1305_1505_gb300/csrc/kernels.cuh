@@ -157,7 +157,7 @@ struct ArgsZ {
   float tau_root;  // FP64 redo when kappa < tau_root
   unsigned long long* counters;  // [0] eigen redo, [1] root redo, [2] list overflow
   RedoEntry* redo_list;          // FP64 redo queue of this radius
-  unsigned* redo_count;          // zeroed before the z pass
+  unsigned* redo_count;          // zero before the z pass; one per radius of the call
   unsigned redo_cap;
   // dump mode
   float* out[kMaxFields];

@@ -46,29 +46,30 @@ constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 constexpr size_t spec_bytes(int n) { return (size_t)n * n * ((n / 2 + 1 + 3) & ~3) * sizeof(float2); }
 
 // Where things lie in the workspace for grids of n points a side and groups of
-// `group` radii (RadGroup): Phi0, U and V, the running maximum of a group, the
-// tables, {counters, queue counts, error word, the word that turns the bands
-// off} (cleared by every call), the redo queues.
+// `group` radii (RadGroup): Phi0, U and V; the tables {twiddles, bands,
+// multipliers}, copied in as one piece; {counters, queue counts, error word,
+// the word that turns the bands off, the running maximum of a group}, cleared
+// as one; the redo queues.
 struct Layout {
   int group;
   size_t cap;  // redo entries per radius
-  size_t phi0, U, V, state, mult, band, tw, cnt, redo_count, err, wide, redo, end;
+  size_t phi0, U, V, tw, band, mult, cnt, redo_count, err, wide, state, redo, end;
   constexpr Layout(int n, int g)
-      : group(g), cap(), phi0(), U(), V(), state(), mult(), band(), tw(), cnt(), redo_count(), err(), wide(), redo(),
+      : group(g), cap(), phi0(), U(), V(), tw(), band(), mult(), cnt(), redo_count(), err(), wide(), state(), redo(),
         end() {
     const size_t n3 = (size_t)n * n * n;
     cap = g > 1 && n3 < kRedoCap ? n3 : kRedoCap;
     U = spec_bytes(n);
     V = U + 3 * spec_bytes(n) * g;
-    state = V + 6 * spec_bytes(n) * g;
-    mult = state + (g > 1 ? n3 * 8 : 0);
-    band = mult + (size_t)kMaxScales * 3 * n * sizeof(float);
-    tw = band + (size_t)kMaxScales * 4 * sizeof(int);
-    cnt = tw + (size_t)n * sizeof(float2);
+    tw = V + 6 * spec_bytes(n) * g;
+    band = tw + (size_t)n * sizeof(float2);
+    mult = band + (size_t)kMaxScales * 4 * sizeof(int);
+    cnt = mult + (size_t)kMaxScales * 3 * n * sizeof(float);
     redo_count = cnt + 4 * sizeof(unsigned long long);
-    err = redo_count + pin::kMaxGroup * sizeof(unsigned);
+    err = redo_count + kMaxScales * sizeof(unsigned);
     wide = err + 8;
-    redo = align256(err + 16);
+    state = wide + 8;
+    redo = align256(state + (g > 1 ? n3 * 8 : 0));
     end = align256(redo + cap * g * sizeof(pin::RedoEntry));
   }
 };
@@ -95,9 +96,12 @@ size_t g_last_err[kMaxDevices] = {};
 // Host staging of the tables (filled and copied under g_stage_mu; a copy from
 // pageable host memory has consumed its source when cudaMemcpyAsync returns).
 std::mutex g_stage_mu;
-float g_h_mult[(size_t)kMaxScales * 3 * kMaxN];
-int g_h_band[kMaxScales * 4];
-float2 g_h_tw[kMaxN];
+struct Tables {  // as Layout places them (the twiddles end where the bands begin)
+  float2 tw[kMaxN];
+  int band[kMaxScales * 4];
+  float mult[(size_t)kMaxScales * 3 * kMaxN];
+};
+Tables g_h_tables;
 
 // Once per device, with that device current: the scratch address, the
 // constant twiddle tables and the kernels' shared-memory limits.
@@ -174,24 +178,21 @@ extern "C" pin_status pin_collapse_times_noalloc(const void* delta_k, int dtype,
   {
     // per radius [3][n] multipliers (cubic grid: one table serves all axes)
     std::lock_guard<std::mutex> lk(g_stage_mu);
+    float2* h_tw = g_h_tables.tw + (kMaxN - n);
     for (int s = 0; s < nscales; ++s) {
-      float* m = g_h_mult + (size_t)s * 3 * n;
+      float* m = g_h_tables.mult + (size_t)s * 3 * n;
       pin::fill_mult(m, n, box, radii[s]);
-      pin::fill_band(g_h_band + 4 * s, m, n, m, n, m, n, nhp);
+      pin::fill_band(g_h_tables.band + 4 * s, m, n, m, n, m, n, nhp);
     }
-    pin::fill_twiddles(g_h_tw, n, sh);
-    if (cudaMemcpyAsync(mult, g_h_mult, (size_t)nscales * 3 * n * sizeof(float), cudaMemcpyHostToDevice, cs) !=
-            cudaSuccess ||
-        cudaMemcpyAsync(band, g_h_band, (size_t)nscales * 4 * sizeof(int), cudaMemcpyHostToDevice, cs) !=
-            cudaSuccess ||
-        cudaMemcpyAsync(tw, g_h_tw, (size_t)n * sizeof(float2), cudaMemcpyHostToDevice, cs) != cudaSuccess)
+    pin::fill_twiddles(h_tw, n, sh);
+    if (cudaMemcpyAsync(tw, h_tw, at.mult - at.tw + (size_t)nscales * 3 * n * sizeof(float), cudaMemcpyHostToDevice,
+                        cs) != cudaSuccess)
       return PIN_ECUDA;
   }
-  if (cudaMemsetAsync(cnt, 0, at.err + 16 - at.cnt, cs) != cudaSuccess ||
+  if (cudaMemsetAsync(cnt, 0, at.state - at.cnt + (state ? n3 * sizeof(*state) : 0), cs) != cudaSuccess ||
       pin::launch_load_phi0(delta_k, dtype, n, n, n, nhp, box, 1, phi0, wide, cs) != cudaSuccess ||
-      (state ? cudaMemsetAsync(state, 0, n3 * sizeof(*state), cs) != cudaSuccess
-             : cudaMemsetAsync(F_max, 0, n3 * sizeof(float), cs) != cudaSuccess ||
-                   cudaMemsetAsync(scale_idx, 0xFF, n3 * sizeof(int32_t), cs) != cudaSuccess))
+      (!state && (cudaMemsetAsync(F_max, 0, n3 * sizeof(float), cs) != cudaSuccess ||
+                  cudaMemsetAsync(scale_idx, 0xFF, n3 * sizeof(int32_t), cs) != cudaSuccess)))
     return PIN_ECUDA;
 
   static const int vout[6] = {0, 3, 4, 1, 2, 5};
@@ -271,10 +272,9 @@ extern "C" pin_status pin_collapse_times_noalloc(const void* delta_k, int dtype,
     az.tau_root = 1e-3f;
     az.counters = cnt;
     az.redo_list = redo_list;
-    az.redo_count = redo_count;
+    az.redo_count = redo_count + k;
     az.redo_cap = (unsigned)at.cap;
     if (pin::launch_x(n, tc, 0, ax, cs) != cudaSuccess || pin::launch_y(n, tc, 0, ay, cs) != cudaSuccess ||
-        cudaMemsetAsync(redo_count, 0, rad.n * sizeof(unsigned), cs) != cudaSuccess ||
         pin::launch_z(n, az, false, cs) != cudaSuccess ||
         pin::launch_redo(az, cs) != cudaSuccess)
       return PIN_ECUDA;

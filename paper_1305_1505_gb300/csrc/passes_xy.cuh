@@ -625,16 +625,23 @@ static cudaError_t set_attrs_xy_all() {
   return e;
 }
 
-// Persistent grid: as many blocks as fit on the device at once, at most one
-// per tile.
-template <class K>
-static unsigned persistent_grid(K kernel, int threads, size_t smem, long ntiles) {
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
-  long g = (long)std::max(1, sms) * std::max(1, per_sm);
-  return (unsigned)std::min<long>(g, std::max<long>(1, ntiles));
+// Blocks of a kernel resident on the device at once (asked once per kernel and
+// process: every device the library runs on is a GB300).
+template <auto Kernel>
+static long resident(int threads, size_t smem) {
+  static const long r = [&] {
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, Kernel, threads, smem);
+    return (long)std::max(1, sms) * std::max(1, per_sm);
+  }();
+  return r;
+}
+// Persistent grid: as many blocks as fit on the device, at most one per tile.
+template <auto Kernel>
+static unsigned persistent_grid(int threads, size_t smem, long ntiles) {
+  return (unsigned)std::min<long>(resident<Kernel>(threads, smem), std::max<long>(1, ntiles));
 }
 
 template <int N, int TC, int V>
@@ -649,7 +656,7 @@ static cudaError_t run_x(const ArgsX& a_in, cudaStream_t st) {
     if (e != cudaSuccess) return e;
   }
   const long ntiles = (((long)a.ny * a.nhp + TC - 1) / TC) * a.batch * a.rad.n;
-  const unsigned grid = persistent_grid(k_pass_x<N, TC, V>, C::threads, C::smem, ntiles);
+  const unsigned grid = persistent_grid<k_pass_x<N, TC, V>>(C::threads, C::smem, ntiles);
   k_pass_x<N, TC, V><<<grid, C::threads, C::smem, st>>>(a);
   return cudaGetLastError();
 }
@@ -669,11 +676,11 @@ static cudaError_t run_y(const ArgsY& a, cudaStream_t st) {
                                            TC, Store<N>::kRows);
       if (e != cudaSuccess) return e;
     }
-    const unsigned grid = persistent_grid(k_pass_y<N, TC, false, V>, C::threads, C::smem, ntiles);
+    const unsigned grid = persistent_grid<k_pass_y<N, TC, false, V>>(C::threads, C::smem, ntiles);
     k_pass_y<N, TC, false, V><<<grid, C::threads, C::smem, st>>>(b);
     return cudaGetLastError();
   }
-  const unsigned grid = persistent_grid(k_pass_y<N, TC, true, V>, C::threads, C::smem, ntiles);
+  const unsigned grid = persistent_grid<k_pass_y<N, TC, true, V>>(C::threads, C::smem, ntiles);
   k_pass_y<N, TC, true, V><<<grid, C::threads, C::smem, st>>>(a);
   return cudaGetLastError();
 }

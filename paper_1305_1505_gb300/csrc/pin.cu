@@ -61,7 +61,7 @@ struct pin_plan_s {
   float2* tw = nullptr;
   unsigned long long* counters = nullptr;  // [0] eig redo, [1] root redo, [2] queue overflow
   RedoEntry* redo_list = nullptr;          // FP64 redo queue, reused by every radius
-  unsigned* redo_count = nullptr;
+  unsigned* redo_count = nullptr;          // entries queued by each radius of the loop, cleared per call
   unsigned redo_cap = 0;
   int* err = nullptr;                      // set by a pass whose bounded TMA wait gave up
   long long wait_cycles = 0;               // TMA wait budget of the x/y passes (0: default)
@@ -437,7 +437,7 @@ size_t footprint(int nx, int ny, int nz, int nscales, int batch, bool velocities
          v_bytes(spec, n3, group, velocities) + n3 * 8 + (velocities ? n3 * 24 : 0) +
          (size_t)(kMaxScales + 1) * 3 * (nx + ny + nz) * 4 + kBandInts * sizeof(int) +
          (size_t)(nx + ny + nz + 3 * 64) * 8 + 64 + cap * group * sizeof(RedoEntry) +
-         kMaxGroup * sizeof(unsigned) + 16 + sizeof(int);
+         kMaxScales * sizeof(unsigned) + 16 + sizeof(int);
 }
 
 pin_status ensure_device_init(pin_plan_t p) {
@@ -649,26 +649,43 @@ ArgsY radius_args_y(pin_plan_t p, const RadGroup& rad, bool collapse, float2* vb
 // The serial loop of a captured call runs the redo on a stream of its own
 // (rs), beside the x and y passes of the next radius: 25 us of FP64 latency
 // for a few thousand particles.  It has to be over before the next z pass,
-// which refills its queue and updates the same particles: z_wait, recorded as
-// redo_done after the redo; z_end marks the end of the z pass for rs.
+// which refills its queue and updates the same particles (redo_done); z_end
+// marks the end of the z pass for rs.  It is captured after those x and y
+// passes, so that they are not launched behind it.
 struct RadiusSched {
   cudaStream_t xs, zs;
   float2* vbuf;
   cudaEvent_t y_wait, y_done, z_done;
   cudaStream_t rs = nullptr;
-  cudaEvent_t z_wait = nullptr, z_end = nullptr, redo_done = nullptr;
+  cudaEvent_t z_end = nullptr, redo_done = nullptr;
+  ArgsZ redo{};         // the redo to run after the next y pass is queued
+  int redo_scale = -1;  // its profile slot; -1: none
 };
+
+// The redo held back by the last radius, on its branch; the z stream waits.
+pin_status enqueue_redo(pin_plan_t p, RadiusSched& rs) {
+  PIN_CK(p, cudaStreamWaitEvent(rs.rs, rs.z_end, 0));
+  PIN_CK(p, launch_redo(rs.redo, rs.rs));
+  if (p->profile && !p->events.empty())
+    PIN_CK(p, cudaEventRecordWithFlags(p->events[7 * rs.redo_scale + 6], rs.rs, cudaEventRecordExternal));
+  PIN_CK(p, cudaEventRecord(rs.redo_done, rs.rs));
+  PIN_CK(p, cudaStreamWaitEvent(rs.zs, rs.redo_done, 0));
+  rs.redo_scale = -1;
+  return PIN_OK;
+}
 
 // Filter-and-transform passes of a group of radii (one, unless the plan runs
 // groups and this is the collapse loop), ending in the collapse update (dump
 // and source null), a dump of the six real components, or the 2LPT source
 // field S of every particle (source, batch 1).  A multiplier set is the index
-// of its radius.
+// of its radius; k0 is the place of the first radius in the loop, and of the
+// counter of its redo queue.
 pin_status enqueue_radii(pin_plan_t p, const RadGroup& rad, float* const* dump, float* source = nullptr,
-                         const RadiusSched* sched = nullptr) {
+                         RadiusSched* sched = nullptr, int k0 = 0) {
   const bool collapse = dump == nullptr && source == nullptr;
   const int scale = rad.ms[0];
-  const RadiusSched rs = sched ? *sched : RadiusSched{p->stream, p->stream, p->V, nullptr, nullptr, nullptr};
+  RadiusSched plain{p->stream, p->stream, p->V, nullptr, nullptr, nullptr};
+  RadiusSched& rs = sched ? *sched : plain;
   const bool rec = p->profile && collapse && !p->events.empty();
   auto mark = [&](int k, cudaStream_t st) {
     return rec ? cudaEventRecordWithFlags(p->events[7 * scale + k], st, cudaEventRecordExternal) : cudaSuccess;
@@ -688,6 +705,10 @@ pin_status enqueue_radii(pin_plan_t p, const RadGroup& rad, float* const* dump, 
     PIN_CK(p, cudaStreamWaitEvent(rs.zs, rs.y_done, 0));
   }
 
+  if (rs.redo_scale >= 0) {
+    pin_status st = enqueue_redo(p, rs);
+    if (st != PIN_OK) return st;
+  }
   ArgsZ az{};
   const int nf = (p->velocities && collapse) ? 9 : 6;
   for (int f = 0; f < nf; ++f) az.src[f] = spec(p, rs.vbuf, f);
@@ -714,7 +735,7 @@ pin_status enqueue_radii(pin_plan_t p, const RadGroup& rad, float* const* dump, 
   az.tau_root = 1e-3f;
   az.counters = p->counters;
   az.redo_list = p->redo_list;
-  az.redo_count = p->redo_count;
+  az.redo_count = p->redo_count + (collapse ? k0 : 0);
   az.redo_cap = p->redo_cap;
   if (dump)
     for (int f = 0; f < 6; ++f) az.out[f] = dump[f];
@@ -723,20 +744,17 @@ pin_status enqueue_radii(pin_plan_t p, const RadGroup& rad, float* const* dump, 
     PIN_CK(p, launch_z_source(p->nz, az, rs.zs));
     return PIN_OK;
   }
-  if (rs.z_wait) PIN_CK(p, cudaStreamWaitEvent(rs.zs, rs.z_wait, 0));
   PIN_CK(p, mark(4, rs.zs));
-  if (!dump) PIN_CK(p, cudaMemsetAsync(p->redo_count, 0, rad.n * sizeof(unsigned), rs.zs));
   PIN_CK(p, launch_z(p->nz, az, dump != nullptr, rs.zs));
   PIN_CK(p, mark(5, rs.zs));
-  cudaStream_t redo_stream = rs.zs;
-  if (rs.rs) {
-    redo_stream = rs.rs;
+  if (rs.rs && !dump) {
     PIN_CK(p, cudaEventRecord(rs.z_end, rs.zs));
-    PIN_CK(p, cudaStreamWaitEvent(rs.rs, rs.z_end, 0));
+    rs.redo = az;
+    rs.redo_scale = scale;
+    return PIN_OK;
   }
-  if (!dump) PIN_CK(p, launch_redo(az, redo_stream));
-  PIN_CK(p, mark(6, redo_stream));
-  if (rs.rs) PIN_CK(p, cudaEventRecord(rs.redo_done, rs.rs));
+  if (!dump) PIN_CK(p, launch_redo(az, rs.zs));
+  PIN_CK(p, mark(6, rs.zs));
   if (rs.z_done) PIN_CK(p, cudaEventRecord(rs.z_done, rs.zs));
   return PIN_OK;
 }
@@ -751,17 +769,15 @@ pin_status enqueue_collapse(pin_plan_t p) {
   const int* order = p->order.data();
   // the serial loop, in groups of `group` radii
   auto serial = [&](int group) -> pin_status {
-    RadiusSched rs{p->stream, p->stream, p->V, nullptr, nullptr, nullptr, p->s_redo, nullptr, p->redo_ev[0],
-                   p->redo_ev[1]};
+    RadiusSched rs{p->stream, p->stream, p->V, nullptr, nullptr, nullptr, p->s_redo, p->redo_ev[0], p->redo_ev[1]};
     for (int k = 0; k < p->nscales; k += group) {
       pin_status st =
-          enqueue_radii(p, p->radii_of(order, k, std::min(group, p->nscales - k), group), nullptr, nullptr, &rs);
+          enqueue_radii(p, p->radii_of(order, k, std::min(group, p->nscales - k), group), nullptr, nullptr, &rs, k);
       if (st != PIN_OK) return st;
-      rs.z_wait = rs.redo_done;
     }
-    PIN_CK(p, cudaStreamWaitEvent(p->stream, rs.redo_done, 0));
-    return PIN_OK;
+    return enqueue_redo(p, rs);
   };
+  PIN_CK(p, cudaMemsetAsync(p->redo_count, 0, kMaxScales * sizeof(unsigned), p->stream));
   if (p->group > 1) {
     PIN_CK(p, cudaMemsetAsync(p->state, 0, n3 * sizeof(*p->state), p->stream));
     pin_status st = serial(p->even_group());
@@ -785,10 +801,10 @@ pin_status enqueue_collapse(pin_plan_t p) {
   PIN_CK(p, cudaStreamWaitEvent(p->s_xy, p->cap_ev[0], 0));
   PIN_CK(p, cudaStreamWaitEvent(p->s_z, p->cap_ev[0], 0));
   for (int k = 0; k < p->nscales; ++k) {
-    const RadiusSched rs{p->s_xy, p->s_z, (nbuf == 2 && (k & 1)) ? p->V2 : p->V,
+    RadiusSched rs{p->s_xy, p->s_z, (nbuf == 2 && (k & 1)) ? p->V2 : p->V,
                          k >= nbuf ? p->cap_ev[2 + 2 * (k - nbuf)] : nullptr, p->cap_ev[1 + 2 * k],
                          p->cap_ev[2 + 2 * k]};
-    pin_status st = enqueue_radii(p, p->radii_of(order, k, 1, nbuf), nullptr, nullptr, &rs);
+    pin_status st = enqueue_radii(p, p->radii_of(order, k, 1, nbuf), nullptr, nullptr, &rs, k);
     if (st != PIN_OK) return st;
   }
   // join: the plan's stream continues after the last redo and the last y pass
@@ -1016,7 +1032,7 @@ pin_status pin_plan(pin_plan_t* out, const pin_plan_desc* d) {
       A(&p->mult, mult_elems * 4 + kBandInts * sizeof(int)) != cudaSuccess || A(&p->tw, tw_elems * 8) != cudaSuccess ||
       A(&p->counters, 3 * sizeof(unsigned long long)) != cudaSuccess ||
       A(&p->redo_list, (size_t)p->redo_cap * p->group * sizeof(RedoEntry)) != cudaSuccess ||
-      A(&p->redo_count, kMaxGroup * sizeof(unsigned)) != cudaSuccess || A(&p->err, sizeof(int)) != cudaSuccess ||
+      A(&p->redo_count, kMaxScales * sizeof(unsigned)) != cudaSuccess || A(&p->err, sizeof(int)) != cudaSuccess ||
       (p->precision == PIN_FP64 &&
        (A(&p->d64, (size_t)p->nx * p->ny * (p->nz / 2 + 1) * 16) != cudaSuccess ||
         A(&p->w64, n3 * 16) != cudaSuccess || A(&p->h64, 6 * n3 * 8) != cudaSuccess ||
