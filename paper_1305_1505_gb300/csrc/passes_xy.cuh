@@ -143,12 +143,13 @@ __device__ __forceinline__ BoxRange boxes_of(int b) {
 // for more resident blocks (one line per block, 96 threads, nine blocks per
 // SM at 72 registers: measured against four 192-thread blocks at 80
 // registers, 768^3 z pass 5.21 -> 4.90 ms per radius); with the velocity
-// fields (five transforms per line, 160 threads) four blocks.
+// fields (five transforms per line, 160 threads) five blocks (384^3 x 10: three
+// 17.4, four 15.5, five 14.8, six 15.3 ms a call).
 #ifndef PIN_Z_MINB3
 #define PIN_Z_MINB3 9
 #endif
 #ifndef PIN_Z_MINB3V
-#define PIN_Z_MINB3V 4
+#define PIN_Z_MINB3V 5
 #endif
 template <int N, int TC = 16, int V = 0> struct MinBlocks {
   using S = Shape<N, V>;
