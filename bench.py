@@ -139,8 +139,8 @@ def algorithmic_bytes(n, velocities, box, radii):
 TRAFFIC_SOURCES = ["kernels.cu", "kernels_v1.cu", "passes_xy.cuh", "kernels.cuh", "fft.cuh", "packed.cuh",
                    "collapse.cuh", "collapse_x2.cuh", "pin.cu"]
 MEASURED_TRAFFIC = {
-    # profiles/z_pass_instruction_mix_384.md
-    ("k_pass_z", 768, False): {"sources": "3f2b757b0f7242b0", "bytes_per_particle": 30.239, "warp_inst_per_particle": 9.6018,
+    # profiles/passes_384x40.md
+    ("k_pass_z", 768, False): {"sources": "ea2f3cdb66fee8fc", "bytes_per_particle": 30.241, "warp_inst_per_particle": 8.9705,
                                "measured_at": "384^3 x 40, the 40 launches of one step, scaled by particles"},
 }
 
@@ -647,9 +647,10 @@ def run_ensemble(args):
 
 
 # bytes each particle costs the fragmentation front end: the key range and the
-# digit counts (F read 4 B each), three radix passes (pass 0 reads F 4 B and
-# writes key + index 8 B, pass 1 reads and writes 8 B, pass 2 reads 8 B and
-# writes the index 4 B) and the neighbour count (F read 4 B, count write 1 B)
+# digit counts (F read 4 B each), three radix passes, which 27 bits of key
+# range take (pass 0 reads F 4 B and writes key + index 8 B, pass 1 reads and
+# writes 8 B, pass 2 reads 8 B and writes the index 4 B; a wider range takes a
+# fourth) and the neighbour count (F read 4 B, count write 1 B)
 FRAGMENT_BYTES = 2 * 4 + (4 + 8) + (8 + 8) + (8 + 4) + (4 + 1)
 
 
