@@ -183,12 +183,13 @@ void fill_band(int* band4, const float* mx, int nx, const float* my, int ny, con
   const float* m[3] = {mx, my, mz};
   const int n[3] = {nx, ny, nz};
   for (int a = 0; a < 3; ++a) {
-    band4[a] = 0;
-    for (int i = 0; i < n[a]; ++i) {
-      const int s = i < n[a] / 2 ? i : n[a] - i;
-      for (int k = 0; k < 3; ++k)
-        if (m[a][(size_t)k * n[a] + i] != 0.0f) band4[a] = std::max(band4[a], s);
-    }
+    // from the Nyquist index down to the first with a non-zero factor
+    const float* w = m[a];
+    const int len = n[a];
+    int i = len / 2;
+    auto live = [&](int at) { return w[at] != 0.0f || w[len + at] != 0.0f || w[2 * len + at] != 0.0f; };
+    while (i > 0 && !live(i) && !live(len - i)) --i;
+    band4[a] = i;
   }
   if (band4[2] == nz / 2) band4[2] = nhp - 1;
   band4[3] = 0;
@@ -1042,13 +1043,13 @@ pin_status pin_plan(pin_plan_t* out, const pin_plan_desc* d) {
   }
   p->band = reinterpret_cast<int*>(p->mult + mult_elems);
   if (p->group > 1) p->state = reinterpret_cast<unsigned long long*>(p->V + 6 * p->group * p->field_elems);
-  const std::vector<float> mult = mult_table(p);
+  std::vector<float> mult = mult_table(p);
   const std::vector<int> band = band_table(p, mult);
+  mult.resize(mult_elems + kBandInts, 0.0f);  // the bands follow the factors
+  std::memcpy(mult.data() + mult_elems, band.data(), band.size() * sizeof(int));
   std::vector<float2> tw(tw_elems);
   for (int a = 0; a < 3; ++a) fill_twiddles(tw.data() + p->tw_off[a], ns[a], *shapes[a]);
-  if (cudaMemcpy(p->mult, mult.data(), mult_elems * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemset(p->band, 0, kBandInts * sizeof(int)) != cudaSuccess ||
-      cudaMemcpy(p->band, band.data(), band.size() * sizeof(int), cudaMemcpyHostToDevice) != cudaSuccess ||
+  if (cudaMemcpy(p->mult, mult.data(), mult.size() * 4, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(p->tw, tw.data(), tw.size() * 8, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemset(p->counters, 0, 3 * sizeof(unsigned long long)) != cudaSuccess ||
       cudaMemset(p->err, 0, sizeof(int)) != cudaSuccess)
