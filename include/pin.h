@@ -292,8 +292,9 @@ int pin_get_schedule(pin_plan_t p);
  * counterpart; its code is an MPI job).
  *
  * pin_set_wait_budget: the budget, in SM clock cycles, of each bounded wait of
- * the x and y passes for a staged transfer (0: the default, 2^31 cycles, about
- * a second).  A block whose wait runs out waits once more, with the default
+ * the x and y passes for a staged transfer, and (to about a thousand cycles)
+ * of pin_fragment_order's blocks for the counts of earlier ones (0: the
+ * default, 2^31 cycles, about a second).  A block whose wait runs out waits once more, with the default
  * budget, for its transfers in flight, sets the plan's error word and returns;
  * the next pin_sync (or host-output call) reports PIN_ECUDA once ("results are
  * invalid") and clears the word, so the plan stays usable.  A tiny budget

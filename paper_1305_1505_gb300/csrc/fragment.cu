@@ -155,10 +155,12 @@ __global__ void __launch_bounds__(kThreads) k_sort_base(Sort* s) {
 // Published count of a tile's digit: nothing yet, its own count, or the count
 // of it and all earlier tiles.
 constexpr unsigned kOwn = 1u << 30, kAll = 2u << 30, kCount = kOwn - 1;  // n3 <= 768^3 < 2^30
-// Polls of an earlier tile's count before a block gives up (about a second).
-// The tiles are handed out in order by a ticket, so every tile waited for is
-// running or done and publishes without waiting for a later one.
+// Polls of an earlier tile's count before a block gives up: a poll takes about
+// a thousand clocks, so the default is about a second.  The tiles are handed
+// out in order by a ticket, so every tile waited for is running or done and
+// publishes without waiting for a later one.
 constexpr int kPolls = 1 << 21;
+constexpr int kPollCycles = 1 << 10;
 constexpr int kWindow = 8;
 constexpr int kCrowd = 6;  // lanes that lost their slot: 3 to 12 made no difference
 
@@ -194,9 +196,9 @@ __device__ __forceinline__ unsigned same_digit(unsigned d, int lane, uint8_t* sl
 __global__ void __launch_bounds__(kThreads, 2) k_sort_pass(const float* __restrict__ fmax, const unsigned* keys_a,
                                                            const unsigned* vals_a, unsigned* keys_b, unsigned* vals_b,
                                                            unsigned* order, int n, int pass, Sort* s,
-                                                           unsigned* status, int* err) {
+                                                           unsigned* status, int max_polls, int* err) {
   const int passes = s->passes;
-  if (pass >= passes || *(volatile int*)err) return;
+  if (pass >= passes) return;
   extern __shared__ unsigned smem[];
   unsigned* s_k = smem;                                             // [kTile]
   unsigned* s_v = smem + kTile;                                     // [kTile]
@@ -212,8 +214,14 @@ __global__ void __launch_bounds__(kThreads, 2) k_sort_pass(const float* __restri
   const unsigned ntiles = (unsigned)((n + kTile - 1) / kTile);
   volatile unsigned* st = status + (size_t)pass * ntiles * kBins + tid;
   unsigned* out = last ? order : vals_b;
+  // Nothing to do after a failed wait, whose outputs are incomplete.  Another
+  // block may set the word while this one starts, so one thread reads it and
+  // the block leaves by the tile that it broadcasts, all threads or none: a
+  // block that lost some of its warps here would rank with counts that were
+  // never cleared and write out of range.
+  const bool failed = tid == 0 && *(volatile int*)err != 0;
   for (;;) {
-    if (tid == 0) s_tile = atomicAdd(&s->ticket[pass], 1u);
+    if (tid == 0) s_tile = failed ? ntiles : atomicAdd(&s->ticket[pass], 1u);
     for (int j = lane; j < kBins; j += 32) s_cnt[w][j] = 0;
     __syncthreads();
     const unsigned tile = s_tile;
@@ -291,7 +299,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_sort_pass(const float* __restri
       }
       if (all) break;
       t -= seen;
-      if (seen == 0 && ++polls > kPolls) {
+      if (seen == 0 && ++polls > max_polls) {
         gave_up = true;
         break;
       }
@@ -377,7 +385,7 @@ static size_t status_bytes(long n3) {
 size_t fragment_scratch_bytes(long n3) { return (size_t)n3 * 16 + status_bytes(n3) + sizeof(Sort) + 512; }
 
 cudaError_t fragment_order(const float* fmax, int nx, int ny, int nz, void* scratch, int32_t* order,
-                           uint8_t* n_before, int* err, cudaStream_t st) {
+                           uint8_t* n_before, long long wait_cycles, int* err, cudaStream_t st) {
   const long n3 = (long)nx * ny * nz;
   if (n_before) {
     k_neighbours_before<<<(unsigned)std::min<long>((n3 / 4 + 255) / 256, 152 * 64), 256, 0, st>>>(fmax, nx, ny, nz,
@@ -391,6 +399,7 @@ cudaError_t fragment_order(const float* fmax, int nx, int ny, int nz, void* scra
   unsigned* status = vb + n3;
   Sort* s = reinterpret_cast<Sort*>(((uintptr_t)status + status_bytes(n3) + 255) & ~(uintptr_t)255);
   const unsigned ntiles = (unsigned)((n3 + kTile - 1) / kTile);
+  const int max_polls = wait_cycles > 0 ? (int)std::min<long long>(wait_cycles / kPollCycles, kPolls) : kPolls;
   cudaError_t e = cudaFuncSetAttribute(k_sort_pass, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPassSmem);
   if (e == cudaSuccess && ntiles > 1) e = cudaMemsetAsync(status, 0, status_bytes(n3), st);
   if (e != cudaSuccess) return e;
@@ -402,7 +411,8 @@ cudaError_t fragment_order(const float* fmax, int nx, int ny, int nz, void* scra
   for (int p = 0; p < kPasses; ++p) {
     const bool odd = p & 1;  // pass 0 writes A, 1 reads A and writes B, ...
     k_sort_pass<<<std::min(ntiles, 2u * 152u), kThreads, kPassSmem, st>>>(fmax, odd ? ka : kb, odd ? va : vb, odd ? kb : ka, odd ? vb : va,
-                                                     reinterpret_cast<unsigned*>(order), (int)n3, p, s, status, err);
+                                                     reinterpret_cast<unsigned*>(order), (int)n3, p, s, status,
+                                                     max_polls, err);
   }
   return cudaGetLastError();
 }

@@ -270,10 +270,12 @@ cudaError_t generate_ic(int n, double box, const uint64_t* keys_dev, double* tab
 // Fragmentation front end (fragment.cu): the particles of one nx*ny*nz grid in
 // descending F_max (ties: ascending index) into `order`, and the number of
 // their six periodic neighbours that precede them into `n_before`; either
-// output may be null.  `scratch` holds fragment_scratch_bytes(N^3) bytes.
+// output may be null.  `scratch` holds fragment_scratch_bytes(N^3) bytes.  A
+// block whose wait for an earlier one runs out (wait_cycles as in ArgsX) sets
+// *err.
 size_t fragment_scratch_bytes(long n3);
 cudaError_t fragment_order(const float* fmax, int nx, int ny, int nz, void* scratch, int32_t* order,
-                           uint8_t* n_before, int* err, cudaStream_t st);
+                           uint8_t* n_before, long long wait_cycles, int* err, cudaStream_t st);
 int fragment_kernels(bool order, bool counts);  // launches of one fragment_order call
 
 }  // namespace pin

@@ -1221,7 +1221,8 @@ pin_status pin_fragment_order(pin_plan_t p, int32_t* order, uint8_t* n_before, i
     if (order) order_dev = reinterpret_cast<int32_t*>(scratch + at_order);
     if (n_before) nb_dev = reinterpret_cast<uint8_t*>(scratch + at_nb);
   }
-  PIN_CK(p, fragment_order(p->fmax, p->nx, p->ny, p->nz, scratch, order_dev, nb_dev, p->err, p->stream));
+  PIN_CK(p, fragment_order(p->fmax, p->nx, p->ny, p->nz, scratch, order_dev, nb_dev, p->wait_cycles, p->err,
+                           p->stream));
   if (!on_device) {
     if (order) PIN_CK(p, cudaMemcpyAsync(order, order_dev, (size_t)n3 * 4, cudaMemcpyDeviceToHost, p->stream));
     if (n_before) PIN_CK(p, cudaMemcpyAsync(n_before, nb_dev, (size_t)n3, cudaMemcpyDeviceToHost, p->stream));
