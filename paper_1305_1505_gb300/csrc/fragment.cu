@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_sort_pass(const float* __restri
 #pragma unroll
     for (int i = 0; i < kItems; ++i) s_v[pos[i]] = val[i];
     if (__syncthreads_or(gave_up)) {
-      if (tid == 0) atomicExch(err, 1);
+      if (tid == 0) atomicCAS(err, kErrNone, kErrOrder);  // an earlier failure stays the one reported
       return;
     }
 #pragma unroll

@@ -19,6 +19,10 @@ namespace pin {
 
 constexpr int kMaxFields = 9;
 
+// The error word of a plan (and of the allocation-free entry point): what gave
+// up a bounded wait since the host last read it.
+enum { kErrNone = 0, kErrTransfer = 1, kErrOrder = 2 };
+
 // Filter support.  W = exp(-k^2 R^2 / 2) underflows: past about kR = 14 the
 // FP32 axis factors {W, k W, k^2 W} / n are exactly zero, and with them every
 // product and every line they multiply.  At 768^3 with 4 Mpc/h cells and 40
@@ -77,7 +81,7 @@ struct ArgsX {
   int batch;          // realisations stacked back to back (same N, radii)
   RadGroup rad;       // radius g's outputs: dst[f] + g * 3 spectra (of all realisations)
   int col_unit;       // the y pass reads the band's columns in tiles of this many: all of them are stored
-  int* err;           // set to 1 if a TMA wait gave up (bounded wait)
+  int* err;           // set to kErrTransfer if a TMA wait gave up (bounded wait)
   long long wait_cycles;  // budget of a TMA wait in SM clocks; <= 0: the default (2^31)
   CUtensorMap tm_out[3];  // maps of dst[f] (filled at launch when outputs go out by TMA stores)
 };
@@ -272,7 +276,7 @@ cudaError_t generate_ic(int n, double box, const uint64_t* keys_dev, double* tab
 // their six periodic neighbours that precede them into `n_before`; either
 // output may be null.  `scratch` holds fragment_scratch_bytes(N^3) bytes.  A
 // block whose wait for an earlier one runs out (wait_cycles as in ArgsX) sets
-// *err.
+// *err to kErrOrder.
 size_t fragment_scratch_bytes(long n3);
 cudaError_t fragment_order(const float* fmax, int nx, int ny, int nz, void* scratch, int32_t* order,
                            uint8_t* n_before, long long wait_cycles, int* err, cudaStream_t st);

@@ -76,7 +76,7 @@ __device__ __forceinline__ bool stage_ready(uint32_t bar, uint32_t parity, int* 
   const bool ok = mbar_wait_bounded(bar, parity, budget > 0 ? budget : kWaitDefault);
   if (__syncthreads_and(ok)) return true;
   mbar_wait_bounded(bar, parity, kWaitDefault);
-  if (threadIdx.x == 0) atomicExch(err, 1);
+  if (threadIdx.x == 0) atomicExch(err, kErrTransfer);
   return false;
 }
 __device__ __forceinline__ void fence_proxy_async() {

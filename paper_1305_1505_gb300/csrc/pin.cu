@@ -857,7 +857,9 @@ pin_status check_error_word(pin_plan_t p) {
   PIN_CK(p, cudaMemcpy(&err, p->err, sizeof(int), cudaMemcpyDeviceToHost));
   if (err) {
     PIN_CK(p, cudaMemset(p->err, 0, sizeof(int)));
-    return fail(p, PIN_ECUDA, "a transfer wait in the x/y pass timed out; results are invalid");
+    return fail(p, PIN_ECUDA,
+                err == kErrOrder ? "a wait between blocks of the particle order timed out; the order is invalid"
+                                 : "a transfer wait in the x/y pass timed out; results are invalid");
   }
   return PIN_OK;
 }

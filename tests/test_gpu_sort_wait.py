@@ -44,3 +44,29 @@ def test_waits_run_out_and_the_plan_recovers(n):
     assert torch.equal(o, ref)
     assert np.array_equal(F.cpu().numpy().ravel()[o.cpu().numpy()], np.sort(F.cpu().numpy().ravel())[::-1])
     plan.close()
+
+
+def test_the_failure_names_the_call_that_gave_up():
+    import torch
+    from paper_1305_1505_gb300 import pin
+    n = 128
+    plan = pin.Plan(n, 2.0 * n, [8.0, 2.0], stream=torch.cuda.Stream())
+    plan.set_ic(torch.from_numpy(parity.inputs(n, 2.0 * n, 5)[0]).cuda())
+    plan.collapse_times()
+    order = torch.empty(n ** 3, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    pin.pin_set_wait_budget(plan.handle, 1)
+    for _ in range(8):
+        pin.pin_fragment_order(plan.handle, order.data_ptr(), 0, 1)
+        if pin.pin_sync(plan.handle, -1) == pin.PIN_ECUDA:
+            break
+    else:
+        pytest.fail("no wait ran out")
+    msg = pin.pin_last_error(plan.handle)
+    assert "order" in msg and "transfer" not in msg, msg
+    # a failed radius loop before the order: the loop's failure is the one reported
+    plan.collapse_times(sync=False)
+    pin.pin_fragment_order(plan.handle, order.data_ptr(), 0, 1)
+    assert pin.pin_sync(plan.handle, -1) == pin.PIN_ECUDA
+    assert "transfer" in pin.pin_last_error(plan.handle)
+    plan.close()
