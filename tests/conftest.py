@@ -1,3 +1,4 @@
+import gc
 import os
 import sys
 
@@ -17,3 +18,12 @@ def pytest_configure(config):
 def gpu_available():
     import torch
     return torch.cuda.is_available()
+
+
+@pytest.fixture(autouse=True)
+def _collect_before(request):
+    """A plan of an earlier test that sits in a reference cycle (the traceback
+    that pytest.raises keeps) is freed here, not in the middle of a test that
+    compares the device's free memory before and after."""
+    if request.node.get_closest_marker("gpu"):
+        gc.collect()
