@@ -69,10 +69,6 @@ struct pin_plan_s {
   int tc_x = 0, tc_y = 0;                  // tile widths (columns per block) of the x and y passes
   int vx = 0, vy = 0;                      // radix schedules of the x and y line transforms
   bool ic_set = false;
-  // amplitude of the spectrum {ns, gamma, sigma8} that pin_set_ic_seed last
-  // used (amp 0: none), a host integral of 65537 points (5.3 ms)
-  pin_spectrum amp_of{};
-  double amp = 0.0;
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t graph_exec = nullptr;
   // graphs captured for other radius lists (pin_set_radii), keyed by the order
@@ -1112,11 +1108,7 @@ pin_status pin_set_ic_seed(pin_plan_t p, uint64_t seed, const pin_spectrum* ps) 
   if (p->nx != p->ny || p->ny != p->nz) return fail(p, PIN_EINVAL, "pin_set_ic_seed needs a cubic grid");
   if (!(ps->gamma > 0.0) || !std::isfinite(ps->ns) || !(ps->sigma8 > 0.0))
     return fail(p, PIN_EINVAL, "bad spectrum parameters");
-  if (p->amp == 0.0 || p->amp_of.ns != ps->ns || p->amp_of.gamma != ps->gamma || p->amp_of.sigma8 != ps->sigma8) {
-    p->amp = pin_ic_amplitude(ps);
-    p->amp_of = *ps;
-  }
-  const double amp = p->amp;
+  const double amp = pin_ic_amplitude(ps);  // a host integral over 65537 points, of every call
   std::vector<uint64_t> keys(p->batch);
   for (int b = 0; b < p->batch; ++b) keys[b] = pin_ic_splitmix64(seed + (uint64_t)b);
   // stage: the keys and the table of scales after the generated half-spectra
