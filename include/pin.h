@@ -87,7 +87,12 @@ typedef struct {
                             pin_velocities); costs three more spectra per radius.  0: off. */
 } pin_plan_desc;
 
-/* Runtime counters of a plan (cumulative over its pin_collapse_times calls). */
+/* Runtime counters of a plan (cumulative over its pin_collapse_times calls).
+ * A particle that cannot beat its running maximum is not redone.  Where a
+ * launch covers a group of radii (pin_kernels_per_call), how far the maximum
+ * has come when a radius is tested depends on which blocks ran first, so the
+ * first two counters may vary by a few from run to run; F_max and the index do
+ * not. */
 typedef struct {
   uint64_t eig_fp64_redo;   /* particle-scales redone in FP64 for a near-degenerate pair */
   uint64_t root_fp64_redo;  /* particle-scales redone in FP64 for a near-tangent root */
@@ -350,7 +355,7 @@ pin_status pin_collapse_times_noalloc(const void* delta_k, int dtype, int n, dou
  * call returns PIN_ECUDA).  counters3[0] and [1]: particle-scales redone in
  * FP64 for a near-degenerate eigenvalue pair and for a near-tangent root;
  * counters3[2]: of those, kept at FP32 because the redo queue of a radius was
- * full (as in pin_stats).  PIN_ESTATE if no call has run on this device. */
+ * full (as in pin_stats, whose note on groups of radii holds here too).  PIN_ESTATE if no call has run on this device. */
 pin_status pin_noalloc_status(int* wait_failed, uint64_t* counters3);
 
 const char* pin_strerror(pin_status s);

@@ -187,6 +187,19 @@ __device__ __forceinline__ unsigned no_root_from_x2(float2 c1, float2 c2, float2
   return (n0 ? 1u : 0u) | (n1 ? 2u : 0u);
 }
 
+// The same with a margin `lim` > 0 that the cubic has to keep at t and at its
+// right critical point (the inflection where it has none): see cannot_beat_x2.
+__device__ __forceinline__ unsigned no_root_from_x2(float2 c1, float2 c2, float2 c3, float2 t, float2 lim) {
+  using namespace x2;
+  const float2 gt = sub(mul(sub(mul(sub(t, c1), t), c2), t), c3);
+  const float2 d = fma(c1, c1, mul(splat(3.0f), c2));
+  const float2 fs = mul(add(c1, sqrt_approx(d)), splat(1.0f / 3.0f));
+  const float2 gs = sub(mul(sub(mul(sub(fs, c1), fs), c2), fs), c3);
+  const bool n0 = (gt.x > lim.x) & ((fs.x <= t.x) | (gs.x > lim.x));
+  const bool n1 = (gt.y > lim.y) & ((fs.y <= t.y) | (gs.y > lim.y));
+  return (n0 ? 1u : 0u) | (n1 ? 2u : 0u);
+}
+
 // Per-pair state between the common part and the rare minor-axis solve.
 struct CollapseStateX2 {
   float2 best, kappa, corr;
@@ -278,6 +291,23 @@ __device__ __forceinline__ void collapse_main_x2(const float2 lam[3], const Coll
 // that a lane it clears could not have been updated by the full computation
 // (nor by its FP64 redo).  Exact up to rounding, like no_root_from.
 //
+// MARGIN makes that hold at near-tangent roots as well, where g is flat and the
+// rounding of g decides whether a root exists (FP32 calls a double root absent
+// that the FP64 redo finds: seen for one in 6e7 random draws).  The radius
+// groups need it: there fm depends on which blocks ran first, and the result
+// may not.  With L the largest |lambda| and u = 2^-24: |c1| <= L, |c2| <= (3/7)
+// L^2, |c3| < 0.59 L^3; c2 and c3 carry errors of 2.1 u L^2 and 3.6 u L^3, and
+// a cubic evaluated at x is off by at most 5 u (x + L)^3.  The root that the
+// solver accepts comes out of a step below 2e-6 x of a third-order iteration,
+// so its residual is that rounding again and the rounding of x, together 8 u
+// (x + L)^3 (the FP64 redo's is far less).  So where g, as computed, exceeds 13
+// u (x + L)^3 = 8e-7 (x + L)^3, no accepted root can lie.  g is smallest on [t,
+// inf) at t or at fs < 0.84 L, and the limit here is 2e-6 (t + 2 L)^3 at both.
+// The minor axes inherit it, as g_i >= g_0 there (below).  It holds a root back
+// for 9 % of random triples whose fm is 1e-3 above F, for 0.6 % at 1e-2.  Line
+// sizes of radius groups take it in all their kernels, so that grouped and
+// single radii agree.
+//
 // Only the axis of the largest eigenvalue takes that test.  With k the
 // remaining index, the cubics differ by (the identity follows from e_i, c3)
 //   g_i(F) - g_0(F) = (lam_0 - lam_i) q_i(F),
@@ -289,12 +319,25 @@ __device__ __forceinline__ void collapse_main_x2(const float2 lam[3], const Coll
 // them (one in 700) takes the tests of the other axes.  Two of the three tests,
 // their square roots and the coefficients of two axes go: z pass 11.01 -> 10.57
 // ps per particle and radius at 768^3, 12.1 -> 11.3 at 256^3.
+template <bool MARGIN>
 __device__ __forceinline__ unsigned cannot_beat_x2(const float2 lam[3], const CollapseConsts<float>& cc, float2 fm) {
   using namespace x2;
   const AxisZeroX2 a = axis_zero_x2(lam);
   const float2 t = mul(sub(fm, correction_x2(lam, a.mu1, cc)), splat(1.0f - 1e-5f));
-  const unsigned nonneg = (t.x >= 0.0f ? 1u : 0u) | (t.y >= 0.0f ? 2u : 0u);
-  const unsigned a0 = no_root_from_x2(a.c[0], a.c[1], a.c[2], t) & nonneg;
+  float2 lim = splat(0.0f);
+  if constexpr (MARGIN) {
+    const float2 L = make_float2(fmaxf(fabsf(lam[0].x), fabsf(lam[2].x)), fmaxf(fabsf(lam[0].y), fabsf(lam[2].y)));
+    const float2 u = fma(splat(2.0f), L, t);
+    lim = mul(mul(u, u), mul(u, splat(2e-6f)));
+  }
+  auto none_from = [&](const float2 c[3]) {
+    if constexpr (MARGIN) return no_root_from_x2(c[0], c[1], c[2], t, lim);
+    else return no_root_from_x2(c[0], c[1], c[2], t);
+  };
+  // (t = 0 is F = corr = fm, a tie)
+  const unsigned nonneg = ((MARGIN ? t.x > 0.0f : t.x >= 0.0f) ? 1u : 0u) |
+                          ((MARGIN ? t.y > 0.0f : t.y >= 0.0f) ? 2u : 0u);
+  const unsigned a0 = none_from(a.c) & nonneg;
   const float2 m = fma(splat(3.0f / 14.0f), t, mul(splat(5.0f / 84.0f), a.mu1));
   const float2 tt = mul(mul(t, splat(1.0f - 1e-4f)), t);
   const float2 q1 = fma(lam[2], m, tt), q2 = fma(lam[1], m, tt);
@@ -309,7 +352,7 @@ __device__ __forceinline__ unsigned cannot_beat_x2(const float2 lam[3], const Co
   if (a0 & ~minor) {
     float2 c1[3], c2[3];
     minor_axes_x2(lam, a, c1, c2);
-    return a0 & (minor | (no_root_from_x2(c1[0], c1[1], c1[2], t) & no_root_from_x2(c2[0], c2[1], c2[2], t)));
+    return a0 & (minor | (none_from(c1) & none_from(c2)));
   }
   return a0;
 }

@@ -295,7 +295,8 @@ __global__ void __launch_bounds__(NP * LINES * Shape<N>::P, MODE != kZCollapse ?
         // eigenvalues and F_max in the particle's own (already read) field
         // slots 0-3
         const unsigned done =
-            cannot_beat_x2(lam, ccf, make_float2(fm[0], fm[1])) | (valid[0] ? 0u : 1u) | (valid[1] ? 0u : 2u);
+            cannot_beat_x2<kMultiRad<N>>(lam, ccf, make_float2(fm[0], fm[1])) | (valid[0] ? 0u : 1u) |
+            (valid[1] ? 0u : 2u);
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
           if ((done >> u) & 1u) continue;
