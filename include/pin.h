@@ -102,11 +102,14 @@ typedef struct {
 } pin_stats;
 
 /* Creates a plan: validates the description, allocates the device workspace
- * on the current CUDA device, and builds the per-radius filter tables.
+ * on the current CUDA device, and builds the per-radius filter tables.  On a
+ * device too full for the spectra of a group of radii (pin_kernels_per_call)
+ * the plan runs one radius at a time, with the same results.
  * On error *out is NULL and nothing stays allocated. */
 pin_status pin_plan(pin_plan_t* out, const pin_plan_desc* d);
 
-/* Device bytes a plan with this description would allocate (0 if invalid). */
+/* Device bytes a plan with this description would allocate (0 if invalid);
+ * less on a device that has no room for them (pin_plan). */
 size_t pin_footprint_bytes(const pin_plan_desc* d);
 
 /* Loads the linear density field delta(k) (Sec. 2.1.1, Eq. "deltal"), a

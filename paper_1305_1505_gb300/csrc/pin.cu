@@ -379,12 +379,16 @@ bool validate(const pin_plan_desc* d, std::string* why) {
 // g_fail_alloc >= 0, the device allocation of pin_plan with that index
 // (counted from 0 over later pin_plan calls) fails as out of memory.
 std::atomic<int> g_fail_alloc{-1};
+thread_local bool g_injected = false;  // this thread's last failure was an injected one
 
 cudaError_t plan_alloc(void** ptr, size_t bytes) {
   int k = g_fail_alloc.load();
   while (k >= 0) {
     if (g_fail_alloc.compare_exchange_weak(k, k - 1)) {
-      if (k == 0) return cudaErrorMemoryAllocation;
+      if (k == 0) {
+        g_injected = true;
+        return cudaErrorMemoryAllocation;
+      }
       break;
     }
   }
@@ -461,33 +465,39 @@ pin_status ensure_device_init(pin_plan_t p) {
 
 void drop_graph(pin_plan_t p);
 
+template <class T>
+void free_array(T** ptr) {
+  cudaFree(*ptr);
+  *ptr = nullptr;
+}
+
+// The device arrays that pin_plan allocates.
+void free_arrays(pin_plan_t p) {
+  free_array(&p->phi0);
+  free_array(&p->U);
+  free_array(&p->V);
+  free_array(&p->psi);
+  free_array(&p->vstate);
+  free_array(&p->fmax);
+  free_array(&p->idx);
+  free_array(&p->mult);
+  free_array(&p->tw);
+  free_array(&p->counters);
+  free_array(&p->redo_list);
+  free_array(&p->redo_count);
+  free_array(&p->err);
+  free_array(&p->d64);
+  free_array(&p->w64);
+  free_array(&p->h64);
+  free_array(&p->fmax64);
+}
+
 void release(pin_plan_t p) {
   drop_graph(p);
-  cudaFree(p->phi0);
-  cudaFree(p->U);
-  cudaFree(p->V);
-  cudaFree(p->psi);
-  cudaFree(p->vstate);
-  cudaFree(p->fmax);
-  cudaFree(p->idx);
-  cudaFree(p->mult);
-  cudaFree(p->tw);
-  cudaFree(p->counters);
-  cudaFree(p->redo_list);
-  cudaFree(p->redo_count);
-  cudaFree(p->err);
+  free_arrays(p);
   for (cudaEvent_t e : p->events) cudaEventDestroy(e);
   p->events.clear();
-  cudaFree(p->V2);
-  p->V2 = nullptr;
-  cudaFree(p->d64);
-  cudaFree(p->w64);
-  cudaFree(p->h64);
-  cudaFree(p->fmax64);
-  p->d64 = nullptr;
-  p->w64 = nullptr;
-  p->h64 = nullptr;
-  p->fmax64 = nullptr;
+  free_array(&p->V2);
   for (cudaEvent_t e : p->cap_ev) cudaEventDestroy(e);
   p->cap_ev.clear();
   for (cudaEvent_t e : p->redo_ev)
@@ -996,8 +1006,6 @@ pin_status pin_plan(pin_plan_t* out, const pin_plan_desc* d) {
   p->spec_elems = (size_t)p->nx * p->ny * p->nhp;
   p->field_elems = p->spec_elems * p->batch;
   p->dcorr = correction_dcorr();
-  p->group = radius_group(p->nx, p->ny, p->nz, p->batch, p->velocities);
-  p->redo_cap = group_redo_cap(redo_capacity(p->n3(), p->batch), p->n3() * p->batch, p->group);
   auto bail = [&](pin_status s) {
     release(p);
     delete p;
@@ -1023,22 +1031,33 @@ pin_status pin_plan(pin_plan_t* out, const pin_plan_desc* d) {
     // n + 64 entries: a three-level line has P <= 64 threads)
     tw_elems += (size_t)ns[a] + (a < 2 ? 64 : (shapes[a]->P2 > 1 ? shapes[a]->P : 0));
   }
-  auto A = [](auto** ptr, size_t bytes) { return plan_alloc(reinterpret_cast<void**>(ptr), bytes); };
-  if (A(&p->phi0, p->field_elems * 8) != cudaSuccess || A(&p->U, 3 * p->group * p->field_elems * 8) != cudaSuccess ||
-      A(&p->V, v_bytes(p->field_elems, n3, p->group, p->velocities)) != cudaSuccess ||
-      (p->velocities && (A(&p->psi, 3 * n3 * 4) != cudaSuccess || A(&p->vstate, 3 * n3 * 4) != cudaSuccess)) ||
-      A(&p->fmax, n3 * 4) != cudaSuccess || A(&p->idx, n3 * 4) != cudaSuccess ||
-      A(&p->mult, mult_elems * 4 + kBandInts * sizeof(int)) != cudaSuccess || A(&p->tw, tw_elems * 8) != cudaSuccess ||
-      A(&p->counters, 3 * sizeof(unsigned long long)) != cudaSuccess ||
-      A(&p->redo_list, (size_t)p->redo_cap * p->group * sizeof(RedoEntry)) != cudaSuccess ||
-      A(&p->redo_count, kMaxScales * sizeof(unsigned)) != cudaSuccess || A(&p->err, sizeof(int)) != cudaSuccess ||
-      (p->precision == PIN_FP64 &&
-       (A(&p->d64, (size_t)p->nx * p->ny * (p->nz / 2 + 1) * 16) != cudaSuccess ||
-        A(&p->w64, n3 * 16) != cudaSuccess || A(&p->h64, 6 * n3 * 8) != cudaSuccess ||
-        A(&p->fmax64, n3 * 8) != cudaSuccess))) {
-    cudaGetLastError();
-    return bail(PIN_ENOMEM);
-  }
+  auto A = [](auto** ptr, size_t bytes) { return plan_alloc(reinterpret_cast<void**>(ptr), bytes) == cudaSuccess; };
+  auto allocate = [&](int group) {
+    p->group = group;
+    p->redo_cap = group_redo_cap(redo_capacity(p->n3(), p->batch), n3, group);
+    const bool ok =
+        A(&p->phi0, p->field_elems * 8) && A(&p->U, 3 * group * p->field_elems * 8) &&
+        A(&p->V, v_bytes(p->field_elems, n3, group, p->velocities)) &&
+        (!p->velocities || (A(&p->psi, 3 * n3 * 4) && A(&p->vstate, 3 * n3 * 4))) && A(&p->fmax, n3 * 4) &&
+        A(&p->idx, n3 * 4) && A(&p->mult, mult_elems * 4 + kBandInts * sizeof(int)) && A(&p->tw, tw_elems * 8) &&
+        A(&p->counters, 3 * sizeof(unsigned long long)) &&
+        A(&p->redo_list, (size_t)p->redo_cap * group * sizeof(RedoEntry)) &&
+        A(&p->redo_count, kMaxScales * sizeof(unsigned)) && A(&p->err, sizeof(int)) &&
+        (p->precision != PIN_FP64 ||
+         (A(&p->d64, (size_t)p->nx * p->ny * (p->nz / 2 + 1) * 16) && A(&p->w64, n3 * 16) && A(&p->h64, 6 * n3 * 8) &&
+          A(&p->fmax64, n3 * 8)));
+    if (!ok) {
+      cudaGetLastError();
+      free_arrays(p);
+    }
+    return ok;
+  };
+  // A group's spectra are up to sixteen times those of one radius: a device
+  // that is too full for them runs one radius at a time, and leaves what
+  // remains to the caller.
+  const int group = radius_group(p->nx, p->ny, p->nz, p->batch, p->velocities);
+  g_injected = false;
+  if (!allocate(group) && (group == 1 || g_injected || !allocate(1))) return bail(PIN_ENOMEM);
   p->band = reinterpret_cast<int*>(p->mult + mult_elems);
   if (p->group > 1) p->state = reinterpret_cast<unsigned long long*>(p->V + 6 * p->group * p->field_elems);
   std::vector<float> mult = mult_table(p);
