@@ -112,6 +112,14 @@ pin_status pin_plan(pin_plan_t* out, const pin_plan_desc* d);
  * less on a device that has no room for them (pin_plan). */
 size_t pin_footprint_bytes(const pin_plan_desc* d);
 
+/* The same for a caller with a memory budget: a plan whose groups of radii are
+ * made small enough for its workspace to stay within max_bytes, and the bytes
+ * it would allocate.  One radius at a time is the smallest workspace there is
+ * (max_bytes = 0 asks for it); it is taken where it exceeds max_bytes, too.
+ * Results do not depend on max_bytes. */
+pin_status pin_plan_within(pin_plan_t* out, const pin_plan_desc* d, size_t max_bytes);
+size_t pin_footprint_within(const pin_plan_desc* d, size_t max_bytes);
+
 /* Loads the linear density field delta(k) (Sec. 2.1.1, Eq. "deltal"), a
  * half-spectrum as described above (B of them back to back for a batch), dtype PIN_C64 (interleaved float) or
  * PIN_C128 (interleaved double, rounded to FP32 on the device), from host

@@ -395,9 +395,10 @@ cudaError_t plan_alloc(void** ptr, size_t bytes) {
   return cudaMalloc(ptr, bytes);
 }
 
-// FP64 redo queue capacity: 1/64 of the grid (observed rate ~2e-4), at least 64 Ki.
-unsigned redo_capacity(size_t n3, int batch) {
-  return (unsigned)std::max<size_t>(65536, n3 * batch / 64);
+// FP64 redo queue capacity per radius: 1/64 of the grid (observed rate ~2e-4),
+// at least 64 Ki; never more than the particles, each queued once per radius.
+unsigned redo_capacity(size_t npart) {
+  return (unsigned)std::min<size_t>(npart, std::max<size_t>(65536, npart / 64));
 }
 
 // Radii per launch (RadGroup): as many as fit in kGroupBytes of spectra (9
@@ -420,25 +421,28 @@ int radius_group(int nx, int ny, int nz, int batch, bool velocities) {
 size_t v_bytes(size_t field_elems, size_t npart, int group, bool velocities) {
   return field_elems * 8 * (velocities ? 9 : 6) * group + (group > 1 ? npart * 8 : 0);
 }
-// A particle is queued at most once per radius: a group's queues need no more
-// than one entry per particle each.
-unsigned group_redo_cap(unsigned cap, size_t npart, int group) {
-  return group > 1 ? (unsigned)std::min<size_t>(cap, npart) : cap;
-}
 
 int batch_of(const pin_plan_desc* d) { return d->batch <= 0 ? 1 : d->batch; }
 
-size_t footprint(int nx, int ny, int nz, int nscales, int batch, bool velocities, bool fp64) {
-  (void)nscales;
+size_t footprint(int nx, int ny, int nz, int batch, bool velocities, bool fp64, int group) {
   const size_t spec = (size_t)nx * ny * padded_half(nz) * batch;
   const size_t n3 = (size_t)nx * ny * nz * batch;
-  const int group = radius_group(nx, ny, nz, batch, velocities);
-  const size_t cap = group_redo_cap(redo_capacity((size_t)nx * ny * nz, batch), n3, group);
+  const size_t cap = redo_capacity(n3);
   return (fp64 ? fp64_workspace_bytes(nx, ny, nz) : 0) + spec * 8 * (1 + 3 * group) +
          v_bytes(spec, n3, group, velocities) + n3 * 8 + (velocities ? n3 * 24 : 0) +
          (size_t)(kMaxScales + 1) * 3 * (nx + ny + nz) * 4 + kBandInts * sizeof(int) +
          (size_t)(nx + ny + nz + 3 * 64) * 8 + 64 + cap * group * sizeof(RedoEntry) +
          kMaxScales * sizeof(unsigned) + 16 + sizeof(int);
+}
+
+// Radii per launch of a plan that may take max_bytes: the largest group within
+// them, one radius at a time where none is.
+int group_within(const pin_plan_desc* d, size_t max_bytes) {
+  int group = radius_group(d->nx, d->ny, d->nz, batch_of(d), d->velocities != 0);
+  while (group > 1 && footprint(d->nx, d->ny, d->nz, batch_of(d), d->velocities != 0, d->precision == PIN_FP64,
+                                group) > max_bytes)
+    --group;
+  return group;
 }
 
 pin_status ensure_device_init(pin_plan_t p) {
@@ -976,12 +980,19 @@ pin_status time_pass(pin_plan_t p, bool y_pass, int tc, int reps, float* ms) {
 extern "C" {
 
 size_t pin_footprint_bytes(const pin_plan_desc* d) {
-  std::string why;
-  if (!validate(d, &why)) return 0;
-  return footprint(d->nx, d->ny, d->nz, d->nscales, batch_of(d), d->velocities != 0, d->precision == PIN_FP64);
+  return pin_footprint_within(d, SIZE_MAX);
 }
 
-pin_status pin_plan(pin_plan_t* out, const pin_plan_desc* d) {
+size_t pin_footprint_within(const pin_plan_desc* d, size_t max_bytes) {
+  std::string why;
+  if (!validate(d, &why)) return 0;
+  return footprint(d->nx, d->ny, d->nz, batch_of(d), d->velocities != 0, d->precision == PIN_FP64,
+                   group_within(d, max_bytes));
+}
+
+pin_status pin_plan(pin_plan_t* out, const pin_plan_desc* d) { return pin_plan_within(out, d, SIZE_MAX); }
+
+pin_status pin_plan_within(pin_plan_t* out, const pin_plan_desc* d, size_t max_bytes) {
   if (!out) return PIN_EINVAL;
   *out = nullptr;
   std::string why;
@@ -1034,7 +1045,7 @@ pin_status pin_plan(pin_plan_t* out, const pin_plan_desc* d) {
   auto A = [](auto** ptr, size_t bytes) { return plan_alloc(reinterpret_cast<void**>(ptr), bytes) == cudaSuccess; };
   auto allocate = [&](int group) {
     p->group = group;
-    p->redo_cap = group_redo_cap(redo_capacity(p->n3(), p->batch), n3, group);
+    p->redo_cap = redo_capacity(n3);
     const bool ok =
         A(&p->phi0, p->field_elems * 8) && A(&p->U, 3 * group * p->field_elems * 8) &&
         A(&p->V, v_bytes(p->field_elems, n3, group, p->velocities)) &&
@@ -1055,7 +1066,7 @@ pin_status pin_plan(pin_plan_t* out, const pin_plan_desc* d) {
   // A group's spectra are up to sixteen times those of one radius: a device
   // that is too full for them runs one radius at a time, and leaves what
   // remains to the caller.
-  const int group = radius_group(p->nx, p->ny, p->nz, p->batch, p->velocities);
+  const int group = group_within(d, max_bytes);
   g_injected = false;
   if (!allocate(group) && (group == 1 || g_injected || !allocate(1))) return bail(PIN_ENOMEM);
   p->band = reinterpret_cast<int*>(p->mult + mult_elems);

@@ -53,7 +53,7 @@ class pin_stats(ctypes.Structure):
 
 
 # every symbol include/pin.h declares
-EXPORTS = ("pin_plan", "pin_footprint_bytes", "pin_set_ic", "pin_collapse_times", "pin_collapse_times_f64",
+EXPORTS = ("pin_plan", "pin_footprint_bytes", "pin_plan_within", "pin_footprint_within", "pin_set_ic", "pin_collapse_times", "pin_collapse_times_f64",
            "pin_hessian",
            "pin_displacements", "pin_sync", "pin_get_stats", "pin_kernels_per_call",
            "pin_profile", "pin_pass_times", "pin_collapse_times_noalloc", "pin_velocities",
@@ -81,6 +81,9 @@ def load(path=None):
     L.pin_plan.restype = ctypes.c_int
     L.pin_footprint_bytes.argtypes = [ctypes.POINTER(pin_plan_desc)]
     L.pin_footprint_bytes.restype = ctypes.c_size_t
+    L.pin_plan_within.argtypes = [ctypes.POINTER(P), ctypes.POINTER(pin_plan_desc), ctypes.c_size_t]
+    L.pin_footprint_within.argtypes = [ctypes.POINTER(pin_plan_desc), ctypes.c_size_t]
+    L.pin_footprint_within.restype = ctypes.c_size_t
     L.pin_set_ic.argtypes = [P, P, ctypes.c_int, ctypes.c_int]
     L.pin_set_ic.restype = ctypes.c_int
     L.pin_collapse_times.argtypes = [P, P, P, ctypes.c_int]
@@ -202,6 +205,18 @@ def pin_plan(desc):
 
 def pin_footprint_bytes(desc):
     return load().pin_footprint_bytes(ctypes.byref(desc))
+
+
+def pin_plan_within(desc, max_bytes):
+    """pin_plan with groups of radii small enough for max_bytes of workspace
+    (at least one radius at a time)."""
+    h = ctypes.c_void_p()
+    _check(load().pin_plan_within(ctypes.byref(h), ctypes.byref(desc), int(max_bytes)))
+    return h
+
+
+def pin_footprint_within(desc, max_bytes):
+    return load().pin_footprint_within(ctypes.byref(desc), int(max_bytes))
 
 
 def pin_set_ic(plan, delta_k_ptr, dtype, on_device):
@@ -397,9 +412,9 @@ class Plan:
     """Owns one pin plan; methods take torch tensors (device or host)."""
 
     def __init__(self, n, box, radii, correction=PIN_CORR_SPHERE, stream=None, batch=1,
-                 velocities=False, precision=PIN_FP32_FALLBACK64):
+                 velocities=False, precision=PIN_FP32_FALLBACK64, max_bytes=None):
         """n: grid side, or (nx, ny, nz) for a non-cubic grid with cubic cells
-        (box is the side along x)."""
+        (box is the side along x).  max_bytes: see pin_plan_within."""
         import torch
         if not torch.cuda.is_available():
             raise RuntimeError("pin needs a CUDA device; none is available")
@@ -411,7 +426,7 @@ class Plan:
         s = stream.cuda_stream if stream is not None else None
         self._desc = make_desc(self.shape, self.box, self.radii, correction, s, self.batch, velocities,
                                precision)
-        self.handle = pin_plan(self._desc)
+        self.handle = pin_plan(self._desc) if max_bytes is None else pin_plan_within(self._desc, max_bytes)
 
     def __del__(self):
         h = getattr(self, "handle", None)

@@ -3,7 +3,7 @@ admission by device-memory footprint.
 
 A request asks for the collapse times of one realisation (grid N, box L,
 seed, radii).  The server keeps a FIFO queue; a request is admitted as soon
-as a slot is free and its workspace (pin_footprint_bytes) fits in what is
+as a slot is free and its workspace (pin_footprint_within) fits in what is
 left of the memory budget, so requests that arrive while others are running
 start on their own streams and their work overlaps on the device.  The
 engine runs each request on a pooled plan of its grid size (no device
@@ -35,7 +35,7 @@ from . import pin
 
 class Request:
     __slots__ = ("rid", "n", "box", "seed", "radii", "arrival", "deadline", "t_admit", "t_done",
-                 "status", "result", "error", "footprint", "_event")
+                 "status", "result", "error", "footprint", "plan_bytes", "_event")
 
     def __init__(self, rid, n, box, seed, radii, deadline_s=None):
         self.rid = rid
@@ -51,6 +51,7 @@ class Request:
         self.result = None
         self.error = None
         self.footprint = 0
+        self.plan_bytes = None  # pin_plan_within's max_bytes for its plan; None: no limit
         self._event = threading.Event()
 
     def wait(self, timeout=None):
@@ -100,14 +101,26 @@ class PinEngine:
         self.lock = threading.Lock()
         self.plans_made = 0
 
-    def _make(self, n, box):
+    # radii of a pooled plan until a request brings its own (the workspace is
+    # the same for any radii)
+    RADII = (8.0, 4.0)
+
+    @staticmethod
+    def _footprint(n, box, radii, plan_bytes):
+        desc = pin.make_desc(n, box, radii)
+        return pin.pin_footprint_bytes(desc) if plan_bytes is None else pin.pin_footprint_within(desc, plan_bytes)
+
+    def _key(self, n, box, plan_bytes):
+        return (int(n), float(box), self._footprint(n, box, self.RADII, plan_bytes))
+
+    def _make(self, n, box, plan_bytes=None):
         torch = self.torch
         torch.cuda.set_device(self.device)
         high = self.priority_from_n > 0 and n >= self.priority_from_n
         s = _Slot()
-        s.key = (int(n), float(box))
+        s.key = self._key(n, box, plan_bytes)
         s.stream = torch.cuda.Stream(priority=-1 if high else 0)
-        s.plan = pin.Plan(n, box, [8.0, 4.0], stream=s.stream)
+        s.plan = pin.Plan(n, box, self.RADII, stream=s.stream, max_bytes=plan_bytes)
         s.plan.autotune()  # the kept choice for this shape (timed once per process)
         s.F = torch.empty((n, n, n), dtype=torch.float32, device="cuda")
         s.I = torch.empty((n, n, n), dtype=torch.int32, device="cuda")
@@ -130,12 +143,13 @@ class PinEngine:
                 self._release(s)
         return out
 
-    def _acquire(self, n, box):
+    def _acquire(self, n, box, plan_bytes=None):
+        key = self._key(n, box, plan_bytes)
         with self.lock:
-            idle = self.pool[(int(n), float(box))]
+            idle = self.pool[key]
             if idle:
                 return idle.pop()
-        return self._make(n, box)
+        return self._make(n, box, plan_bytes)
 
     def _release(self, slot):
         with self.lock:
@@ -153,14 +167,14 @@ class PinEngine:
             s.plan.close()
 
     def footprint(self, req):
-        return pin.pin_footprint_bytes(pin.make_desc(req.n, req.box, req.radii))
+        return self._footprint(req.n, req.box, req.radii, req.plan_bytes)
 
     def run(self, req, timeout_s=None):
         """Returns (F_max, scale_idx, release): numpy views of the plan's host
         buffers and the callable that hands the plan back to the pool."""
         torch = self.torch
         torch.cuda.set_device(self.device)
-        slot = self._acquire(req.n, req.box)
+        slot = self._acquire(req.n, req.box, req.plan_bytes)
         ok = False
         try:
             plan = slot.plan
@@ -187,7 +201,12 @@ class Server:
     per admitted request.  Large requests (N >= big_n) are admitted at most
     max_big at a time: two of them sharing the device would both take about
     twice as long, which sets the latency tail, while small requests cost the
-    device little and overlap freely (and do not wait behind a large one)."""
+    device little and overlap freely (and do not wait behind a large one).
+
+    Plans of small grids take many times the memory when a launch covers a
+    group of radii.  Their groups are kept within a quarter of the budget in
+    all (budget / (4 max_slots) each), so a budget that admits a request, or a
+    number of them at once, with one radius at a time still does."""
 
     def __init__(self, engine, budget_bytes, max_slots=4, keep_results=True, big_n=512, max_big=1):
         """keep_results: copy each result into arrays of the request (False:
@@ -201,6 +220,7 @@ class Server:
         self.running_big = 0
         self.budget = int(budget_bytes)
         self.max_slots = int(max_slots)
+        self.plan_bytes = self.budget // (4 * max(1, self.max_slots))
         self.queue = collections.deque()
         self.lock = threading.Condition()
         self.in_use = 0
@@ -217,6 +237,7 @@ class Server:
 
     def submit(self, req, now=None):
         req.arrival = time.perf_counter() if now is None else now
+        req.plan_bytes = self.plan_bytes
         req.footprint = self.engine.footprint(req)
         with self.lock:
             if req.footprint > self.budget:
