@@ -109,7 +109,11 @@ typedef struct {
 pin_status pin_plan(pin_plan_t* out, const pin_plan_desc* d);
 
 /* Device bytes a plan with this description would allocate (0 if invalid);
- * less on a device that has no room for them (pin_plan). */
+ * less on a device that has no room for them (pin_plan).  For PIN_FP64 it is a
+ * bound: 16 bytes per half-spectrum mode and 72 per particle more than the
+ * FP32 plan, of which such a plan leaves a complex cube (16 bytes per particle)
+ * and the groups of radii unused and unallocated; pin_footprint_within has
+ * what it does allocate. */
 size_t pin_footprint_bytes(const pin_plan_desc* d);
 
 /* The same for a caller with a memory budget: a plan whose groups of radii are

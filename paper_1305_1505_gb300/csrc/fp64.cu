@@ -321,7 +321,7 @@ unsigned grid_for(size_t count) { return (unsigned)std::min<size_t>((count + 255
 
 size_t fp64_workspace_bytes(int nx, int ny, int nz) {
   const size_t n3 = (size_t)nx * ny * nz, half = (size_t)nx * ny * (nz / 2 + 1);
-  return half * 16 + n3 * 16 + 6 * n3 * 8 + n3 * 8;
+  return half * 16 + (size_t)(nx + ny + nz) * 16 + 6 * n3 * 8 + n3 * 8;
 }
 
 cudaError_t fp64_load(const void* src, int dtype, int nx, int ny, int nz, double2* d64, cudaStream_t st) {
@@ -331,12 +331,11 @@ cudaError_t fp64_load(const void* src, int dtype, int nx, int ny, int nz, double
 }
 
 cudaError_t fp64_collapse(const double2* d64, int nx, int ny, int nz, double box, int nscales, const double* radii,
-                          int correction, double dcorr, double2* work, double* h6, double* fmax, int* idx,
+                          int correction, double dcorr, double2* tw, double* h6, double* fmax, int* idx,
                           cudaStream_t st) {
   const size_t n3 = (size_t)nx * ny * nz;
   const double norm = 1.0 / (double)n3;
   double2* cubes = reinterpret_cast<double2*>(h6);
-  double2* tw = work;  // nx + ny + nz values; the work cube holds at least 512
   const double2 *twx = tw, *twy = tw + nx, *twz = tw + nx + ny;
   // 128-byte rows of columns where the lines leave the shared memory for it
   const int ty = ny <= 384 ? 8 : 4, tx = nx <= 192 ? 8 : 4, nl = std::max(1, 128 / nz);

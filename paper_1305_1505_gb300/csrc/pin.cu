@@ -88,10 +88,10 @@ struct pin_plan_s {
   cudaEvent_t redo_ev[2] = {nullptr, nullptr};
   cudaStream_t s_xy = nullptr, s_z = nullptr;  // high / low priority streams of the overlapped schedule
   float2* V2 = nullptr;                        // second V buffer (schedule 2)
-  // PIN_FP64 plans: FP64 half-spectrum, one full complex cube, the tensor,
-  // F_max in FP64 (fp64.cu)
+  // PIN_FP64 plans: FP64 half-spectrum, twiddles, the tensor (as three complex
+  // cubes), F_max in FP64 (fp64.cu)
   double2* d64 = nullptr;
-  double2* w64 = nullptr;
+  double2* tw64 = nullptr;
   double* h64 = nullptr;
   double* fmax64 = nullptr;
   std::vector<cudaEvent_t> cap_ev;             // fork/join events of the overlapped capture
@@ -436,8 +436,10 @@ size_t footprint(int nx, int ny, int nz, int batch, bool velocities, bool fp64, 
 }
 
 // Radii per launch of a plan that may take max_bytes: the largest group within
-// them, one radius at a time where none is.
+// them, one radius at a time where none is.  The FP64 loop has no groups, and
+// the FP32 products of its plans take one radius.
 int group_within(const pin_plan_desc* d, size_t max_bytes) {
+  if (d->precision == PIN_FP64) return 1;
   int group = radius_group(d->nx, d->ny, d->nz, batch_of(d), d->velocities != 0);
   while (group > 1 && footprint(d->nx, d->ny, d->nz, batch_of(d), d->velocities != 0, d->precision == PIN_FP64,
                                 group) > max_bytes)
@@ -491,7 +493,7 @@ void free_arrays(pin_plan_t p) {
   free_array(&p->redo_count);
   free_array(&p->err);
   free_array(&p->d64);
-  free_array(&p->w64);
+  free_array(&p->tw64);
   free_array(&p->h64);
   free_array(&p->fmax64);
 }
@@ -980,7 +982,14 @@ pin_status time_pass(pin_plan_t p, bool y_pass, int tc, int reps, float* ms) {
 extern "C" {
 
 size_t pin_footprint_bytes(const pin_plan_desc* d) {
-  return pin_footprint_within(d, SIZE_MAX);
+  std::string why;
+  if (!validate(d, &why)) return 0;
+  if (d->precision != PIN_FP64) return pin_footprint_within(d, SIZE_MAX);
+  // the bound that pin.h states
+  pin_plan_desc f32 = *d;
+  f32.precision = PIN_FP32_FALLBACK64;
+  return pin_footprint_within(&f32, SIZE_MAX) +
+         (size_t)d->nx * d->ny * ((size_t)(d->nz / 2 + 1) * 16 + (size_t)d->nz * (16 + 48 + 8));
 }
 
 size_t pin_footprint_within(const pin_plan_desc* d, size_t max_bytes) {
@@ -1055,7 +1064,7 @@ pin_status pin_plan_within(pin_plan_t* out, const pin_plan_desc* d, size_t max_b
         A(&p->redo_list, (size_t)p->redo_cap * group * sizeof(RedoEntry)) &&
         A(&p->redo_count, kMaxScales * sizeof(unsigned)) && A(&p->err, sizeof(int)) &&
         (p->precision != PIN_FP64 ||
-         (A(&p->d64, (size_t)p->nx * p->ny * (p->nz / 2 + 1) * 16) && A(&p->w64, n3 * 16) && A(&p->h64, 6 * n3 * 8) &&
+         (A(&p->d64, (size_t)p->nx * p->ny * (p->nz / 2 + 1) * 16) && A(&p->tw64, (size_t)(p->nx + p->ny + p->nz) * 16) && A(&p->h64, 6 * n3 * 8) &&
           A(&p->fmax64, n3 * 8)));
     if (!ok) {
       cudaGetLastError();
@@ -1163,7 +1172,7 @@ pin_status pin_set_ic_seed(pin_plan_t p, uint64_t seed, const pin_spectrum* ps) 
 pin_status run_fp64(pin_plan_t p) {
   const size_t n3 = p->n3();
   PIN_CK(p, fp64_collapse(p->d64, p->nx, p->ny, p->nz, p->box, p->nscales, p->radii.data(), p->correction, p->dcorr,
-                          p->w64, p->h64, p->fmax64, p->idx, p->stream));
+                          p->tw64, p->h64, p->fmax64, p->idx, p->stream));
   PIN_CK(p, fp64_cast(p->fmax64, n3, p->fmax, p->stream));
   return PIN_OK;
 }

@@ -42,3 +42,22 @@ def test_a_full_device_takes_one_radius_at_a_time(n, left_mb):
     assert got[4] == 4 * len(radii)
     assert all(torch.equal(a, b) for a, b in zip(got[:4], ref[:4]))
     assert (ref[1] >= 0).float().mean() > 0.05 and np.isfinite(ref[0].cpu().numpy()).all()
+
+
+@pytest.mark.parametrize("n", [64, 128])
+def test_fp64_plans_hold_only_what_their_loop_uses(n):
+    import torch
+    from paper_1305_1505_gb300 import pin
+    pin.Plan(n, 2.0 * n, [4.0, 2.0], precision=pin.PIN_FP64).close()  # loads the kernels
+    desc = pin.make_desc(n, 2.0 * n, [4.0, 2.0], precision=pin.PIN_FP64)
+    need = pin.pin_footprint_within(desc, 0)
+    single = pin.pin_footprint_within(pin.make_desc(n, 2.0 * n, [4.0, 2.0]), 0)
+    # half-spectrum, twiddles, tensor, F_max
+    assert need == single + 16 * (n * n * (n // 2 + 1) + 3 * n) + 56 * n ** 3
+    assert need == pin.pin_footprint_within(desc, 1 << 62) < pin.pin_footprint_bytes(desc)
+    torch.cuda.synchronize()
+    free0, _ = torch.cuda.mem_get_info()
+    plan = pin.Plan(n, 2.0 * n, [4.0, 2.0], precision=pin.PIN_FP64)
+    free1, _ = torch.cuda.mem_get_info()
+    plan.close()
+    assert free0 - free1 <= need + 15 * (2 << 20)  # fifteen arrays, each at most 2 MB over
