@@ -45,31 +45,35 @@ static_assert((size_t)kMaxN * kMaxN * kMaxN / 64 <= kRedoCap, "redo capacity bel
 constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 constexpr size_t spec_bytes(int n) { return (size_t)n * n * ((n / 2 + 1 + 3) & ~3) * sizeof(float2); }
 
-// Where things lie in the workspace for grids of n points a side and groups of
-// `group` radii (RadGroup): Phi0, U and V; the tables {twiddles, bands,
-// multipliers}, copied in as one piece; {counters, queue counts, error word,
-// the word that turns the bands off, the running maximum of a group}, cleared
-// as one; the redo queues.
+// The head of the workspace: {counters, queue counts, error word, the word that
+// turns the bands off}, cleared as one by every call.  It lies at the same
+// place for every grid, so that pin_noalloc_status reads what the last call to
+// have run left there, whichever call was made or captured since.
+constexpr size_t kOffCnt = 0;
+constexpr size_t kOffRedoCount = kOffCnt + 4 * sizeof(unsigned long long);
+constexpr size_t kOffErr = kOffRedoCount + kMaxScales * sizeof(unsigned);
+constexpr size_t kOffWide = kOffErr + 8;
+constexpr size_t kHeadBytes = align256(kOffWide + 8);
+
+// Where the rest lies for grids of n points a side and groups of `group` radii
+// (RadGroup): the running maximum of a group, cleared with the head; Phi0, U
+// and V; the tables {twiddles, bands, multipliers}, copied in as one piece; the
+// redo queues.
 struct Layout {
   int group;
   size_t cap;  // redo entries per radius
-  size_t phi0, U, V, tw, band, mult, cnt, redo_count, err, wide, state, redo, end;
-  constexpr Layout(int n, int g)
-      : group(g), cap(), phi0(), U(), V(), tw(), band(), mult(), cnt(), redo_count(), err(), wide(), state(), redo(),
-        end() {
+  size_t state, phi0, U, V, tw, band, mult, redo, end;
+  constexpr Layout(int n, int g) : group(g), cap(), state(), phi0(), U(), V(), tw(), band(), mult(), redo(), end() {
     const size_t n3 = (size_t)n * n * n;
     cap = g > 1 && n3 < kRedoCap ? n3 : kRedoCap;
-    U = spec_bytes(n);
+    state = kHeadBytes;
+    phi0 = align256(state + (g > 1 ? n3 * 8 : 0));
+    U = phi0 + spec_bytes(n);
     V = U + 3 * spec_bytes(n) * g;
     tw = V + 6 * spec_bytes(n) * g;
     band = tw + (size_t)n * sizeof(float2);
     mult = band + (size_t)kMaxScales * 4 * sizeof(int);
-    cnt = mult + (size_t)kMaxScales * 3 * n * sizeof(float);
-    redo_count = cnt + 4 * sizeof(unsigned long long);
-    err = redo_count + kMaxScales * sizeof(unsigned);
-    wide = err + 8;
-    state = wide + 8;
-    redo = align256(state + (g > 1 ? n3 * 8 : 0));
+    redo = align256(mult + (size_t)kMaxScales * 3 * n * sizeof(float));
     end = align256(redo + cap * g * sizeof(pin::RedoEntry));
   }
 };
@@ -90,8 +94,6 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 constexpr int kMaxDevices = 64;
 std::mutex g_setup_mu;
 unsigned char* g_scratch_ptr[kMaxDevices] = {};
-size_t g_last_cnt[kMaxDevices] = {};  // counters and error word of the last call
-size_t g_last_err[kMaxDevices] = {};
 
 // Host staging of the tables (filled and copied under g_stage_mu; a copy from
 // pageable host memory has consumed its source when cudaMemcpyAsync returns).
@@ -148,22 +150,17 @@ extern "C" pin_status pin_collapse_times_noalloc(const void* delta_k, int dtype,
   const int nhp = pin::padded_half(n);
   const size_t spec = (size_t)n * n * nhp;
   const Layout at(n, group_of(n));
-  {
-    std::lock_guard<std::mutex> lk(g_setup_mu);
-    g_last_cnt[dev] = at.cnt;
-    g_last_err[dev] = at.err;
-  }
   float2* phi0 = reinterpret_cast<float2*>(base + at.phi0);
   float2* U = reinterpret_cast<float2*>(base + at.U);
   float2* V = reinterpret_cast<float2*>(base + at.V);
   unsigned long long* state = at.group > 1 ? reinterpret_cast<unsigned long long*>(base + at.state) : nullptr;
   float* mult = reinterpret_cast<float*>(base + at.mult);
   float2* tw = reinterpret_cast<float2*>(base + at.tw);
-  unsigned long long* cnt = reinterpret_cast<unsigned long long*>(base + at.cnt);
-  unsigned* redo_count = reinterpret_cast<unsigned*>(base + at.redo_count);
-  int* err = reinterpret_cast<int*>(base + at.err);
+  unsigned long long* cnt = reinterpret_cast<unsigned long long*>(base + kOffCnt);
+  unsigned* redo_count = reinterpret_cast<unsigned*>(base + kOffRedoCount);
+  int* err = reinterpret_cast<int*>(base + kOffErr);
   int* band = reinterpret_cast<int*>(base + at.band);
-  int* wide = reinterpret_cast<int*>(base + at.wide);
+  int* wide = reinterpret_cast<int*>(base + kOffWide);
   pin::RedoEntry* redo_list = reinterpret_cast<pin::RedoEntry*>(base + at.redo);
   CUtensorMap tm_x[2], tm_y[2];  // staged and whole-line boxes
   const int tc = sh.tc;  // the default tile width, as a new plan runs
@@ -189,7 +186,7 @@ extern "C" pin_status pin_collapse_times_noalloc(const void* delta_k, int dtype,
                         cs) != cudaSuccess)
       return PIN_ECUDA;
   }
-  if (cudaMemsetAsync(cnt, 0, at.state - at.cnt + (state ? n3 * sizeof(*state) : 0), cs) != cudaSuccess ||
+  if (cudaMemsetAsync(cnt, 0, kHeadBytes + (state ? n3 * sizeof(*state) : 0), cs) != cudaSuccess ||
       pin::launch_load_phi0(delta_k, dtype, n, n, n, nhp, box, 1, phi0, wide, cs) != cudaSuccess ||
       (!state && (cudaMemsetAsync(F_max, 0, n3 * sizeof(float), cs) != cudaSuccess ||
                   cudaMemsetAsync(scale_idx, 0xFF, n3 * sizeof(int32_t), cs) != cudaSuccess)))
@@ -288,18 +285,15 @@ extern "C" pin_status pin_noalloc_status(int* wait_failed, uint64_t* counters3) 
   const int dev = current_device();
   if (dev < 0) return PIN_ECUDA;
   unsigned char* base = nullptr;
-  size_t off_cnt = 0, off_err = 0;
   {
     std::lock_guard<std::mutex> lk(g_setup_mu);
     base = g_scratch_ptr[dev];
-    off_cnt = g_last_cnt[dev];
-    off_err = g_last_err[dev];
   }
-  if (!base || !off_cnt) return PIN_ESTATE;  // no call has run on this device
+  if (!base) return PIN_ESTATE;  // no call has run on this device
   unsigned long long c[3] = {0, 0, 0};
   int e = 0;
-  if (cudaMemcpy(c, base + off_cnt, sizeof(c), cudaMemcpyDeviceToHost) != cudaSuccess ||
-      cudaMemcpy(&e, base + off_err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
+  if (cudaMemcpy(c, base + kOffCnt, sizeof(c), cudaMemcpyDeviceToHost) != cudaSuccess ||
+      cudaMemcpy(&e, base + kOffErr, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
     return PIN_ECUDA;
   *wait_failed = e != 0;
   for (int i = 0; i < 3; ++i) counters3[i] = c[i];
