@@ -646,12 +646,20 @@ def run_ensemble(args):
     return 0
 
 
-# bytes each particle costs the fragmentation front end: the key range and the
-# digit counts (F read 4 B each), three radix passes, which 27 bits of key
-# range take (pass 0 reads F 4 B and writes key + index 8 B, pass 1 reads and
-# writes 8 B, pass 2 reads 8 B and writes the index 4 B; a wider range takes a
-# fourth) and the neighbour count (F read 4 B, count write 1 B)
-FRAGMENT_BYTES = 2 * 4 + (4 + 8) + (8 + 8) + (8 + 4) + (4 + 1)
+def fragment_passes(fmin, fmax):
+    """Radix passes of the particle order for F_max between its smallest
+    non-zero and its largest value (both 0: nothing collapses): digits of at
+    most nine bits over a key range of the steps between their FP32 bits."""
+    lo, hi = (int(np.float32(f).view(np.uint32)) for f in (fmin, fmax))
+    return -(-(hi - lo + 1).bit_length() // 9)
+
+
+def fragment_bytes(passes):
+    """Bytes each particle costs the fragmentation front end: the key range and
+    the digit counts (F read 4 B each), the radix passes (the first reads F
+    4 B, the others key + index 8 B; the last writes the index 4 B, the others
+    8 B) and the neighbour count (F read 4 B, count write 1 B)."""
+    return 2 * 4 + 4 + 16 * (passes - 1) + 4 + (4 + 1)
 
 
 def run_fragment(args):
@@ -712,7 +720,9 @@ def run_fragment(args):
         cb = {"value": m ** 3 / tc, "unit": "particles/s", "cores": 1, "kind": "oracle",
               "sample": "%d^3 block of the same F_max field (numpy lexsort + rolls), %.1f s" % (m, tc)}
     peak, peak_kind = _peaks()
-    achieved = FRAGMENT_BYTES * n ** 3 / t / 1e9
+    live = F[F > 0]
+    passes = fragment_passes(live.min().item(), live.max().item()) if live.numel() else fragment_passes(0.0, 0.0)
+    achieved = fragment_bytes(passes) * n ** 3 / t / 1e9
     line = {"metric": "fragmentation order (particles/s) at %d^3" % n, "value": n ** 3 / t,
             "unit": "particles/s", "n_gpus": 1, "steps": args.steps, "warmup": args.warmup,
             "ms_per_step": t * 1e3, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
@@ -720,10 +730,10 @@ def run_fragment(args):
             "config": {"workload": "F_max of the %d^3 x %d collapse workload, seed %d" % (n, w["nscales"], w["seed"]),
                        "l2": "inputs larger than L2 (F_max %.1f GB, sort buffers %.1f GB)"
                              % (4 * n ** 3 / 1e9, 16 * n ** 3 / 1e9)},
-            "roofline": {"bound": "hbm", "kernel": "fragment_order (4 radix passes + neighbour count)",
+            "roofline": {"bound": "hbm", "kernel": "fragment_order (%d radix passes + neighbour count)" % passes,
                          "achieved": achieved, "peak": peak, "peak_kind": peak_kind, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": None,
-                         "alg_bytes_per_particle": FRAGMENT_BYTES},
+                         "alg_bytes_per_particle": fragment_bytes(passes)},
             "cpu_baseline": cb, "e2e": e2e,
             "gpu_launches": int(args.steps * 10), "clocks": clk.summary()}
     print(json.dumps(line), flush=True)
