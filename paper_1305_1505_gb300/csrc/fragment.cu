@@ -216,12 +216,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_sort_pass(const float* __restri
   unsigned* out = last ? order : vals_b;
   // Nothing to do after a failed wait, whose outputs are incomplete.  Another
   // block may set the word while this one starts, so one thread reads it and
-  // the block leaves by the tile that it broadcasts, all threads or none: a
-  // block that lost some of its warps here would rank with counts that were
-  // never cleared and write out of range.
-  const bool failed = tid == 0 && *(volatile int*)err != 0;
+  // the block leaves as a whole: one that lost some of its warps here would
+  // rank with counts that were never cleared and write out of range.
+  if (__syncthreads_or(tid == 0 && *(volatile int*)err != 0)) return;
   for (;;) {
-    if (tid == 0) s_tile = failed ? ntiles : atomicAdd(&s->ticket[pass], 1u);
+    if (tid == 0) s_tile = atomicAdd(&s->ticket[pass], 1u);
     for (int j = lane; j < kBins; j += 32) s_cnt[w][j] = 0;
     __syncthreads();
     const unsigned tile = s_tile;
