@@ -140,7 +140,7 @@ TRAFFIC_SOURCES = ["kernels.cu", "kernels_v1.cu", "passes_xy.cuh", "kernels.cuh"
                    "collapse.cuh", "collapse_x2.cuh", "pin.cu"]
 MEASURED_TRAFFIC = {
     # profiles/passes_384x40.md
-    ("k_pass_z", 768, False): {"sources": "86a84589cb5aefc6", "bytes_per_particle": 30.241, "warp_inst_per_particle": 8.9705,
+    ("k_pass_z", 768, False): {"sources": "b321156e7d69d90a", "bytes_per_particle": 30.241, "warp_inst_per_particle": 8.9705,
                                "measured_at": "384^3 x 40, the 40 launches of one step, scaled by particles"},
 }
 

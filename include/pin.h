@@ -231,11 +231,13 @@ int pin_kernels_per_call(pin_plan_t p);
  * record CUDA events around each pass of each radius (on the plan's stream,
  * inside its graph); pin_pass_times() then waits for the plan's work and
  * returns, for the last completed call, the device time in milliseconds summed
- * over radii (or groups of radii) of: ms4[0] the x pass (filter + transform), ms4[1] the y pass,
- * ms4[2] the z pass (c2r, eigenvalues, collapse time and running max), ms4[3]
- * the FP64 redo of the queued ill-conditioned particles.  Each is measured on the stream its pass runs on; under an
- * overlapped schedule (pin_set_schedule) the passes overlap, so the four sums
- * exceed the call's time. */
+ * over radii (or groups of radii) of: ms4[0] the x pass (filter + transform),
+ * ms4[1] the y pass, ms4[2] the z pass (c2r, eigenvalues, collapse time and
+ * running max), ms4[3] the FP64 redo of the queued ill-conditioned particles.
+ * Each is measured on the stream its pass runs on.  The redo of a radius runs
+ * beside the x and y passes of the next one in every schedule, and under an
+ * overlapped schedule (pin_set_schedule) the other passes overlap as well, so
+ * the four sums exceed the call's time. */
 pin_status pin_profile(pin_plan_t p, int enable);
 pin_status pin_pass_times(pin_plan_t p, double* ms4);
 
@@ -347,7 +349,8 @@ void pin_debug_fail_alloc(int nth);
  * (NULL: the legacy default stream) and the call returns without waiting for
  * the kernels; the per-radius tables are copied in from a static host staging
  * area on that stream, a copy from pageable memory that may wait for the
- * stream's earlier work.
+ * stream's earlier work.  A captured call reads that area again whenever its
+ * graph runs, so the graph may only run while no later call has been made.
  *
  * The workspace is one static device array of 13.9 MB, sized for
  * n <= PIN_NOALLOC_MAX_N, which every GPU that loads this library holds until

@@ -9,8 +9,9 @@
 // F_max falls (F_max >= 0 and never NaN, so its bits order as F does), carrying
 // the particle index.  It is bound by memory traffic and by the shared-memory
 // reordering, both per pass, so it takes as few passes as the keys need: the
-// keys run from 0 (the largest F_max) to umax - umin + 1 (F_max = 0), some 26
-// to 27 bits on collapse times, three digits of 9 bits in place of four of 8.
+// keys run from 0 (the largest F_max) to umax - umin + 1 (F_max = 0), 26 to 27
+// bits on the collapse times of a few radii, three digits of 9 bits; a wider
+// range takes a fourth pass (the 40 radii of the benchmark: 28 bits, four of 7).
 // One kernel finds the range, one counts every digit of every pass, and each
 // pass is a single kernel: a tile's digits are ranked and reordered by digit in
 // shared memory, its place among the earlier tiles comes from a look-back over
@@ -18,8 +19,10 @@
 // of equal digits go out to consecutive addresses.  Pass 0 reads F_max and
 // makes the index on the fly; the last pass writes only the indices.
 //
-// 768^3: 11.25 ms for order and counts (15.9 with a histogram pass, a scan of
-// the histogram table and a scatter for each of four digits).
+// 768^3, order and counts: 12.2 ms a call in a run of calls, 11.3 for a single
+// one, with three passes (4 radii), 14.1 with four (40 radii); 15.8 with a
+// histogram pass, a scan of the histogram table and a scatter for each of four
+// digits.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -31,7 +31,7 @@ enum { kErrNone = 0, kErrTransfer = 1, kErrOrder = 2 };
 // radius, the largest |wavenumber index| with a non-zero factor of each axis,
 // {x, y, z, 0}; the x and y passes neither load nor transform what lies
 // outside (per radius of such a run the x pass takes 0.95 instead of 1.62 ms,
-// the y pass 2.35 instead of 3.35).  The z pass reads whole lines: a test per
+// the y pass, beside the redo, 2.51 instead of 3.35).  The z pass reads whole lines: a test per
 // mode costs its issue slots more (3 %) than the loads it saves.  So the
 // columns past a radius's z band have to hold zeros in V; the y pass writes
 // them where the radius before it in the same buffer (RadGroup::prev) had

@@ -280,7 +280,7 @@ def pin_profile(plan, enable):
 
 
 def pin_pass_times(plan):
-    """[x, y, z, roots] device milliseconds of the last call, summed over radii."""
+    """[x, y, z, redo] device milliseconds of the last call, summed over radii."""
     ms = (ctypes.c_double * 4)()
     _check(load().pin_pass_times(plan, ms), plan)
     return list(ms)
@@ -384,8 +384,9 @@ def pin_get_schedule(plan):
 
 
 def pin_set_wait_budget(plan, cycles):
-    """Budget (SM clocks) of the x/y passes' bounded transfer waits; 0 restores
-    the default (2^31 clocks)."""
+    """Budget (SM clocks) of the x/y passes' bounded transfer waits and of the
+    waits between blocks of the particle order; 0 restores the default (2^31
+    clocks)."""
     _check(load().pin_set_wait_budget(plan, int(cycles)), plan)
 
 
